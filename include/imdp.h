@@ -266,8 +266,9 @@ IMDP_API imdp_status imdp_session_create(imdp_model* const* models, const imdp_s
 /* Reset every problem to V_0 and iteration 0 (asynchronous on `stream`). */
 IMDP_API imdp_status imdp_session_reset(imdp_session* s, void* stream);
 
-/* Launch `n_iters` Bellman iterations (one kernel each; problems that are done
- * or past their horizon are skipped on the device). Asynchronous on `stream`;
+/* Launch `n_iters` Bellman iterations (one kernel each, or all in one where the
+ * launch rule says so; problems that are done or past their horizon are skipped
+ * on the device). Asynchronous on `stream`;
  * chunks of iterations are replayed from a captured CUDA graph when `stream`
  * is not the legacy default stream. */
 IMDP_API imdp_status imdp_session_step(imdp_session* s, int32_t n_iters, void* stream);
@@ -282,7 +283,8 @@ IMDP_API imdp_status imdp_session_read(imdp_session* s, int32_t index, double* V
                                        double* residual_out, int32_t* policy_out, void* stream);
 
 /* Bellman iterations launched by the session so far (one kernel launch each,
- * except on the single-CTA kernel, which runs a step call's iterations in one). */
+ * except on the single-CTA and resident kernels, which run a step call's
+ * iterations in one). */
 IMDP_API int64_t imdp_session_launches(const imdp_session* s);
 
 IMDP_API void imdp_session_destroy(imdp_session* s);
@@ -292,7 +294,14 @@ IMDP_API void imdp_session_destroy(imdp_session* s);
  * paper, whose GPU kernels have one fixed shape). Every configuration computes
  * the same words; they differ in speed only. Zero fields mean "by rule".
  *   kernel        0 by rule: the single-CTA kernel for a session of one small
- *                 problem; else, from the shape of the session's problems (the
+ *                 problem; else step calls of 4 or more iterations run them in one
+ *                 launch of the resident kernel where its values fit shared memory
+ *                 and its cost model says it pays (no state slices, one storage
+ *                 format): every problem, or every part of one finite-horizon
+ *                 problem that no transition leaves, belongs to a thread-block
+ *                 cluster that iterates it with the values on chip. Everything
+ *                 else runs one iteration per launch (what imdp_session_get_launch
+ *                 reports), from the shape of the session's problems (the
  *                 autotuner's choices on GB300 for the benchmark shapes), direct
  *                 with 3 CTAs per SM and 1024-entry tiles when their columns hold
  *                 256 or more transitions on average, otherwise slice with 3 CTAs

@@ -118,6 +118,9 @@ struct DevModel {
   std::vector<int32_t> h_wide;      // wide states (in no tile)
   int2* wide = nullptr;             // device copy as (problem 0, state)
   int32_t n_wide = 0;
+  // State boundaries that no transition crosses, 0 and n_states included: the
+  // states between two of them are a Markov decision process of their own.
+  std::vector<int32_t> h_parts;
   SliceLayout* slices = nullptr;    // built on first use by a session that runs the slice kernel
   std::mutex slices_mu;
 };
@@ -256,6 +259,34 @@ struct StepLaunch {
   int32_t stall;       // test hook: the producer issues nothing, so every wait runs out
 };
 
+// The resident kernel (resident.cu): all iterations of a step call in one
+// launch, each part (a problem, or the states between two boundaries of its
+// model's h_parts) run by one thread-block cluster that keeps the part's values
+// in shared memory.
+constexpr int kMaxCluster = 16;
+constexpr int32_t kResidentThreads = 768;  // threads of an SM (80 registers each), as one CTA or two
+constexpr size_t kResidentSmem = 232448;  // dynamic shared memory one CTA can have
+constexpr int32_t kResidentSteps = 4;  // step calls of fewer iterations launch one by one
+struct ResidentUnit {
+  int32_t p;       // problem
+  int32_t s0, s1;  // its states [s0, s1)
+};
+struct ResidentPlan {
+  const ResidentUnit* units;  // in the order the clusters take them (longest work first)
+  const int32_t* bounds;      // cluster + 1 per unit: the states of each rank
+  int32_t n_units;
+  int32_t cluster;            // CTAs of a cluster
+  int32_t clusters;           // clusters in the launch
+  int32_t threads;            // of a CTA
+  int32_t group;              // lanes to a column in the warm start
+  int32_t parts;              // the units are parts of one finite-horizon problem
+  int32_t f32;                // 32-bit storage
+  int32_t single;             // every state has one action
+  int32_t cap_states, cap_cols, cap_own;  // largest unit; most columns and states of one rank
+  int32_t max_col;            // longest column
+  uint32_t smem;
+};
+
 // NVTX range for the host-side phases (model upload, session steps, server
 // chunks); shows up in Nsight timelines, free when no tool is attached.
 struct TraceRange {
@@ -277,6 +308,13 @@ cudaError_t launch_bellman_step(const StepLaunch& L, int grid, cudaStream_t st, 
 // n_iters Bellman iterations of a session's single small problem (L.tiny_ok) in
 // one launch of one CTA.
 cudaError_t launch_bellman_tiny(const StepLaunch& L, int32_t n_iters, bool f32, cudaStream_t st);
+// resident.cu
+// Shared memory of one CTA for parts of `states` states, `cols` columns and `own` states of a rank.
+size_t resident_bytes(int32_t states, int32_t cols, int32_t own, bool f32, int32_t threads);
+// Fills R.clusters (how many fit the GPU).
+cudaError_t resident_prepare(ResidentPlan& R);
+// n_iters Bellman iterations of every unit in one launch.
+cudaError_t launch_bellman_resident(const StepLaunch& L, const ResidentPlan& R, int32_t n_iters, cudaStream_t st);
 // CTAs of the persistent tiled kernel: one per SM.
 int bellman_grid();
 // The configuration a launch of `L` with `cfg` (nullable) actually uses: kernel,
@@ -352,6 +390,9 @@ struct Session {
   // Point every problem at its model's slice layout (built if needed) and
   // allocate the per-column q; idempotent.
   imdp_status prepare_slices(cudaStream_t st);
+  // Step calls by rule: the resident kernel's plan (n_units 0: not taken).
+  ResidentPlan resident{};
+  imdp_status plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st);
   SideStream side;  // created when the session has both tiles and wide states
   LaunchConfig cfg;  // launch configuration (rule, set_launch or the autotuner)
   StepLaunch L{};

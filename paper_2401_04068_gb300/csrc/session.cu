@@ -293,8 +293,10 @@ imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<
     S->L.shape_f32 = all32 ? 1 : 0;
   }
   S->grid = bellman_grid();
+  imdp_status r = S->plan_resident(specs, st);
+  if (r != IMDP_OK) { delete S; return r; }
   const bool slice = resolve_launch(S->L, &S->cfg).kernel == kKernelSlice;
-  imdp_status r = slice ? S->prepare_slices(st) : IMDP_OK;
+  r = slice ? S->prepare_slices(st) : IMDP_OK;
   if (r != IMDP_OK) { delete S; return r; }
   std::vector<Tile> tiles;
   std::vector<int2> wide;
@@ -304,6 +306,157 @@ imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<
   r = S->reset(st);
   if (r != IMDP_OK) { delete S; return r; }
   *out = S;
+  return IMDP_OK;
+}
+
+imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st) {
+  resident = ResidentPlan{};
+  if (L.tiny_ok) return IMDP_OK;
+  bool any32 = false, any64 = false;
+  for (const DevModel* m : models) {
+    if (is_slice(m)) return IMDP_OK;
+    (m->lg32 ? any32 : any64) = true;
+  }
+  if (any32 && any64) return IMDP_OK;
+  const bool f32 = any32;
+  // units: the problems, or the parts of one finite-horizon problem (small
+  // neighbours together, so that a CTA's warps have columns enough)
+  struct Work {
+    ResidentUnit u;
+    int64_t entries, work;
+  };
+  std::vector<Work> us;
+  auto entries_of = [&](const DevModel* m, int32_t a, int32_t b) {
+    return (int64_t)m->h_colptr[m->h_stateptr[b]] - m->h_colptr[m->h_stateptr[a]];
+  };
+  const bool parts = count == 1 && !specs[0]->infinite_time && models[0]->h_parts.size() > 2;
+  if (parts) {
+    const DevModel* m = models[0];
+    const std::vector<int32_t>& b = m->h_parts;
+    const int64_t least = std::min<int64_t>(192, std::max<int64_t>(1, m->n_cols / (8 * grid)));  // columns of a unit
+    for (size_t i = 0; i + 1 < b.size();) {
+      size_t j = i + 1;
+      while (j + 1 < b.size() && m->h_stateptr[b[j]] - m->h_stateptr[b[i]] < least) ++j;
+      const int64_t e = entries_of(m, b[i], b[j]);
+      us.push_back(Work{ResidentUnit{0, b[i], b[j]}, e, e});
+      i = j;
+    }
+  } else {
+    for (int p = 0; p < count; ++p) {
+      const int64_t e = entries_of(models[p], 0, models[p]->n_states);
+      const int64_t K = specs[p]->infinite_time ? 1000 : specs[p]->horizon;
+      us.push_back(Work{ResidentUnit{p, 0, models[p]->n_states}, e, e * std::max<int64_t>(K, 1)});
+    }
+  }
+  int64_t entries = 0, work = 0, most = 0, cols = 0;
+  int32_t states = 0, max_col = 0;
+  for (const Work& w : us) {
+    entries += w.entries;
+    work += w.work;
+    most = std::max(most, w.work);
+    states = std::max(states, w.u.s1 - w.u.s0);
+  }
+  resident.single = 1;
+  for (const DevModel* m : models) {
+    max_col = std::max(max_col, m->max_col);
+    cols += m->n_cols;
+    resident.single = resident.single && m->n_cols == m->n_states;
+  }
+  const int32_t n_units = (int32_t)us.size();
+  std::stable_sort(us.begin(), us.end(), [](const Work& a, const Work& b) { return a.work > b.work; });
+  // Cluster size. More CTAs to a unit cost synchronisation; fewer leave the GPU
+  // idle (too few units), end on one long unit (uneven work), or keep so much in
+  // progress that it no longer sits in L2. Measured (64-bit storage, ms): 4096
+  // parts of 0.5 MB 66 / 69 / 96 with 1 / 2 / 4 CTAs; 256 problems of 5 MB on
+  // average with horizons from 100 to 500 82 / 88 / 98 with 4 / 6 / 8.
+  const double unit_bytes = (double)entries / n_units * (f32 ? 12.0 : 20.0);
+  int c = 1;
+  while (c < kMaxCluster && ((int64_t)n_units * c < grid || unit_bytes * (grid / c) > 200e6 ||
+                             (double)most / c > 1.7 * (double)work / grid))
+    c *= 2;
+  // Two CTAs of an SM overlap each other's barriers while both their units stay
+  // in L2 (4096 parts of 0.3 MB on 32-bit storage: 68 ms against 74 with one).
+  const bool two = n_units * (int64_t)c >= 2 * grid && unit_bytes * (2 * grid / c) <= 100e6;
+  resident.threads = two ? kResidentThreads / 2 : kResidentThreads;
+  // Against the per-iteration launches: those take about 10 us and stream 0.64
+  // transitions a cycle and SM, this kernel about 3 us and 1.17 on the SMs it covers.
+  const double sms = std::min<double>(grid, (double)n_units * c), hz = 1.9e9;
+  if (3e-6 + (double)entries / (1.17 * sms * hz) > 10e-6 + (double)entries / (0.64 * grid * hz)) return IMDP_OK;
+  // ranks of a unit: contiguous states of about equal work
+  std::vector<int32_t> bounds;
+  int64_t rank_entries = 0;
+  for (;; c *= 2) {
+    if (c > kMaxCluster || resident_bytes(states, 1, 1, f32, resident.threads) > kResidentSmem) return IMDP_OK;
+    resident.cap_cols = 32;
+    resident.cap_own = 0;
+    rank_entries = 0;
+    bounds.clear();
+    bounds.reserve((size_t)n_units * (c + 1));
+    for (const Work& w : us) {
+      const DevModel* m = models[w.u.p];
+      const int32_t* sp = m->h_stateptr.data();
+      const int32_t* cp = m->h_colptr.data();
+      const uint8_t* fx = fixed_h.data() + base_h[w.u.p];
+      auto cost = [&](int32_t s) -> int64_t {
+        return fx[s] ? 1 : cp[sp[s + 1]] - cp[sp[s]] + 24 * (sp[s + 1] - sp[s]);
+      };
+      int64_t total = 0, done = 0;
+      if (c > 1)
+        for (int32_t s = w.u.s0; s < w.u.s1; ++s) total += cost(s);
+      int32_t s = w.u.s0, prev = s;
+      bounds.push_back(s);
+      for (int r = 1; r <= c; ++r) {
+        if (r == c)
+          s = w.u.s1;
+        else
+          while (s < w.u.s1 && done * c < total * r) done += cost(s++);
+        bounds.push_back(s);
+        resident.cap_own = std::max(resident.cap_own, s - prev);
+        resident.cap_cols = std::max(resident.cap_cols, sp[s] - sp[prev]);
+        rank_entries = std::max<int64_t>(rank_entries, cp[sp[s]] - cp[sp[prev]]);
+        prev = s;
+      }
+    }
+    const size_t need = resident_bytes(states, resident.cap_cols, resident.cap_own, f32, resident.threads);
+    if (need <= kResidentSmem && resident.cap_cols <= 65535) {
+      // one unit: its entries go to shared memory as well where they fit (no L2
+      // latency in its iterations; pendulum_240 alone 1.03 ms against 1.11). With
+      // many units the wider clusters that takes cost more than it saves.
+      const size_t all = need + 64 + (size_t)rank_entries * 20;
+      resident.smem = (uint32_t)(n_units == 1 && all <= kResidentSmem ? all : need);
+      break;
+    }
+  }
+  const double k = (double)entries / std::max<int64_t>(cols, 1);
+  // lanes to a column: whole warps when the columns are long or too few for groups
+  resident.group = k >= 256 || (double)cols / n_units / c < 4.0 * resident.threads / 32 / 2 ? 32 : 8;
+  resident.cluster = c;
+  resident.parts = parts ? 1 : 0;
+  resident.f32 = f32 ? 1 : 0;
+  resident.cap_states = states;
+  resident.max_col = max_col;
+  resident.n_units = n_units;
+  cudaError_t e = resident_prepare(resident);
+  if (e != cudaSuccess) {  // clusters this wide do not fit the device: the per-iteration kernels run
+    cudaGetLastError();
+    resident.n_units = 0;
+    return IMDP_OK;
+  }
+  std::vector<ResidentUnit> uh(n_units);
+  for (int32_t i = 0; i < n_units; ++i) uh[i] = us[i].u;
+  ResidentUnit* du = alloc<ResidentUnit>(uh.size());
+  int32_t* db = alloc<int32_t>(bounds.size());
+  if (!du || !db) {
+    resident.n_units = 0;
+    set_error("device allocation failed (session)");
+    return IMDP_ENOMEM;
+  }
+  e = cudaMemcpyAsync(du, uh.data(), sizeof(ResidentUnit) * uh.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(db, bounds.data(), sizeof(int32_t) * bounds.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host vectors go out of scope
+  if (e != cudaSuccess) return cuda_status(e, "session plan");
+  resident.units = du;
+  resident.bounds = db;
   return IMDP_OK;
 }
 
@@ -513,6 +666,14 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
   if (resolve_launch(L, &cfg).kernel == kKernelTiny) {
     // one small problem: all n iterations in one launch of one CTA
     e = launch_bellman_tiny(L, n, models[0]->lg32 != nullptr, st);
+    if (e != cudaSuccess) return cuda_status(e, "bellman step");
+    launches += n;
+    launched_since_reset += n;
+    return IMDP_OK;
+  }
+  if (cfg.kernel == kKernelRule && resident.n_units > 0 && n >= kResidentSteps) {
+    // by rule: all n iterations in one launch of the resident kernel
+    e = launch_bellman_resident(L, resident, n, st);
     if (e != cudaSuccess) return cuda_status(e, "bellman step");
     launches += n;
     launched_since_reset += n;
