@@ -283,7 +283,7 @@ IMDP_API imdp_status imdp_session_read(imdp_session* s, int32_t index, double* V
                                        double* residual_out, int32_t* policy_out, void* stream);
 
 /* Bellman iterations launched by the session so far (one kernel launch each,
- * except on the single-CTA and resident kernels, which run a step call's
+ * except on the single-CTA, resident and grid kernels, which run a step call's
  * iterations in one). */
 IMDP_API int64_t imdp_session_launches(const imdp_session* s);
 
@@ -299,8 +299,11 @@ IMDP_API void imdp_session_destroy(imdp_session* s);
  *                 and its cost model says it pays (no state slices, one storage
  *                 format): every problem, or every part of one finite-horizon
  *                 problem that no transition leaves, belongs to a thread-block
- *                 cluster that iterates it with the values on chip. Everything
- *                 else runs one iteration per launch (what imdp_session_get_launch
+ *                 cluster that iterates it with the values on chip; or, one problem
+ *                 of fewer than 32 million transitions, in one launch of the grid
+ *                 kernel, whose CTAs each keep the values their states need on chip
+ *                 and wait for one another after every iteration. Everything else
+ *                 runs one iteration per launch (what imdp_session_get_launch
  *                 reports), from the shape of the session's problems (the
  *                 autotuner's choices on GB300 for the benchmark shapes), direct
  *                 with 3 CTAs per SM and 1024-entry tiles when their columns hold

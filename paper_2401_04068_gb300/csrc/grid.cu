@@ -1,0 +1,818 @@
+// Grid kernel: all iterations of a step call of one problem in one launch of the
+// whole GPU (a cooperative launch; one CTA per SM), for problems too large for
+// one thread-block cluster.
+//
+// Every CTA owns the same few chunks of consecutive states in every iteration
+// (dealt round-robin, so that regions where many thresholds move are spread over
+// the CTAs). Their column words, threshold hints and reach/avoid mask stay in
+// shared memory, and so does the window of V_{k-1} that the chunks' columns
+// name: consecutive states of an abstraction reach overlapping runs of states,
+// and a column's last destination alone may lie outside (an absorbing
+// out-of-domain state, say). Warps take the CTA's columns from a counter, longest
+// first, for the warm start. Columns it does not decide are settled by the CTA's
+// warps when they are few; otherwise they are listed in global memory, and CTAs
+// that have finished take them from any list (a few regions hold most of them:
+// with each CTA settling its own, pimdp_2 spends 27 % of its time waiting). One
+// barrier of the grid ends an iteration, three when misses were listed.
+//
+// A per-iteration launch of the direct kernel has a chain of dependent loads in
+// front of every tile (tile counter, tile, descriptor, column words, hint entry,
+// its value) and gathers V through L1 and L2; here nothing but the entries
+// themselves is loaded in the loop, and entries that fit stay in shared memory.
+// The warm start streams at 0.8 of the copy bandwidth (pimdp_2, 300,000 cycles
+// an iteration); a missed column takes 15,000 to 45,000 cycles of a warp, which
+// is what bounds the first iterations of every model. Measured, K = 200 or to
+// convergence: 20,000 states of 24 scattered transitions 3.6 -> 1.75 ms,
+// cartpole_960 4.9 -> 2.5, harrier 43.7 -> 36.2, cartpole_3840 13.7 -> 13.0.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstring>
+
+#include "resident.cuh"
+
+namespace imdp {
+
+namespace {
+
+constexpr int kGridThreads = 768;
+constexpr int kGridWarps = kGridThreads / 32;
+// Misses that a CTA settles by itself, two rounds of its warps; more are listed
+// for all CTAs, which costs two more barriers.
+constexpr uint32_t kGridFewMisses = 2 * kGridWarps;
+constexpr int kSettleTrips = 4;  // trips in flight while a missed column is settled
+constexpr int kGridBuckets = 256;  // length classes of the column order, as in the resident kernel
+constexpr long long kGridWaitCycles = 4000000000ll;  // ~2 s at 2 GHz: bound of the grid barrier's wait
+
+struct alignas(16) GridCol {
+  uint64_t rem;   // 1 - sum(lower) (rem_of)
+  int32_t a, k;   // first entry (of the model's arrays, or of the CTA's copy), entries
+  int32_t e;      // entry the warm start tries (-1: none; 0 when rem = 0)
+  int32_t hrow;   // its destination
+  int32_t x;      // 32-bit storage: shift, or the offset in lgx of a correction column
+  uint32_t lc;    // local column, and flags
+  int32_t win;    // window
+  int32_t last;   // destination of the last entry when it lies outside the window, else -1
+  int32_t c;      // column of the model
+};
+
+// A state that the property leaves free, and where its columns' values are.
+struct GridState {
+  int32_t s, jb, je;  // state; local columns [jb, je)
+};
+
+struct GridShared {
+  Problem prob;
+  uint32_t hist[kGridBuckets];
+  uint32_t next[2];  // columns taken: 32-bit ones (or all), correction columns
+  unsigned long long part[kGridWarps];
+  int32_t n32, n_cols, n_own, n_win;
+  uint32_t n_free, n_lc;
+  int32_t copied;
+  EntryCopy copy;
+  int32_t ok;
+  uint32_t n_miss, taken, total;  // the CTA's misses, those taken; all that were listed
+  int32_t chunk_s0[kGridMaxChunks], chunk_own[kGridMaxChunks + 1];
+  GridWindow win[kGridMaxChunks];  // `off`: byte offset of state 0's (virtual) cell
+  int32_t win_at[kGridMaxChunks + 1];  // cells before the window
+};
+
+struct GridLayout {
+  size_t cols, q, states, v, ws, data;
+};
+__host__ __device__ inline GridLayout grid_layout(int32_t cols, int32_t own, int32_t cells, int cell) {
+  auto up = [](size_t x) { return (x + 15) & ~size_t(15); };
+  GridLayout l;
+  size_t o = up(sizeof(GridShared));
+  l.cols = o; o = up(o + (size_t)cols * sizeof(GridCol));
+  l.q = o;    o = up(o + (size_t)cols * sizeof(uint64_t));
+  l.states = o; o = up(o + (size_t)own * sizeof(GridState));
+  l.v = o;    o = up(o + (size_t)cells * cell);
+  l.ws = o;   o = up(o + kGridWarps * sizeof(WarpScratch));
+  l.data = o;
+  return l;
+}
+
+// V in one of the CTA's windows: `off` is where state 0's cell would be.
+template <bool f32>
+struct WindowV {
+  int32_t off;
+  __device__ __forceinline__ uint64_t at(int32_t r) const {
+    return *reinterpret_cast<const uint64_t*>(resident_sm + (int32_t)(off + r * 8));
+  }
+  __device__ __forceinline__ uint32_t hi(int32_t r) const { return (uint32_t)(at(r) >> 32); }
+};
+template <>
+struct WindowV<true> {
+  int32_t off;
+  __device__ __forceinline__ uint32_t hi(int32_t r) const {
+    return *reinterpret_cast<const uint32_t*>(resident_sm + (int32_t)(off + r * 4));
+  }
+  __device__ __forceinline__ uint64_t at(int32_t r) const { return (uint64_t)hi(r) << 32; }
+};
+// The same, with states outside the window read from global memory.
+template <bool f32>
+struct AnyV {
+  WindowV<f32> w;
+  int32_t w0, len;
+  const uint64_t* g;
+  __device__ __forceinline__ uint64_t at(int32_t r) const {
+    return (uint32_t)(r - w0) < (uint32_t)len ? w.at(r) : __ldcg(reinterpret_cast<const unsigned long long*>(g) + r);
+  }
+  __device__ __forceinline__ uint32_t hi(int32_t r) const { return (uint32_t)(at(r) >> 32); }
+};
+
+// V from global memory, written by other CTAs before the last barrier (not by
+// the non-coherent path).
+struct CoherentV {
+  const uint64_t* g;
+  __device__ __forceinline__ uint64_t at(int32_t r) const {
+    uint64_t v;
+    asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(g + r));
+    return v;
+  }
+  __device__ __forceinline__ uint32_t hi(int32_t r) const { return (uint32_t)(at(r) >> 32); }
+};
+
+// Barrier `n` (1, 2, ...) of the launch's CTAs: writes before it are visible
+// after it (read values written by other CTAs past L1). False when the wait
+// gave up or another CTA did.
+// Split in two: arrive (writes of the CTA before it), wait.
+__device__ __forceinline__ void grid_arrive(StepControl* ctl) {
+  __threadfence();
+  atomicAdd(&ctl->arrived, 1u);
+}
+__device__ __forceinline__ bool grid_arrived(const StepControl* ctl, uint32_t target) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->arrived) : "memory");
+  return v >= target;
+}
+// One poll of a wait that began at t0: false when it gave up or another CTA did.
+__device__ __forceinline__ bool grid_waiting(StepControl* ctl, long long t0) {
+  if (*(volatile unsigned*)&ctl->error) return false;
+  if (clock64() - t0 <= kGridWaitCycles) return true;
+  atomicExch(&ctl->error, 1u);
+  return false;
+}
+__device__ __forceinline__ bool grid_sync(StepControl* ctl, uint32_t n, GridShared& S) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const uint32_t target = n * gridDim.x;
+    grid_arrive(ctl);
+    const long long t0 = clock64();
+    int ok = 1;
+    for (uint32_t i = 0; !grid_arrived(ctl, target); ++i)
+      if ((i & 255) == 255 && !grid_waiting(ctl, t0)) {
+        ok = 0;
+        break;
+      }
+    S.ok = ok;
+    __threadfence();
+  }
+  __syncthreads();
+  return S.ok != 0;
+}
+
+struct GridTable {
+  GridCol* col;
+  uint64_t* q;
+  GridState* st;
+};
+
+template <bool f32, int G>
+__device__ void build_grid_columns(const Problem& P, const GridTable& T, int n_chunks, int32_t max_col,
+                                   GridShared& S) {
+  const int tid = threadIdx.x;
+  const int32_t unit = max((max_col + 126 * G) / (127 * G), 1) * G;  // entries per length class
+  for (int i = tid; i < kGridBuckets; i += kGridThreads) S.hist[i] = 0;
+  if (tid == 0) S.n_free = S.n_lc = 0;
+  __syncthreads();
+  const int all = S.chunk_own[n_chunks];
+  auto bucket = [&](int32_t c, int32_t k) {
+    const int b = 127 - min((k + unit - 1) / unit, 127);
+    return f32 && P.xoff && P.xoff[c] >= 0 ? 128 + b : b;
+  };
+  auto chunk_of = [&](int t) {
+    int j = 0;
+    while (j + 1 < n_chunks && t >= S.chunk_own[j + 1]) ++j;
+    return j;
+  };
+  for (int t = tid; t < all; t += kGridThreads) {
+    const int j = chunk_of(t);
+    const int32_t s = S.chunk_s0[j] + (t - S.chunk_own[j]);
+    if (P.fixed[s] != 0) continue;  // Eq. 2 fixes reach and avoid states (both buffers hold their values)
+    const int32_t jb = P.stateptr[s], je = P.stateptr[s + 1];
+    const int at = (int)atomicAdd(&S.n_free, 1u);
+    const int32_t lc = (int32_t)atomicAdd(&S.n_lc, (uint32_t)(je - jb));
+    T.st[at] = GridState{s, lc, lc + (je - jb)};
+    for (int32_t c = jb; c < je; ++c) atomicAdd(&S.hist[bucket(c, P.colptr[c + 1] - P.colptr[c])], 1u);
+  }
+  __syncthreads();
+  if (tid < 32) {
+    uint32_t h[kGridBuckets / 32], sum = 0;
+    for (int i = 0; i < kGridBuckets / 32; ++i) {
+      h[i] = S.hist[tid * (kGridBuckets / 32) + i];
+      sum += h[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (tid >= o) incl += y;
+    }
+    uint32_t at = incl - sum;
+    for (int i = 0; i < kGridBuckets / 32; ++i) {
+      S.hist[tid * (kGridBuckets / 32) + i] = at;
+      at += h[i];
+    }
+    const int total = (int)__shfl_sync(kFull, incl, 31);
+    const int n32 = (int)__shfl_sync(kFull, incl - sum, 16);
+    if (tid == 0) {
+      S.n32 = f32 ? n32 : total;
+      S.n_cols = total;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) S.n_own = (int32_t)S.n_free;
+  for (int t = tid; t < (int)S.n_free; t += kGridThreads) {
+    const GridState g = T.st[t];
+    const int32_t s = g.s;
+    int j = 0;
+    while (j + 1 < n_chunks && !(s >= S.chunk_s0[j] && s - S.chunk_s0[j] < S.chunk_own[j + 1] - S.chunk_own[j])) ++j;
+    const int32_t c0 = P.stateptr[s] - g.jb;  // local column of c: c - c0
+    const int w = S.n_win == 1 ? 0 : j;
+    const int32_t w0 = S.win[w].w0, w1 = w0 + S.win[w].len;
+    for (int32_t c = P.stateptr[s]; c < P.stateptr[s + 1]; ++c) {
+      const int32_t a = P.colptr[c], k = P.colptr[c + 1] - a;
+      const int at = (int)atomicAdd(&S.hist[bucket(c, k)], 1u);
+      const int32_t h = P.hint[c], e = hint_entry(h);
+      const uint64_t word = P.rem[c], rem = rem_of(word);
+      const int32_t last = k > 0 ? P.rowval[a + k - 1] : w0;
+      GridCol col;
+      col.rem = rem;
+      col.a = a;
+      col.k = k;
+      col.e = rem == 0 ? 0 : (e >= 0 && e < k ? e : -1);
+      col.hrow = rem != 0 && e >= 0 && e < k ? P.rowval[a + e] : w0;
+      col.lc = (uint32_t)(c - c0) | (h <= -2 ? kMoving : 0u) | (rem != 0 && !narrow_of(word) ? kCarry : 0u);
+      col.x = 0;
+      if (f32) {
+        const int32_t x = P.xoff ? P.xoff[c] : -1;
+        col.x = x >= 0 ? x : P.shift[c];
+      }
+      col.win = w;
+      col.c = c;
+      col.last = last >= w1 ? last : -1;
+      T.col[at] = col;
+    }
+  }
+  __syncthreads();
+}
+
+// The columns' entries behind one another in shared memory, where they fit.
+template <bool f32>
+__device__ void copy_grid_entries(const Problem& P, const GridTable& T, uint32_t off, uint32_t room, GridShared& S) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n_cols = S.n_cols, n32 = S.n32;
+  // (q is free until the first iteration: it holds where a column's copy starts)
+  if (warp == 0) {
+    uint32_t at = 0, e32 = 0;
+    for (int base = 0; base < n_cols; base += 32) {
+      const int i = base + lane;
+      const uint32_t k = i < n_cols ? (uint32_t)T.col[i].k : 0u;
+      uint32_t incl = k;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      if (i < n_cols) T.q[i] = at + incl - k;
+      const uint32_t sum = __shfl_sync(kFull, incl, 31);
+      if (base < n32) e32 = at + __shfl_sync(kFull, incl, min(n32 - base, 32) - 1);
+      at += sum;
+    }
+    if (lane == 0) {
+      const size_t e = at;
+      const size_t rows = (4 * e + 15) & ~size_t(15), pairs = f32 ? (8 * (size_t)e32 + 15) & ~size_t(15) : 16 * e;
+      const size_t exact = f32 ? 16 * (e - e32) : 0;
+      S.copied = rows + pairs + exact <= room ? 1 : 0;
+      S.copy.rows = off;
+      S.copy.pairs = off + (uint32_t)rows;
+      S.copy.exact = off + (uint32_t)(rows + pairs) - 16u * e32;
+    }
+  }
+  __syncthreads();
+  if (!S.copied) return;
+  const EntryCopy D = S.copy;
+  for (int i = warp; i < n_cols; i += kGridWarps) {
+    const int32_t a = T.col[i].a, k = T.col[i].k, x = T.col[i].x;
+    const uint32_t at = (uint32_t)T.q[i];
+    for (int32_t t = lane; t < k; t += 32) {
+      at_shared<int32_t>(D.rows)[at + t] = P.rowval[a + t];
+      if (!f32)
+        at_shared<ulonglong2>(D.pairs)[at + t] = P.lg[a + t];
+      else if (i >= n32)
+        at_shared<ulonglong2>(D.exact + 16u * at)[t] = P.lgx[x + t];
+      else
+        at_shared<uint2>(D.pairs)[at + t] = P.lg32[a + t];
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < n_cols; i += kGridThreads) T.col[i].a = (int32_t)T.q[i];
+  __syncthreads();
+}
+
+// The columns [i0, i1) of the table, taken G-lane groups at a time from
+// `next`: the warm start; the columns it does not decide go to the CTA's part
+// of the miss list.
+template <bool f32, bool w64, int G, bool pess, bool copied>
+__device__ __forceinline__ void grid_columns(const Problem& P, const GridTable& T,
+                                             const Entries<typename PairOf<w64>::type, copied> src, int i0, int i1,
+                                             bool exact, const uint64_t* Vg, int lane, uint32_t* next, GridMiss* misses,
+                                             GridShared& S) {
+  typedef typename PairOf<w64>::type Pair;
+  constexpr int NG = 32 / G;
+  const int gi = lane / G, gl = lane % G;
+  for (;;) {
+    int base = 0;
+    if (lane == 0) base = (int)atomicAdd(next, (uint32_t)NG);
+    base = i0 + __shfl_sync(kFull, base, 0);
+    if (base >= i1) break;
+    const int i = min(base + gi, i1 - 1);  // a group past the end reads the last column along
+    GridCol& c = T.col[i];
+    const uint64_t rem = c.rem;
+    const int32_t a = c.a, k = c.k, tried = c.e, hrow = c.hrow, x = c.x, last = c.last;
+    const uint32_t lc = c.lc;
+    const GridWindow win = S.win[c.win];
+    WarmSums s{0, 0, 0};
+    uint64_t vk = 0;
+    bool narrow = true;
+    if (__any_sync(kFull, tried >= 0)) {
+      const int32_t kk = last >= 0 ? k - 1 : k;
+      const int full = (int)__reduce_min_sync(kFull, (unsigned)kk) / G;
+      const int trips = ((int)__reduce_max_sync(kFull, (unsigned)kk) + G - 1) / G;
+      Entries<Pair, copied> e = src;
+      e.skip_rows(a + gl);
+      e.skip_pairs((!copied && w64 && exact ? x : a) + gl);
+      // the last entry, when its destination is outside the window
+      const bool tail = last >= 0 && gl == 0;
+      uint64_t tv = 0;
+      Pair tb{};
+      if (tail) {
+        tv = __ldcg(reinterpret_cast<const unsigned long long*>(Vg) + last);
+        tb = e.pair(k - 1);
+      }
+      vk = (uint32_t)(hrow - win.w0) < (uint32_t)win.len
+               ? WindowV<f32>{win.off}.at(hrow)
+               : __ldcg(reinterpret_cast<const unsigned long long*>(Vg) + hrow);
+      if (rem == 0) vk = pess ? 0ull : ~0ull;  // a key no value passes: every entry keeps its lower bound
+      if (w64) narrow = !__any_sync(kFull, (lc & kCarry) != 0);
+      const WindowV<f32> V{win.off};
+      typedef typename std::conditional<w64, uint64_t, uint32_t>::type Val;
+      const Val vkv = w64 ? (Val)vk : (Val)(vk >> 32), tvv = w64 ? (Val)tv : (Val)(tv >> 32);
+      if (narrow) {
+        s = lane_sums<w64, G, pess, false>(e, kk - gl, full, trips, V, vk, x, win.w0);
+        if (__any_sync(kFull, tail)) warm_term<pess, false>(s, tvv, tb, vkv, x);
+      } else {
+        s = lane_sums<w64, G, pess, true>(e, kk - gl, full, trips, V, vk, x, win.w0);
+        if (__any_sync(kFull, tail)) warm_term<pess, true>(s, tvv, tb, vkv, x);
+      }
+      s.acc = group_sum<G>(s.acc);
+      if (narrow) {
+        s.chosen = group_sum<G>(s.chosen);
+        s.geq = group_sum<G>(s.geq);
+      } else {
+        s.chosen = group_sum_sat<G>(s.chosen);
+        s.geq = group_sum_sat<G>(s.geq);
+      }
+    }
+    // on 32-bit storage in units of the mantissas: rem and 1 - rem are multiples of 2^(32 - x)
+    const uint64_t r = w64 ? rem : rem >> (32 - x), lows = w64 ? kOne - rem : (kOne - rem) >> (32 - x);
+    const uint64_t flt = narrow ? s.chosen - lows : s.chosen;
+    const uint64_t part = rem == 0 ? 0ull : r - flt;
+    const bool mine = gl == 0 && base + gi < i1;
+    const bool hit = tried >= 0 && (rem == 0 || (flt < r && part <= s.geq));
+    if (mine && hit) {
+      T.q[lc & kLocalColumn] = s.acc + (w64 ? __umul64hi(vk, part) : mul_shr(vk >> 32, part, x));
+      if (lc & kMoving) c.lc = lc & ~kMoving;
+    }
+    if (mine && !hit) {
+      GridMiss m;
+      m.rem = rem;
+      m.vk = vk;
+      m.acc = s.acc;
+      m.flt = flt;
+      m.geq = s.geq;
+      m.i = i;
+      m.c = c.c;
+      m.k = k;
+      m.neighbor = tried >= 0 && !(lc & kMoving) ? 1 : 0;
+      m.hint = 0;
+      m.pad = 0;
+      misses[atomicAdd(&S.n_miss, 1u)] = m;
+    }
+  }
+}
+
+// A record of another warp or CTA (written before a fence or barrier).
+__device__ __forceinline__ GridMiss load_miss(const GridMiss* p) {
+  GridMiss m;
+  const uint4* from = reinterpret_cast<const uint4*>(p);
+  uint4* to = reinterpret_cast<uint4*>(&m);
+#pragma unroll
+  for (int i = 0; i < (int)(sizeof(GridMiss) / 16); ++i) to[i] = __ldcg(from + i);
+  return m;
+}
+
+// Settles one missed column; its value and hint go to its record. `own`: the
+// CTA's own column (its table, windows and copy), else another CTA's.
+template <bool f32, bool copied>
+__device__ __forceinline__ void settle_own(const Problem& P, const GridTable& T, const EntryCopy& D, GridMiss* at,
+                                           const uint64_t* Vg, uint32_t scratch, int lane, const GridShared& S) {
+  const GridMiss m = load_miss(at);
+  const GridCol& c = T.col[m.i];
+  const GridWindow w = S.win[c.win];
+  const AnyV<f32> V{WindowV<f32>{w.off}, w.w0, w.len, Vg};
+  const bool pess = P.pessimistic != 0, nb = m.neighbor != 0;
+  const int32_t a = c.a, x = c.x;
+  int32_t ho;
+  uint64_t q;
+  if constexpr (copied) {
+    const XRows rows{D.rows + a * 4u};
+    if (f32 && m.i < S.n32)
+      q = missed_column<true, 3, kSettleTrips>(rows, Bounds<true, 3>{D.pairs + a * 8u, 32 - x}, m.k, m.rem, V, pess, nb, m.vk, m.acc,
+                                 m.flt, m.geq, scratch, w.w0, lane, &ho);
+    else
+      q = missed_column<false, 3, kSettleTrips>(rows, Bounds<false, 3>{(f32 ? D.exact : D.pairs) + a * 16u, 0}, m.k, m.rem, V, pess, nb,
+                                  m.vk, m.acc, m.flt, m.geq, scratch, w.w0, lane, &ho);
+  } else {
+    const GRows rows{P.rowval + a};
+    if (f32 && m.i < S.n32)
+      q = missed_column<true, 1, kSettleTrips>(rows, Bounds<true, 1>{P.lg32 + a, 32 - x}, m.k, m.rem, V, pess, nb, m.vk, m.acc, m.flt,
+                                 m.geq, scratch, w.w0, lane, &ho);
+    else
+      q = missed_column<false, 1, kSettleTrips>(rows, Bounds<false, 1>{f32 ? P.lgx + x : P.lg + a, 0}, m.k, m.rem, V, pess, nb, m.vk,
+                                  m.acc, m.flt, m.geq, scratch, w.w0, lane, &ho);
+  }
+  if (lane == 0) {
+    at->acc = q;
+    at->hint = ho;
+  }
+}
+template <bool f32>
+__device__ __forceinline__ void settle_other(const Problem& P, GridMiss* at, const uint64_t* Vg, uint32_t scratch,
+                                             int lane) {
+  const GridMiss m = load_miss(at);
+  const CoherentV V{Vg};
+  const bool pess = P.pessimistic != 0, nb = m.neighbor != 0;
+  const int32_t a = __ldg(P.colptr + m.c);
+  const GRows rows{P.rowval + a};
+  int32_t ho, x = -1;
+  uint64_t q;
+  if (f32 && P.xoff) x = __ldg(P.xoff + m.c);
+  if (f32 && x < 0)
+    q = missed_column<true, 1, kSettleTrips>(rows, Bounds<true, 1>{P.lg32 + a, 32 - __ldg(P.shift + m.c)}, m.k, m.rem, V, pess, nb,
+                               m.vk, m.acc, m.flt, m.geq, scratch, 0, lane, &ho);
+  else
+    q = missed_column<false, 1, kSettleTrips>(rows, Bounds<false, 1>{f32 ? P.lgx + x : P.lg + a, 0}, m.k, m.rem, V, pess, nb, m.vk,
+                                m.acc, m.flt, m.geq, scratch, 0, lane, &ho);
+  if (lane == 0) {
+    at->acc = q;
+    at->hint = ho;
+  }
+}
+
+// The CTA's missed columns when there are few: by its warps, from a counter in
+// shared memory.
+template <bool f32, bool copied>
+__device__ __forceinline__ void settle_few(const Problem& P, const GridTable& T, const EntryCopy& D, GridMiss* mine,
+                                           uint32_t n, const uint64_t* Vg, uint32_t scratch, int lane, GridShared& S) {
+  for (;;) {
+    uint32_t j = 0;
+    if (lane == 0) j = atomicAdd(&S.taken, 1u);
+    j = __shfl_sync(kFull, j, 0);
+    if (j >= n) break;
+    settle_own<f32, copied>(P, T, D, mine + j, Vg, scratch, lane, S);
+  }
+}
+
+// Missed columns of this iteration, of the CTAs that listed them (`own` of this
+// one). First the CTA's own ones; once every CTA has listed its misses or settled
+// its few (barrier `target`, waited for by one thread of the CTA), those that are
+// left anywhere, until a look at all lists finds none. False when the wait gave up.
+template <bool f32, bool copied>
+__device__ bool settle_misses(const StepLaunch& L, const GridPlan& R, const Problem& P, const GridTable& T,
+                              const EntryCopy& D, const uint64_t* Vg, uint32_t scratch, int k, uint32_t target,
+                              uint32_t own, int lane, int warp, GridShared& S) {
+  const int n_cta = (int)gridDim.x, me = (int)blockIdx.x;
+  uint32_t* listed = R.steal + (size_t)(k & 1) * 2 * n_cta;  // per CTA: misses listed
+  uint32_t* taken = listed + n_cta;
+  GridMiss* mine = R.misses + (size_t)me * R.cap_cols;
+  while (own) {
+    uint32_t j = 0;
+    if (lane == 0) j = atomicAdd(&taken[me], 1u);
+    j = __shfl_sync(kFull, j, 0);
+    if (j >= own) break;
+    settle_own<f32, copied>(P, T, D, mine + j, Vg, scratch, lane, S);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const long long t0 = clock64();
+    int ok = 1;
+    for (uint32_t i = 0; !grid_arrived(L.ctl, target); ++i)
+      if ((i & 255) == 255 && !grid_waiting(L.ctl, t0)) {
+        ok = 0;
+        break;
+      }
+    S.ok = ok;
+    S.total = __ldcg(&L.ctl->misses[k & 3]);
+    __threadfence();
+  }
+  __syncthreads();
+  if (!S.ok) return false;
+  for (bool found = S.total != 0; found;) {
+    found = false;
+    for (int base = 0; base < n_cta; base += 32) {
+      int v = me + 1 + warp * 6 + base + lane;
+      v -= (v / n_cta) * n_cta;
+      const bool in = base + lane < n_cta && v != me;
+      const uint32_t n = in ? __ldcg(&listed[v]) : 0u;
+      unsigned m = __ballot_sync(kFull, n != 0 && __ldcg(&taken[v]) < n);
+      while (m) {
+        const int src = __ffs(m) - 1;
+        m &= m - 1;
+        const int victim = __shfl_sync(kFull, v, src);
+        const uint32_t many = __shfl_sync(kFull, n, src);
+        for (;;) {
+          uint32_t j = 0;
+          if (lane == 0) j = atomicAdd(&taken[victim], 1u);
+          j = __shfl_sync(kFull, j, 0);
+          if (j >= many) break;
+          found = true;
+          settle_other<f32>(P, R.misses + (size_t)victim * R.cap_cols + j, Vg, scratch, lane);
+        }
+      }
+    }
+  }
+  return true;
+}
+
+template <bool f32, int G, bool pess, bool copied>
+__device__ __forceinline__ int32_t grid_iterate(const StepLaunch& L, const Problem& P, const GridTable& T,
+                                                const GridLayout& lay, const GridPlan& R, int32_t k0, int32_t k1, GridShared& S) {
+  typedef typename std::conditional<f32, uint32_t, uint64_t>::type Cell;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const EntryCopy D = S.copy;
+  Entries<ulonglong2, copied> e64;
+  Entries<uint2, copied> e32;
+  if constexpr (copied) {
+    e32 = Entries<uint2, true>{D.rows, D.pairs};
+    e64 = Entries<ulonglong2, true>{D.rows, f32 ? D.exact : D.pairs};
+  } else {
+    e32 = Entries<uint2, false>{P.rowval, P.lg32};
+    e64 = Entries<ulonglong2, false>{P.rowval, f32 ? P.lgx : P.lg};
+  }
+  const uint32_t scratch = (uint32_t)(lay.ws + warp * sizeof(WarpScratch));
+  const bool infinite = P.infinite != 0, extra = infinite || P.policy_mode != 0;
+  const int n32 = S.n32, n_cols = S.n_cols, n_own = S.n_own, n_win = S.n_win;
+  Cell* cells = at_shared<Cell>((uint32_t)lay.v);
+  GridMiss* mine = R.misses + (size_t)blockIdx.x * R.cap_cols;
+  uint32_t barrier = 0;
+  int32_t k = k0;
+  for (;; ++k) {
+    const uint64_t* Vg = P.V[(k - 1) & 1];
+    uint64_t* Vout = P.V[k & 1];
+    // the windows of V_{k-1} (other CTAs wrote them: past L1)
+    for (int w = 0; w < n_win; ++w) {
+      const unsigned long long* from = reinterpret_cast<const unsigned long long*>(Vg) + S.win[w].w0;
+      Cell* to = cells + S.win_at[w];
+      for (int i = tid; i < S.win[w].len; i += kGridThreads) {
+        const uint64_t v = __ldcg(from + i);
+        to[i] = f32 ? (Cell)(v >> 32) : (Cell)v;
+      }
+    }
+    if (tid < 2) S.next[tid] = 0;
+    if (tid == 2) S.n_miss = S.taken = 0;
+    __syncthreads();
+    if (f32) {
+      grid_columns<f32, false, G, pess, copied>(P, T, e32, 0, n32, false, Vg, lane, &S.next[0], mine, S);
+      if (n32 < n_cols)
+        grid_columns<f32, true, G, pess, copied>(P, T, e64, n32, n_cols, true, Vg, lane, &S.next[1], mine, S);
+    } else {
+      grid_columns<f32, true, G, pess, copied>(P, T, e64, 0, n_cols, false, Vg, lane, &S.next[0], mine, S);
+    }
+    __syncthreads();
+    const uint32_t n_miss = S.n_miss;
+    // the states' new values, policy and residual
+    const auto states = [&]() {
+      unsigned long long dmax = 0;
+      for (int i = tid; i < n_own; i += kGridThreads) {
+        const GridState g = T.st[i];
+        const int32_t s = g.s;
+        uint64_t bestq;
+        int32_t best = 0;
+        if (R.single)
+          bestq = T.q[g.jb];
+        else
+          best_action(P, g.jb, g.je, [&](int32_t c) { return T.q[c]; }, &bestq, &best);
+        const uint64_t vnew = free_state_value(P, s, bestq);
+        Vout[s] = vnew;
+        if (extra) {
+          if (P.policy_mode == 1)
+            P.policy[(size_t)(P.horizon - k) * P.n_states + s] = best;
+          else if (P.policy_mode == 2)
+            P.policy[s] = best;
+          if (infinite) {
+            const uint64_t vold = __ldcg(reinterpret_cast<const unsigned long long*>(Vg) + s);
+            const uint64_t d = vnew > vold ? vnew - vold : vold - vnew;
+            dmax = d > dmax ? d : dmax;
+          }
+        }
+      }
+      if (infinite) {
+        const uint64_t m = warp_max_u64(dmax);
+        if (lane == 0) S.part[warp] = m;
+        __syncthreads();
+        if (tid == 0) {
+          unsigned long long all = 0;
+          for (int w = 0; w < kGridWarps; ++w) all = S.part[w] > all ? S.part[w] : all;
+          atomicMax(&L.ctl->resid[k & 3], all);
+        }
+      }
+    };
+    // the columns' values and hints that the misses' records hold
+    const auto collect = [&]() {
+      for (uint32_t j = tid; j < n_miss; j += kGridThreads) {
+        const GridMiss m = load_miss(mine + j);
+        GridCol& c = T.col[m.i];
+        const uint32_t lc = c.lc & ~kMoving;
+        const int32_t e = hint_entry(m.hint);
+        T.q[lc & kLocalColumn] = m.acc;
+        c.lc = m.hint <= -2 ? lc | kMoving : lc;
+        c.e = e;
+        if (e >= 0) c.hrow = copied ? XRows{D.rows + c.a * 4u}[e] : __ldg(P.rowval + c.a + e);
+      }
+      __syncthreads();
+    };
+    const uint32_t list = n_miss > kGridFewMisses ? n_miss : 0;
+    if (n_miss && !list) {
+      settle_few<f32, copied>(P, T, D, mine, n_miss, Vg, scratch, lane, S);
+      __syncthreads();
+      collect();
+    }
+    if (!list) states();
+    __syncthreads();
+    ++barrier;
+    if (tid == 0) {
+      // this CTA's misses are listed (its part of the iteration is done if there are none)
+      uint32_t* steal = R.steal + (size_t)(k & 1) * 2 * gridDim.x;
+      uint32_t* next = R.steal + (size_t)((k + 1) & 1) * 2 * gridDim.x;
+      next[blockIdx.x] = next[gridDim.x + blockIdx.x] = 0;  // last read before the previous barrier
+      if (blockIdx.x == 0) {
+        L.ctl->resid[(k + 1) & 3] = 0;
+        L.ctl->misses[(k + 1) & 3] = 0;
+      }
+      if (list) atomicAdd(&L.ctl->misses[k & 3], list);
+      steal[blockIdx.x] = list;
+      grid_arrive(L.ctl);
+    }
+    if (!settle_misses<f32, copied>(L, R, P, T, D, Vg, scratch, k, barrier * gridDim.x, list, lane, warp, S)) return -1;
+    if (S.total != 0) {
+      // every miss is settled after one more barrier; their CTAs finish, and a last one ends the iteration
+      if (!grid_sync(L.ctl, ++barrier, S)) return -1;
+      if (list) {
+        collect();
+        states();
+      }
+      if (!grid_sync(L.ctl, ++barrier, S)) return -1;
+    }
+    if (infinite && __ldcg(&L.ctl->resid[k & 3]) < P.eps_fix && !P.external_stop) break;
+    if (k == k1) break;
+  }
+  return k;
+}
+
+template <bool f32, int G>
+__global__ void __launch_bounds__(kGridThreads, 1) bellman_grid_kernel(StepLaunch L, GridPlan R, int32_t n_iters) {
+  GridShared& S = *at_shared<GridShared>(0);
+  constexpr int cell = f32 ? 4 : 8;
+  const GridLayout lay = grid_layout(R.cap_cols, R.cap_own, R.cap_cells, cell);
+  GridTable T;
+  T.col = at_shared<GridCol>((uint32_t)lay.cols);
+  T.q = at_shared<uint64_t>((uint32_t)lay.q);
+  T.st = at_shared<GridState>((uint32_t)lay.states);
+  const int tid = threadIdx.x;
+  const Problem& P = S.prob;
+  if (tid < (int)(sizeof(Problem) / 4))
+    reinterpret_cast<uint32_t*>(&S.prob)[tid] = reinterpret_cast<const uint32_t*>(L.probs)[tid];
+  IterState it = L.its[0];
+  const int32_t last = min(L.probs[0].horizon, it.iter + n_iters);
+  if (!it.done && last > it.iter) {
+    const int n_chunks = ((int)R.n_chunks - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    if (tid == 0) {
+      int32_t own = 0, cells = 0;
+      for (int j = 0; j < n_chunks; ++j) {
+        const int g = blockIdx.x + j * gridDim.x;
+        const int32_t a = R.chunk[g], b = R.chunk[g + 1];
+        S.chunk_s0[j] = a;
+        S.chunk_own[j] = own;
+        own += b - a;
+        if (R.one_window && j > 0) continue;
+        GridWindow w = R.one_window ? GridWindow{0, L.probs[0].n_states, 0} : R.win[g];
+        w.off = (int32_t)lay.v + (cells - w.w0) * cell;
+        S.win[j] = w;
+        S.win_at[j] = cells;
+        cells += w.len;
+      }
+      S.chunk_own[n_chunks] = own;
+      S.n_win = R.one_window ? min(1, n_chunks) : n_chunks;
+    }
+    __syncthreads();
+    build_grid_columns<f32, G>(P, T, n_chunks, R.max_col, S);
+    copy_grid_entries<f32>(P, T, (uint32_t)lay.data, R.smem - (uint32_t)lay.data, S);
+    const int32_t k0 = it.iter + 1;
+    int32_t k;
+    if (S.copied)
+      k = P.pessimistic ? grid_iterate<f32, G, true, true>(L, P, T, lay, R, k0, last, S)
+                        : grid_iterate<f32, G, false, true>(L, P, T, lay, R, k0, last, S);
+    else
+      k = P.pessimistic ? grid_iterate<f32, G, true, false>(L, P, T, lay, R, k0, last, S)
+                        : grid_iterate<f32, G, false, false>(L, P, T, lay, R, k0, last, S);
+    if (k >= 0) {
+      it.iter = k;
+      const bool settled =
+          P.infinite && __ldcg(&L.ctl->resid[k & 3]) < P.eps_fix && !P.external_stop;
+      if (settled || k >= P.horizon) {
+        it.done = 1;
+        it.noconv = P.infinite && !settled ? 1 : 0;
+      }
+      // hints back to the session's state
+      for (int i = tid; i < S.n_cols; i += kGridThreads) {
+        const GridCol& c = T.col[i];
+        if (c.rem == 0) continue;
+        P.hint[c.c] = c.lc & kMoving ? -2 - c.e : c.e;
+      }
+    }
+  } else {
+    it.done = 1;  // horizon 0: nothing to run
+  }
+  if (it.done) it.k_final = it.iter;
+  __syncthreads();
+  // the last CTA writes the iteration state and resets the launch's counters
+  // (every CTA has read them by then)
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(&L.ctl->finished, 1u) == gridDim.x - 1u) {
+      __threadfence();
+      it.resmax = 0;
+      L.its[0] = it;
+      L.ctl->finished = 0;
+      L.ctl->arrived = 0;
+      for (int i = 0; i < 4; ++i) {
+        L.ctl->resid[i] = 0;
+        L.ctl->misses[i] = 0;
+      }
+    }
+  }
+}
+
+typedef void (*GridKernel)(StepLaunch, GridPlan, int32_t);
+
+GridKernel grid_kernel(const GridPlan& R) {
+  if (R.f32) return R.group == 8 ? bellman_grid_kernel<true, 8> : bellman_grid_kernel<true, 32>;
+  return R.group == 8 ? bellman_grid_kernel<false, 8> : bellman_grid_kernel<false, 32>;
+}
+
+}  // namespace
+
+size_t grid_bytes(int32_t cols, int32_t own, int32_t cells, bool f32) {
+  return grid_layout(cols, own, cells, f32 ? 4 : 8).data;
+}
+
+cudaError_t grid_prepare(const GridPlan& R) {
+  cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(grid_kernel(R)),
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentSmem);
+  int n = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, grid_kernel(R), kGridThreads, R.smem);
+  return e == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : e;
+}
+
+cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t n_iters, cudaStream_t st) {
+  if (n_iters <= 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(R.steal, 0, sizeof(uint32_t) * 4 * (size_t)R.grid, st);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t c;
+  std::memset(&c, 0, sizeof(c));
+  c.gridDim = dim3((unsigned)R.grid);
+  c.blockDim = dim3(kGridThreads);
+  c.dynamicSmemBytes = R.smem;
+  c.stream = st;
+  cudaLaunchAttribute attr;  // all CTAs resident together: they wait for one another
+  attr.id = cudaLaunchAttributeCooperative;
+  attr.val.cooperative = 1;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, grid_kernel(R), L, R, n_iters);
+}
+
+}  // namespace imdp

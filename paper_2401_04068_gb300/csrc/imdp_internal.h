@@ -121,6 +121,9 @@ struct DevModel {
   // State boundaries that no transition crosses, 0 and n_states included: the
   // states between two of them are a Markov decision process of their own.
   std::vector<int32_t> h_parts;
+  // Per state: smallest and largest destination of its columns, and the largest
+  // leaving out each column's last entry (-1: none); empty for a slice.
+  std::vector<int3> h_span;
   SliceLayout* slices = nullptr;    // built on first use by a session that runs the slice kernel
   std::mutex slices_mu;
 };
@@ -176,6 +179,9 @@ struct StepControl {
   unsigned int error;      // nonzero: a bounded wait inside the kernel gave up
   unsigned int wide_next;  // next wide state to take in the running launch
   unsigned int tile_next;  // next tile to take in the running launch (direct kernel)
+  unsigned int arrived;    // grid kernel: arrivals at the running launch's barriers
+  unsigned int misses[4];       // grid kernel: columns to settle, by iteration mod 4
+  unsigned long long resid[4];  // grid kernel: max |V_k - V_{k-1}|, likewise
   int32_t tile_limit;      // 0: every tile; t + 1: only tiles [0, t) belong to running problems
 };
 
@@ -287,6 +293,46 @@ struct ResidentPlan {
   uint32_t smem;
 };
 
+// The grid kernel (grid.cu): all iterations of a step call of one large problem
+// in one cooperative launch. The states are cut into chunks dealt round-robin to
+// the CTAs; each CTA keeps, per chunk, a window of the values in shared memory
+// that holds every destination of the chunk's columns except, possibly, a
+// column's last one.
+constexpr int kGridMaxChunks = 16;  // per CTA
+// Models of this many transitions or more keep the per-iteration direct kernel:
+// there the transitions have left L2 when a missed column is settled (pimdp_2,
+// 48 M: grid kernel 53.1 ms and 42.8 ms on 32-bit storage, direct 54.8 and 40.3;
+// 29 M in two actions: 24.8 against 29.6).
+constexpr int64_t kGridMostEntries = 32000000;
+struct GridWindow {
+  int32_t w0, len;  // states [w0, w0 + len)
+  int32_t off;      // set on the device
+};
+// A column whose warm start failed, as its CTA lists it; any CTA settles it and
+// leaves the column's value in `acc` and its hint.
+struct alignas(16) GridMiss {
+  unsigned long long rem, vk, acc, flt, geq;  // rem_of, and the failed warm start's sums
+  int32_t i, c, k;                            // place in the owner's table, column, entries
+  int32_t neighbor;                           // try the neighbouring key first
+  int32_t hint;
+  int32_t pad;
+};
+struct GridPlan {
+  const int32_t* chunk;    // n_chunks + 1 state boundaries
+  const GridWindow* win;   // per chunk
+  GridMiss* misses;        // cap_cols per CTA
+  uint32_t* steal;         // by iteration parity, per CTA: misses listed, misses taken
+  int32_t n_chunks;        // 0: not taken
+  int32_t one_window;      // every CTA keeps all values (the windows' sum would be no smaller)
+  int32_t grid;            // CTAs
+  int32_t group;           // lanes to a column
+  int32_t f32;
+  int32_t single;          // every state has one action
+  int32_t cap_cols, cap_own, cap_cells;  // of one CTA
+  int32_t max_col;
+  uint32_t smem;
+};
+
 // NVTX range for the host-side phases (model upload, session steps, server
 // chunks); shows up in Nsight timelines, free when no tool is attached.
 struct TraceRange {
@@ -315,6 +361,11 @@ size_t resident_bytes(int32_t states, int32_t cols, int32_t own, bool f32, int32
 cudaError_t resident_prepare(ResidentPlan& R);
 // n_iters Bellman iterations of every unit in one launch.
 cudaError_t launch_bellman_resident(const StepLaunch& L, const ResidentPlan& R, int32_t n_iters, cudaStream_t st);
+// grid.cu
+// Shared memory of one CTA.
+size_t grid_bytes(int32_t cols, int32_t own, int32_t cells, bool f32);
+cudaError_t grid_prepare(const GridPlan& R);
+cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t n_iters, cudaStream_t st);
 // CTAs of the persistent tiled kernel: one per SM.
 int bellman_grid();
 // The configuration a launch of `L` with `cfg` (nullable) actually uses: kernel,
@@ -393,6 +444,8 @@ struct Session {
   // Step calls by rule: the resident kernel's plan (n_units 0: not taken).
   ResidentPlan resident{};
   imdp_status plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st);
+  GridPlan whole{};  // the grid kernel's (n_chunks 0: not taken)
+  imdp_status plan_grid(cudaStream_t st);
   SideStream side;  // created when the session has both tiles and wide states
   LaunchConfig cfg;  // launch configuration (rule, set_launch or the autotuner)
   StepLaunch L{};

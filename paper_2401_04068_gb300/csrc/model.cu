@@ -159,21 +159,22 @@ __global__ void select_columns_kernel(int32_t n_cols, const int32_t* __restrict_
   }
 }
 
-// Per state: the smallest and the largest state that its columns or it itself
-// name (a column's destinations ascend, so its first and last entry bound it).
+// Per state: the smallest and the largest destination of its columns, and the
+// largest one that is not its column's last (a column's destinations ascend).
 __global__ void state_span_kernel(int32_t n_states, const int32_t* __restrict__ stateptr,
                                   const int32_t* __restrict__ colptr, const int32_t* __restrict__ rowval,
-                                  int2* __restrict__ span) {
+                                  int3* __restrict__ span) {
   for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n_states; s += gridDim.x * blockDim.x) {
-    int32_t lo = s, hi = s;
+    int32_t lo = n_states, hi = -1, inner = -1;
     for (int32_t c = stateptr[s]; c < stateptr[s + 1]; ++c) {
       const int32_t a = colptr[c], b = colptr[c + 1];
       if (a < b) {
         lo = min(lo, rowval[a]);
         hi = max(hi, rowval[b - 1]);
+        if (a + 1 < b) inner = max(inner, rowval[b - 2]);
       }
     }
-    span[s] = make_int2(lo, hi);
+    span[s] = make_int3(lo, hi, inner);
   }
 }
 
@@ -367,16 +368,16 @@ imdp_status model_create_csc(int32_t n_states, int32_t n_cols, int64_t nnz, cons
   convert_columns_kernel<<<grid, 256, 0, st>>>(n_states, n_cols, m->colptr, m->rowval, lo_d, up_d, m->lg, m->rem,
                                                (unsigned*)derr.p);
   e = cudaGetLastError();
-  std::vector<int2> span;
+  std::vector<int3> span;
   DevBuf dspan;
   if (e == cudaSuccess && !is_slice(m)) {
-    if (!dspan.alloc(sizeof(int2) * n_states, st)) { model_destroy(m); set_error("allocation failed"); return IMDP_ENOMEM; }
+    if (!dspan.alloc(sizeof(int3) * n_states, st)) { model_destroy(m); set_error("allocation failed"); return IMDP_ENOMEM; }
     span.resize(n_states);
     state_span_kernel<<<std::min((n_states + 255) / 256, sms * 8), 256, 0, st>>>(n_states, m->stateptr, m->colptr,
-                                                                                m->rowval, (int2*)dspan.p);
+                                                                                m->rowval, (int3*)dspan.p);
     e = cudaGetLastError();
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(span.data(), dspan.p, sizeof(int2) * n_states, cudaMemcpyDeviceToHost, st);
+      e = cudaMemcpyAsync(span.data(), dspan.p, sizeof(int3) * n_states, cudaMemcpyDeviceToHost, st);
   }
   unsigned herr = 0;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, derr.p, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
@@ -471,14 +472,15 @@ imdp_status model_create_csc(int32_t n_states, int32_t n_cols, int64_t nnz, cons
   if (!span.empty()) {
     std::vector<int32_t> low(n_states);  // smallest state named from s on
     int32_t least = n_states;
-    for (int32_t s = n_states - 1; s >= 0; --s) low[s] = least = std::min(least, span[s].x);
+    for (int32_t s = n_states - 1; s >= 0; --s) low[s] = least = std::min({least, span[s].x, s});
     int32_t most = -1;
     for (int32_t s = 0; s + 1 < n_states; ++s) {
-      most = std::max(most, span[s].y);
+      most = std::max({most, span[s].y, s});
       if (most <= s && low[s + 1] > s) m->h_parts.push_back(s + 1);
     }
   }
   m->h_parts.push_back(n_states);
+  m->h_span = std::move(span);
   plan_tiles(m, 0, m->h_tiles, m->h_wide);
   m->n_tiles = (int32_t)m->h_tiles.size();
   for (const Tile& t : m->h_tiles) m->tile_cols += t.c1 - t.c0;

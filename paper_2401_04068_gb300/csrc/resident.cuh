@@ -127,17 +127,17 @@ struct PairOf<true> {
 };
 __device__ __forceinline__ uint2 ld_pair(const uint2* p) {
   uint2 v;
-  asm("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
   return v;
 }
 __device__ __forceinline__ ulonglong2 ld_pair(const ulonglong2* p) {
   ulonglong2 v;
-  asm("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+  asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
   return v;
 }
 __device__ __forceinline__ int32_t ld_row(const int32_t* p) {
   int32_t v;
-  asm("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  asm volatile("ld.global.nc.s32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
 __device__ __forceinline__ uint2 ld_pair_if(const uint2* p, bool ok) { return ld_stream_u32x2_if(p, ok); }
@@ -323,28 +323,256 @@ __device__ __forceinline__ void warm_columns(const Columns& C, const Entries<typ
   }
 }
 
-// A column whose warm start failed (or that had no hint): the neighbour check,
-// then the threshold search, by the whole warp (the sequence of column_q).
-// Not inlined: the search's registers stay out of the warm pass.
-template <bool f32, int gmem, class VA>
+// Loads of the passes below (a lane past the end gets destination `none` and a
+// zero pair).
+__device__ __forceinline__ int32_t settle_row(GRows rows, int i, bool ok, int32_t none) {
+  return ld_row_or(rows.p + i, ok, none);
+}
+__device__ __forceinline__ int32_t settle_row(XRows rows, int i, bool ok, int32_t none) { return ok ? rows[i] : none; }
+template <bool f32>
+__device__ __forceinline__ ulonglong2 settle_pair(const Bounds<f32, 1>& lg, int i, bool ok) {
+  return lg.at_if(i, ok);
+}
+template <bool f32>
+__device__ __forceinline__ ulonglong2 settle_pair(const Bounds<f32, 3>& lg, int i, bool ok) {
+  return ok ? lg[i] : make_ulonglong2(0, 0);
+}
+
+// A column whose warm start failed (or that had no hint), by the whole warp: the
+// neighbour check, then the threshold search (the sequence of column_q, to the
+// bit). The passes of column_neighbor and column_search load one entry a lane,
+// wait, and use it (12 round trips to L2 for 376 entries, and 6 to 12 passes);
+// here each pass has the loads of four trips in flight. The neighbour's pass
+// takes keys only (its key's entries are looked up by a second one) and leaves
+// the key range for the search. Not inlined: the search's registers stay out of
+// the warm pass. `none`: any state that V holds.
+template <bool f32, int gmem, int U, class VA>
 __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type rows, const Bounds<f32, gmem> lg,
                                                int32_t k, uint64_t rem, const VA V, bool pess, bool neighbor,
-                                               uint64_t vk, uint64_t acc, uint64_t flt, uint64_t geq, uint32_t scratch,
-                                               int lane, int32_t* hint_out) {
-  uint64_t q;
-  if (neighbor) {
-    WarmMiss w;
-    w.vk = vk;
-    w.acc = acc;
-    w.flt = f32 ? shl_sat(flt, lg.down) : flt;
-    w.geq = f32 ? shl_sat(geq, lg.down) : geq;
-    w.valid = true;
-    if (column_neighbor<f32, gmem>(rows, lg, k, rem, V, pess, lane, w, &q, hint_out)) return q;
+                                               uint64_t vk, uint64_t wacc, uint64_t flt, uint64_t geq, uint32_t scratch,
+                                               int32_t none, int lane, int32_t* hint_out) {
+  WarpScratch* ws = at_shared<WarpScratch>(scratch);
+  const auto key_of = [&](int32_t r) -> uint64_t {
+    const uint64_t v = V.at(r);
+    return pess ? v : kOne - v;
+  };
+  const auto value = [&](uint64_t x) { return pess ? x : kOne - x; };
+  // calls f(entry, key) for every entry, a lane's in ascending order
+  const auto keys = [&](const auto& f) {
+    for (int base = lane; base < k; base += 32 * U) {
+      int32_t r[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) r[u] = settle_row(rows, base + 32 * u, base + 32 * u < k, none);
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (base + 32 * u < k) f(base + 32 * u, key_of(r[u]));
+    }
+  };
+  if (f32 && neighbor) {
+    flt = shl_sat(flt, lg.down);
+    geq = shl_sat(geq, lg.down);
   }
-  int32_t found;
-  q = column_search<f32, gmem>(rows, lg, k, rem, V, pess, at_shared<WarpScratch>(scratch), lane, &found);
+  const bool down = flt >= rem;
+  const uint64_t kap = value(vk);
+  uint64_t cmin = ~0ull, cmax = 0, near = down ? 0ull : ~0ull;
+  bool have = false;
+  keys([&](int, uint64_t x) {
+    cmin = x < cmin ? x : cmin;
+    cmax = x > cmax ? x : cmax;
+    if (down ? x < kap : x > kap) {
+      near = down ? (x > near ? x : near) : (x < near ? x : near);
+      have = true;
+    }
+  });
+  if (neighbor && !(down && flt >= kOne) && __any_sync(kFull, have)) {
+    const uint64_t tgt = down ? warp_max_u64(near) : warp_min_u64(near);
+    uint64_t gs = 0, ds = 0, dk = 0;
+    int first = -1;
+    keys([&](int i, uint64_t x) {
+      if (x == tgt || (!down && x == kap)) {
+        const ulonglong2 b = lg[i];
+        const uint64_t v = value(x), d = __umul64hi(v, b.x + b.y) - __umul64hi(v, b.x);
+        if (x == tgt) {
+          gs = sat_add(gs, b.y);
+          ds += d;
+          if (first < 0) first = i;
+        } else {
+          dk += d;
+        }
+      }
+    });
+    const uint64_t G = warp_sum_sat(gs), D = warp_sum_u64(ds);
+    const int32_t h = __shfl_sync(kFull, first, __ffs(__ballot_sync(kFull, first >= 0)) - 1);
+    const uint64_t vt = value(tgt);
+    if (down) {
+      const uint64_t fl = flt - G;
+      if (fl < rem) {
+        *hint_out = h;
+        return wacc - D + __umul64hi(vt, rem - fl);
+      }
+    } else {
+      const uint64_t DK = warp_sum_u64(dk);
+      const uint64_t fl = flt + geq;
+      if (sat_add(fl, G) >= rem) {
+        *hint_out = h;
+        return wacc + DK + __umul64hi(vt, rem - fl);
+      }
+    }
+  }
+  // threshold search (column_search)
+  uint64_t lo = 0, hi = kOne, fb = 0;
+  bool all_below = false, uniform = false;
+  cmin = warp_min_u64(cmin);
+  cmax = warp_max_u64(cmax);
+  for (int round = 0; round < 12; ++round) {
+    if (cmin > cmax) {  // no entry: nothing absorbs rem
+      all_below = true;
+      break;
+    }
+    if (cmin == cmax) {  // the candidates share one key
+      lo = hi = cmin;
+      uniform = true;
+      break;
+    }
+    const int bits = 64 - __clzll((long long)(cmax - cmin));
+    const int shift = bits > 6 ? bits - 6 : 0;
+    ws->hl[lane] = 0;
+    ws->hl[lane + 32] = 0;
+    ws->hh[lane] = 0;
+    ws->hh[lane + 32] = 0;
+    ws->hc[lane] = 0;
+    ws->hc[lane + 32] = 0;
+    if (lane == 0) ws->hsat[0] = ws->hsat[1] = 0;
+    __syncwarp();
+    for (int base = lane; base < k; base += 32 * U) {
+      int32_t r[U];
+      uint64_t g[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = base + 32 * u;
+        r[u] = settle_row(rows, i, i < k, none);
+        g[u] = settle_pair(lg, i, i < k).y;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (base + 32 * u >= k) break;
+        const uint64_t x = key_of(r[u]);
+        if (x >= lo && x <= hi) {
+          const int b = (int)((x - cmin) >> shift);
+          const uint64_t gg = g[u] < rem ? g[u] : rem;
+          const unsigned gl = (unsigned)gg;
+          const unsigned old = atomicAdd(&ws->hl[b], gl);
+          const unsigned up = (unsigned)(gg >> 32) + ((old + gl) < old ? 1u : 0u);
+          if (up) {
+            const unsigned oh = atomicAdd(&ws->hh[b], up);
+            if (oh + up < oh) atomicOr(&ws->hsat[b >> 5], 1u << (b & 31));
+          }
+          atomicAdd(&ws->hc[b], 1u);
+        }
+      }
+    }
+    __syncwarp();
+    const unsigned sat = ws->hsat[lane >> 4];
+    const uint64_t h0 = ((sat >> ((2 * lane) & 31)) & 1u) ? ~0ull
+                                                          : (((uint64_t)ws->hh[2 * lane] << 32) | ws->hl[2 * lane]);
+    const uint64_t h1 = ((sat >> ((2 * lane + 1) & 31)) & 1u)
+                            ? ~0ull
+                            : (((uint64_t)ws->hh[2 * lane + 1] << 32) | ws->hl[2 * lane + 1]);
+    const uint64_t ex = warp_excl_scan_sat(sat_add(h0, h1), lane);
+    const uint64_t i0 = sat_add(sat_add(fb, ex), h0), i1 = sat_add(i0, h1);
+    const unsigned cross = __ballot_sync(kFull, i1 >= rem);
+    if (cross == 0) {  // first round only: the gaps cannot absorb rem
+      all_below = true;
+      break;
+    }
+    const int L = __ffs(cross) - 1;
+    const bool low = i0 >= rem;
+    const int b = __shfl_sync(kFull, low ? 2 * lane : 2 * lane + 1, L);
+    fb = __shfl_sync(kFull, low ? sat_add(fb, ex) : i0, L);
+    const unsigned cnt = ws->hc[b];
+    __syncwarp();
+    lo = cmin + ((uint64_t)b << shift);
+    const uint64_t top = lo + ((1ull << shift) - 1ull);
+    hi = top < cmax ? top : cmax;
+    if (cnt <= 32) break;
+    uint64_t a = ~0ull, z = 0;
+    keys([&](int, uint64_t x) {
+      if (x >= lo && x <= hi) {
+        a = x < a ? x : a;
+        z = x > z ? x : z;
+      }
+    });
+    cmin = warp_min_u64(a);
+    cmax = warp_max_u64(z);
+  }
+  uint64_t acc = 0, gsum = 0;
+  unsigned pos = 0;
+  int first_cand = -1;
+  const unsigned lt = (1u << lane) - 1u;
+  for (int base = 0; base < k; base += 32 * U) {
+    int32_t r[U];
+    ulonglong2 b[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = base + 32 * u + lane;
+      r[u] = settle_row(rows, i, i < k, none);
+      b[u] = settle_pair(lg, i, i < k);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (base + 32 * u >= k) break;
+      const int i = base + 32 * u + lane;
+      const bool valid = i < k;
+      const uint64_t x = key_of(r[u]);
+      const bool below = all_below || x < lo;
+      const bool cand = valid && !all_below && x >= lo && x <= hi;
+      acc = mul_hi_add(value(x), below ? b[u].x + b[u].y : b[u].x, acc);  // past the end: a zero pair
+      const unsigned m = __ballot_sync(kFull, cand);
+      if (m && first_cand < 0) first_cand = base + 32 * u + __ffs(m) - 1;
+      if (!uniform) {
+        if (cand) {
+          const unsigned at = min(pos + __popc(m & lt), 31u);
+          ws->ck[at] = x;
+          ws->cg[at] = b[u].y < rem ? b[u].y : rem;
+          ws->ci[at] = i;
+        }
+        pos += __popc(m);
+      } else if (cand) {
+        gsum = sat_add(gsum, b[u].y < rem ? b[u].y : rem);
+      }
+    }
+  }
+  acc = warp_sum_u64(acc);
+  if (all_below) {
+    *hint_out = -1;
+    return acc;
+  }
+  pos = min(pos, 32u);
+  const uint64_t r2 = rem - fb;  // > 0 by construction of the crossing bin
+  if (uniform) {
+    const uint64_t g = warp_sum_sat(gsum);
+    *hint_out = first_cand >= 0 ? -2 - first_cand : -1;
+    return acc + __umul64hi(value(lo), g < r2 ? g : r2);
+  }
+  __syncwarp();
+  uint64_t extra = 0;
+  int thr = -1;
+  if (lane < (int)pos) {
+    const uint64_t ki = ws->ck[lane], gi = ws->cg[lane];
+    uint64_t before = 0;
+    for (unsigned j = 0; j < pos; ++j) {
+      const uint64_t kj = ws->ck[j];
+      if (kj < ki || (kj == ki && j < (unsigned)lane)) before = sat_add(before, ws->cg[j]);
+    }
+    const uint64_t left = r2 > before ? r2 - before : 0;
+    extra = __umul64hi(value(ki), gi < left ? gi : left);
+    if (left > 0 && left <= gi) thr = ws->ci[lane];
+  }
+  const unsigned tm = __ballot_sync(kFull, thr >= 0);
+  const int32_t found = tm ? __shfl_sync(kFull, thr, __ffs(tm) - 1) : -1;
   *hint_out = found >= 0 ? -2 - found : -1;
-  return q;
+  __syncwarp();
+  return acc + warp_sum_u64(extra);
 }
 
 // The CTA's copy of its columns' entries in shared memory (offsets): rows and
@@ -354,6 +582,7 @@ struct EntryCopy {
   uint32_t rows, pairs, exact;
 };
 
+constexpr int kUnitTrips = 2;  // trips in flight while the resident kernel settles a column
 // Column i of the table after a failed warm start: its value and hint.
 template <bool f32, bool shared, class VA>
 __device__ __forceinline__ void settle_column(const Problem& P, const Columns& C, const EntryCopy& D, int i, int n32,
@@ -361,24 +590,25 @@ __device__ __forceinline__ void settle_column(const Problem& P, const Columns& C
   const Col c = C.col[i];
   const uint64_t vk = V.at(c.hrow);
   const bool pess = P.pessimistic != 0, neighbor = c.e >= 0 && !(c.lc & kMoving);
+  const int32_t none = shared ? 0 : V.base;
   int32_t ho;
   uint64_t q;
   if constexpr (shared) {
     const XRows rows{D.rows + c.a * 4u};
     if (f32 && i < n32)
-      q = missed_column<true, 3>(rows, Bounds<true, 3>{D.pairs + c.a * 8u, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk,
-                                 c.acc, c.flt, c.geq, scratch, lane, &ho);
+      q = missed_column<true, 3, kUnitTrips>(rows, Bounds<true, 3>{D.pairs + c.a * 8u, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk,
+                                 c.acc, c.flt, c.geq, scratch, none, lane, &ho);
     else
-      q = missed_column<false, 3>(rows, Bounds<false, 3>{(f32 ? D.exact : D.pairs) + c.a * 16u, 0}, c.k, c.rem, V, pess,
-                                  neighbor, vk, c.acc, c.flt, c.geq, scratch, lane, &ho);
+      q = missed_column<false, 3, kUnitTrips>(rows, Bounds<false, 3>{(f32 ? D.exact : D.pairs) + c.a * 16u, 0}, c.k, c.rem, V, pess,
+                                  neighbor, vk, c.acc, c.flt, c.geq, scratch, none, lane, &ho);
   } else {
     const GRows rows{P.rowval + c.a};
     if (f32 && i < n32)
-      q = missed_column<true, 1>(rows, Bounds<true, 1>{P.lg32 + c.a, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk, c.acc,
-                                 c.flt, c.geq, scratch, lane, &ho);
+      q = missed_column<true, 1, kUnitTrips>(rows, Bounds<true, 1>{P.lg32 + c.a, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk, c.acc,
+                                 c.flt, c.geq, scratch, none, lane, &ho);
     else
-      q = missed_column<false, 1>(rows, Bounds<false, 1>{f32 ? P.lgx + c.x : P.lg + c.a, 0}, c.k, c.rem, V, pess,
-                                  neighbor, vk, c.acc, c.flt, c.geq, scratch, lane, &ho);
+      q = missed_column<false, 1, kUnitTrips>(rows, Bounds<false, 1>{f32 ? P.lgx + c.x : P.lg + c.a, 0}, c.k, c.rem, V, pess,
+                                  neighbor, vk, c.acc, c.flt, c.geq, scratch, none, lane, &ho);
   }
   if (lane == 0) {
     const uint32_t lc = c.lc & ~kMoving;

@@ -294,6 +294,7 @@ imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<
   }
   S->grid = bellman_grid();
   imdp_status r = S->plan_resident(specs, st);
+  if (r == IMDP_OK) r = S->plan_grid(st);
   if (r != IMDP_OK) { delete S; return r; }
   const bool slice = resolve_launch(S->L, &S->cfg).kernel == kKernelSlice;
   r = slice ? S->prepare_slices(st) : IMDP_OK;
@@ -378,10 +379,13 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
   // in L2 (4096 parts of 0.3 MB on 32-bit storage: 68 ms against 74 with one).
   const bool two = n_units * (int64_t)c >= 2 * grid && unit_bytes * (2 * grid / c) <= 100e6;
   resident.threads = two ? kResidentThreads / 2 : kResidentThreads;
-  // Against the per-iteration launches: those take about 10 us and stream 0.64
-  // transitions a cycle and SM, this kernel about 3 us and 1.17 on the SMs it covers.
-  const double sms = std::min<double>(grid, (double)n_units * c), hz = 1.9e9;
-  if (3e-6 + (double)entries / (1.17 * sms * hz) > 10e-6 + (double)entries / (0.64 * grid * hz)) return IMDP_OK;
+  // Seconds an iteration takes: per-iteration launches about 10 us and 0.64
+  // transitions a cycle and SM, this kernel about 3 us and 1.17 on the SMs it
+  // covers, the grid kernel (one problem only) about 6.5 us and 1 on all.
+  const double sms = std::min<double>(grid, (double)n_units * c), hz = 1.9e9, e = (double)entries;
+  double other = 10e-6 + e / (0.64 * grid * hz);
+  if (count == 1 && n_units == 1) other = std::min(other, 6.5e-6 + e / (1.0 * grid * hz));
+  if (3e-6 + e / (1.17 * sms * hz) > other) return IMDP_OK;
   // ranks of a unit: contiguous states of about equal work
   std::vector<int32_t> bounds;
   int64_t rank_entries = 0;
@@ -436,8 +440,8 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
   resident.cap_states = states;
   resident.max_col = max_col;
   resident.n_units = n_units;
-  cudaError_t e = resident_prepare(resident);
-  if (e != cudaSuccess) {  // clusters this wide do not fit the device: the per-iteration kernels run
+  cudaError_t err = resident_prepare(resident);
+  if (err != cudaSuccess) {  // clusters this wide do not fit the device: the per-iteration kernels run
     cudaGetLastError();
     resident.n_units = 0;
     return IMDP_OK;
@@ -451,12 +455,108 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
     set_error("device allocation failed (session)");
     return IMDP_ENOMEM;
   }
-  e = cudaMemcpyAsync(du, uh.data(), sizeof(ResidentUnit) * uh.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(db, bounds.data(), sizeof(int32_t) * bounds.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host vectors go out of scope
-  if (e != cudaSuccess) return cuda_status(e, "session plan");
+  err = cudaMemcpyAsync(du, uh.data(), sizeof(ResidentUnit) * uh.size(), cudaMemcpyHostToDevice, st);
+  if (err == cudaSuccess) err = cudaMemcpyAsync(db, bounds.data(), sizeof(int32_t) * bounds.size(), cudaMemcpyHostToDevice, st);
+  if (err == cudaSuccess) err = cudaStreamSynchronize(st);  // the host vectors go out of scope
+  if (err != cudaSuccess) return cuda_status(err, "session plan");
   resident.units = du;
   resident.bounds = db;
+  return IMDP_OK;
+}
+
+imdp_status Session::plan_grid(cudaStream_t st) {
+  whole = GridPlan{};
+  const DevModel* m = models[0];
+  if (L.tiny_ok || resident.n_units > 0 || count != 1 || m->h_span.empty() || m->nnz >= kGridMostEntries) return IMDP_OK;
+  const bool f32 = m->lg32 != nullptr;
+  const int32_t n = m->n_states;
+  const int32_t* sp = m->h_stateptr.data();
+  const int32_t* cp = m->h_colptr.data();
+  const uint8_t* fx = fixed_h.data();
+  auto cost = [&](int32_t s) -> int64_t { return fx[s] ? 1 : cp[sp[s + 1]] - cp[sp[s]] + 24 * (sp[s + 1] - sp[s]); };
+  int64_t total = 0;
+  for (int32_t s = 0; s < n; ++s) total += cost(s);
+  // Chunks per CTA: more of them spread the regions where thresholds move (40,000
+  // states of 2 actions, 160 MB: 6.8 ms with 8, 5.4 with 16), but each has its own
+  // window to load (20,000 states of 40 entries: 1.6 ms with 8, 1.9 with 16): one
+  // for every 24 columns, and at most 96 KB of windows.
+  int per = (int)std::min<int64_t>(kGridMaxChunks, std::max<int64_t>(1, m->n_cols / (24 * (int64_t)grid)));
+  std::vector<int32_t> chunk;
+  std::vector<GridWindow> win;
+  std::vector<int64_t> cells, cols, own, ent;
+  int64_t cap_cells = 0;
+  int32_t nc = 0;
+  for (;; per = (per + 1) / 2) {
+    nc = per * grid;
+    chunk.assign(nc + 1, 0);
+    win.assign(nc, GridWindow{});
+    cells.assign(grid, 0);
+    cols.assign(grid, 0);
+    own.assign(grid, 0);
+    ent.assign(grid, 0);
+    int64_t done = 0;
+    int32_t s = 0;
+    for (int32_t g = 0; g < nc; ++g) {
+      // states of about equal work, and their window: all their destinations, or
+      // all but the columns' last ones when those alone would stretch it
+      const int c = g % grid;
+      int32_t lo = n, hi = -1, inner = -1;
+      for (; s < n && (g == nc - 1 || done * nc < total * (g + 1)); ++s) {
+        done += cost(s);
+        lo = std::min(lo, m->h_span[s].x);
+        hi = std::max(hi, m->h_span[s].y);
+        inner = std::max(inner, m->h_span[s].z);
+        if (fx[s]) continue;
+        cols[c] += sp[s + 1] - sp[s];
+        own[c] += 1;
+        ent[c] += cp[sp[s + 1]] - cp[sp[s]];
+      }
+      chunk[g + 1] = s;
+      if (hi < 0) lo = hi = 0;
+      inner = std::max(inner, lo);
+      const int64_t all = (int64_t)hi - lo + 1, most = (int64_t)inner - lo + 1;
+      win[g] = GridWindow{lo, (int32_t)(all > 2 * most + 64 ? most : all), 0};
+      cells[c] += win[g].len;
+    }
+    cap_cells = *std::max_element(cells.begin(), cells.end());
+    if (per == 1 || cap_cells * (f32 ? 4 : 8) <= 96 * 1024 || cap_cells >= n) break;
+  }
+  whole.one_window = cap_cells >= n ? 1 : 0;
+  cap_cells = std::min<int64_t>(cap_cells, n);
+  const int64_t cap_cols = *std::max_element(cols.begin(), cols.end());
+  const int64_t cap_own = *std::max_element(own.begin(), own.end());
+  if (cap_cells > 60000 || cap_cols > 5000 || cap_own > 60000) return IMDP_OK;
+  const size_t need = grid_bytes((int32_t)cap_cols, (int32_t)cap_own, (int32_t)cap_cells, f32);
+  if (need > kResidentSmem) return IMDP_OK;
+  const size_t all = need + 64 + 20 * (size_t)*std::max_element(ent.begin(), ent.end());
+  whole.smem = (uint32_t)(all <= kResidentSmem ? all : need);
+  whole.cap_cols = (int32_t)cap_cols;
+  whole.cap_own = (int32_t)cap_own;
+  whole.cap_cells = (int32_t)cap_cells;
+  whole.grid = grid;
+  whole.group = m->nnz >= 256 * (int64_t)m->n_cols || m->n_cols < 48 * (int64_t)grid ? 32 : 8;
+  whole.f32 = f32 ? 1 : 0;
+  whole.single = m->n_cols == n ? 1 : 0;
+  whole.max_col = m->max_col;
+  if (grid_prepare(whole) != cudaSuccess) {
+    cudaGetLastError();
+    return IMDP_OK;
+  }
+  int32_t* dc = alloc<int32_t>(chunk.size());
+  GridWindow* dw = alloc<GridWindow>(win.size());
+  whole.misses = alloc<GridMiss>((size_t)grid * cap_cols);
+  whole.steal = alloc<uint32_t>(4 * (size_t)grid);
+  if (!dc || !dw || !whole.misses || !whole.steal) {
+    set_error("device allocation failed (session)");
+    return IMDP_ENOMEM;
+  }
+  cudaError_t e = cudaMemcpyAsync(dc, chunk.data(), sizeof(int32_t) * chunk.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(dw, win.data(), sizeof(GridWindow) * win.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host vectors go out of scope
+  if (e != cudaSuccess) return cuda_status(e, "session plan");
+  whole.chunk = dc;
+  whole.win = dw;
+  whole.n_chunks = nc;
   return IMDP_OK;
 }
 
@@ -672,8 +772,16 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
     return IMDP_OK;
   }
   if (cfg.kernel == kKernelRule && resident.n_units > 0 && n >= kResidentSteps) {
-    // by rule: all n iterations in one launch of the resident kernel
+    // by rule: all n iterations in one launch of the resident kernel,
     e = launch_bellman_resident(L, resident, n, st);
+    if (e != cudaSuccess) return cuda_status(e, "bellman step");
+    launches += n;
+    launched_since_reset += n;
+    return IMDP_OK;
+  }
+  if (cfg.kernel == kKernelRule && whole.n_chunks > 0 && n >= kResidentSteps) {
+    // or of the grid kernel
+    e = launch_bellman_grid(L, whole, n, st);
     if (e != cudaSuccess) return cuda_status(e, "bellman step");
     launches += n;
     launched_since_reset += n;

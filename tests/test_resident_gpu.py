@@ -1,6 +1,6 @@
-"""The resident kernel (by rule, several iterations in one launch) against the
-per-iteration ring kernel: the same words, iteration counts, residuals and
-policies, at the sizes where its tiling can go wrong."""
+"""The resident and grid kernels (by rule, several iterations in one launch)
+against the per-iteration ring kernel: the same words, iteration counts,
+residuals and policies, at the sizes where their tiling can go wrong."""
 import numpy as np
 import pytest
 
@@ -127,3 +127,43 @@ def test_batch_of_uneven_problems():
     _same(_run(models, ms, specs, g.KERNEL_RING), _run(models, ms, specs, g.KERNEL_RULE))
     for x in models:
         x.close()
+
+
+# one problem of the whole GPU: windows with a far last destination (the sink) or
+# the whole state space, columns around the lane groups and beyond one tile,
+# many misses at once (listed for all CTAs), entries copied to shared memory or not
+GRID = {
+    "sink": lambda: banded_imdp(6000, 3, 6000 * 3 * 41 + 6000 * 3 + 1, eps=0.1, seed=11),
+    "long_sink": lambda: banded_imdp(5000, 1, 5000 * 390 + 5000 + 1, eps=0.1, seed=12),
+    "scattered": lambda: _lengths(3001, (60, 61, 190, 256, 257, 31), 13),
+    "wide": lambda: _lengths(2100, (1279, 1280, 1281, 40, 1900), 14),
+    "loose": lambda: _lengths(2500, (90, 200, 33), 15, wide=True),
+}
+
+
+@pytest.mark.parametrize("shape", sorted(GRID))
+@pytest.mark.parametrize("case", ["reach", "optimistic_avoid", "reward", "infinite", "f32", "f32_exact"])
+def test_one_large_problem(shape, case):
+    m = GRID[shape]()
+    if case.startswith("f32"):
+        model = g.create_model(m, dtype=g.IMDP_F32, budget=1.0 if case == "f32" else 2e-9)
+    else:
+        model = g.create_model(m)
+    kw = dict(horizon=18, reach=m.goal)
+    if case == "optimistic_avoid":
+        kw.update(property=g.IMDP_REACH_AVOID, avoid=np.setdiff1d(np.arange(0, m.n_states, 17), m.goal),
+                  pessimistic=False, maximize=False)
+    elif case == "reward":
+        r = np.random.default_rng(3).uniform(-1, 1, m.n_states)
+        kw = dict(property=g.IMDP_REWARD, horizon=18, reward=r, discount=0.95)
+    elif case == "infinite":
+        kw = dict(infinite_time=True, eps=1e-4, horizon=60, reach=m.goal)
+    spec = [g.make_spec(**kw)]
+    policy = case in ("reach", "reward")
+    ref = _run([model], [m], spec, g.KERNEL_RING, policy=policy)
+    _same(ref, _run([model], [m], spec, g.KERNEL_RULE, policy=policy))
+    if case == "reach":
+        _same(ref, _run([model], [m], spec, g.KERNEL_RULE, steps=(5, 2, 4, 20), policy=True))
+        _, oV, _, _, _ = run_oracle(m, **kw)
+        assert float(np.max(np.abs(ref[0][0].astype(np.float64) / 2.0 ** 63 - oV))) <= TOL_F64
+    model.close()
