@@ -307,16 +307,9 @@ imdp_status imdp_value_iteration_batch(imdp_model* const* models, const imdp_spe
   imdp_status s = Session::create(ms, sp, nullptr, st, &S);
   if (s != IMDP_OK) return s;
   s = S->run(32, st);
-  imdp_status worst = s;
-  for (int32_t i = 0; i < count && s == IMDP_OK; ++i) {
-    int32_t k = 0;
-    imdp_status r = S->read(i, V_out[i], &k, nullptr, nullptr, st);
-    if (r != IMDP_OK && r != IMDP_ENOCONV) { worst = r; break; }
-    if (r == IMDP_ENOCONV) worst = r;
-    if (k_out) k_out[i] = k;
-  }
+  if (s == IMDP_OK) s = S->read_all(V_out, k_out, st);
   delete S;
-  return worst;
+  return s;
 }
 
 imdp_status imdp_session_create(imdp_model* const* models, const imdp_spec* specs, int32_t count,

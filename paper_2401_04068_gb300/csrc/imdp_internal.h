@@ -455,6 +455,10 @@ struct Session {
   int64_t launches = 0;
   int64_t launched_since_reset = 0;
   std::vector<void*> allocs;
+  // small buffers lie behind one another in slabs (among `allocs`): most of a
+  // small query's creation and destruction was a driver call per buffer
+  unsigned char* slab = nullptr;
+  size_t slab_left = 0;
 
   ~Session();
   template <class T> T* alloc(size_t n);
@@ -476,6 +480,9 @@ struct Session {
   imdp_status run(int32_t check_every, cudaStream_t st);
   imdp_status read_states(std::vector<IterState>& out, cudaStream_t st);
   imdp_status read(int32_t p, double* V_out, int32_t* k_out, double* res_out, int32_t* pol_out, cudaStream_t st);
+  // The values and iteration counts of every problem: one look at the iteration
+  // states and one launch for all of them. Returns the worst status.
+  imdp_status read_all(double* const* V_out, int32_t* k_out, cudaStream_t st);
 };
 imdp_status check_spec(const DevModel* m, const imdp_spec* sp);
 // Affine map V = lo + D W of a reward problem (rewards r, discount g, horizon K).

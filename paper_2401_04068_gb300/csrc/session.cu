@@ -52,6 +52,25 @@ uint64_t eps_to_fixed(double eps) {
 
 constexpr int kGraphChunk = 16;
 
+// Device buffers of up to kSlabMost bytes share allocations of kSlab bytes.
+constexpr size_t kSlab = 256 * 1024, kSlabMost = 32 * 1024;
+
+// One problem's values in read_all: its words, and where they go.
+struct ExportItem {
+  const uint64_t* V;
+  double* out;
+  double offset, scale;
+  int32_t n;
+};
+
+// The values of many problems, a row of blocks for each.
+__global__ void export_batch_kernel(const ExportItem* __restrict__ items) {
+  const ExportItem it = items[blockIdx.y];
+  const double scale = it.scale / 9223372036854775808.0;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < it.n; i += gridDim.x * blockDim.x)
+    it.out[i] = it.offset + (double)it.V[i] * scale;
+}
+
 }  // namespace
 
 // Affine map of a reward problem into [0, 1] (V = lo + D W). Rewards r, discount
@@ -114,13 +133,23 @@ Session::~Session() {
 
 template <class T>
 T* Session::alloc(size_t n) {
-  void* p = nullptr;
-  if (cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T)) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
+  const size_t bytes = (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~size_t(255);
+  const bool small = bytes <= kSlabMost;
+  if (!small || bytes > slab_left) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, small ? kSlab : bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    allocs.push_back(p);
+    if (!small) return (T*)p;
+    slab = (unsigned char*)p;
+    slab_left = kSlab;
   }
-  allocs.push_back(p);
-  return (T*)p;
+  T* t = (T*)slab;
+  slab += bytes;
+  slab_left -= bytes;
+  return t;
 }
 
 imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<const imdp_spec*>& specs,
@@ -563,8 +592,9 @@ imdp_status Session::plan_grid(cudaStream_t st) {
 imdp_status Session::install_plan(const std::vector<Tile>& tl, const std::vector<int2>& wl, cudaStream_t st,
                                   bool slice) {
   auto release = [&](void* p) {
-    if (!p) return;
-    allocs.erase(std::remove(allocs.begin(), allocs.end(), p), allocs.end());
+    const auto it = std::find(allocs.begin(), allocs.end(), p);
+    if (!p || it == allocs.end()) return;  // (part of a slab: freed with the session)
+    allocs.erase(it);
     cudaFree(p);
   };
   cudaError_t e = cudaStreamSynchronize(st);  // launches in flight may still read the old plan
@@ -771,17 +801,18 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
     launched_since_reset += n;
     return IMDP_OK;
   }
-  if (cfg.kernel == kKernelRule && resident.n_units > 0 && n >= kResidentSteps) {
-    // by rule: all n iterations in one launch of the resident kernel,
-    e = launch_bellman_resident(L, resident, n, st);
-    if (e != cudaSuccess) return cuda_status(e, "bellman step");
-    launches += n;
-    launched_since_reset += n;
-    return IMDP_OK;
-  }
-  if (cfg.kernel == kKernelRule && whole.n_chunks > 0 && n >= kResidentSteps) {
-    // or of the grid kernel
-    e = launch_bellman_grid(L, whole, n, st);
+  if (cfg.kernel == kKernelRule && n >= kResidentSteps && (resident.n_units > 0 || whole.n_chunks > 0)) {
+    // by rule: all n iterations in one launch of the resident or the grid kernel,
+    // or in several of about half a second, so that a long call does not hold the
+    // SMs that another stream's grid kernel waits for
+    int64_t entries = 0;
+    for (const DevModel* m : models) entries += m->nnz;
+    const int32_t most = (int32_t)std::min<int64_t>(50000, 64 + 100000000000ll / std::max<int64_t>(entries, 1));
+    for (int32_t done = 0; done < n && e == cudaSuccess;) {
+      const int32_t some = std::min(most, n - done);
+      e = resident.n_units > 0 ? launch_bellman_resident(L, resident, some, st) : launch_bellman_grid(L, whole, some, st);
+      done += some;
+    }
     if (e != cudaSuccess) return cuda_status(e, "bellman step");
     launches += n;
     launched_since_reset += n;
@@ -905,6 +936,71 @@ imdp_status Session::read(int32_t p, double* V_out, int32_t* k_out, double* res_
     return IMDP_ENOCONV;
   }
   return IMDP_OK;
+}
+
+imdp_status Session::read_all(double* const* V_out, int32_t* k_out, cudaStream_t st) {
+  std::vector<IterState> s;
+  imdp_status r = read_states(s, st);
+  if (r != IMDP_OK) return r;
+  // host outputs pass through one device buffer and one host buffer
+  std::vector<int64_t> staged(count, -1);
+  std::vector<std::pair<uintptr_t, uintptr_t>> spans;
+  int64_t host = 0;
+  int32_t most = 1;
+  for (int p = 0; p < count; ++p) {
+    const int32_t n = probs_h[p].n_states;
+    most = std::max(most, n);
+    spans.emplace_back((uintptr_t)V_out[p], (uintptr_t)(V_out[p] + n));
+    if (!is_device_pointer(V_out[p])) {
+      staged[p] = host;
+      host += n;
+    }
+  }
+  std::sort(spans.begin(), spans.end());
+  bool apart = count <= 65535;  // (the launch's limit)
+  for (int p = 1; p < count; ++p) apart = apart && spans[p].first >= spans[p - 1].second;
+  if (!apart) {  // outputs that overlap are written one problem after the other
+    imdp_status worst = IMDP_OK;
+    for (int p = 0; p < count; ++p) {
+      int32_t k = 0;
+      r = read(p, V_out[p], &k, nullptr, nullptr, st);
+      if (r != IMDP_OK && r != IMDP_ENOCONV) return r;
+      if (r != IMDP_OK) worst = r;
+      if (k_out) k_out[p] = k;
+    }
+    return worst;
+  }
+  std::vector<ExportItem> items(count);
+  ExportItem* d_items = nullptr;
+  double* stage = nullptr;
+  cudaError_t e = cudaMalloc(&d_items, sizeof(ExportItem) * count);
+  if (e == cudaSuccess && host > 0) e = cudaMalloc(&stage, sizeof(double) * host);
+  for (int p = 0; p < count; ++p) {
+    const Problem& P = probs_h[p];
+    const int32_t k = s[p].done ? s[p].k_final : s[p].iter;
+    items[p] = ExportItem{P.V[k & 1], staged[p] >= 0 ? stage + staged[p] : V_out[p], v_offset[p], v_scale[p], P.n_states};
+  }
+  std::vector<double> back((size_t)host);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(d_items, items.data(), sizeof(ExportItem) * count, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    export_batch_kernel<<<dim3((unsigned)std::min((most + 255) / 256, 64), (unsigned)count), 256, 0, st>>>(d_items);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess && host > 0)
+    e = cudaMemcpyAsync(back.data(), stage, sizeof(double) * host, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  cudaFree(d_items);
+  cudaFree(stage);
+  if (e != cudaSuccess) return cuda_status(e, "session read");
+  imdp_status worst = IMDP_OK;
+  for (int p = 0; p < count; ++p) {
+    if (staged[p] >= 0) std::memcpy(V_out[p], back.data() + staged[p], sizeof(double) * probs_h[p].n_states);
+    if (k_out) k_out[p] = s[p].done ? s[p].k_final : s[p].iter;
+    if (s[p].noconv) worst = IMDP_ENOCONV;
+  }
+  if (worst == IMDP_ENOCONV) set_error("infinite horizon did not converge within the iteration cap");
+  return worst;
 }
 
 }  // namespace imdp
