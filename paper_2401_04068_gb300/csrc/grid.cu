@@ -63,6 +63,7 @@ struct GridState {
 
 struct GridShared {
   Problem prob;
+  GridUnit unit;  // the problem in progress and its CTAs
   uint32_t hist[kGridBuckets];
   uint32_t next[2];  // columns taken: 32-bit ones (or all), correction columns
   unsigned long long part[kGridWarps];
@@ -71,25 +72,29 @@ struct GridShared {
   int32_t copied;
   EntryCopy copy;
   int32_t ok;
+  uint32_t states, v;                  // the unit's layout
   uint32_t n_miss, taken, total;  // the CTA's misses, those taken; all that were listed
   int32_t chunk_s0[kGridMaxChunks], chunk_own[kGridMaxChunks + 1];
   GridWindow win[kGridMaxChunks];  // `off`: byte offset of state 0's (virtual) cell
   int32_t win_at[kGridMaxChunks + 1];  // cells before the window
 };
 
+// Shared memory: what every unit has at the same place (the CTA's state, the
+// warps' scratch, the columns' first word; the columns' values backwards from the
+// end) needs no register in the column loop. Between them the states, the
+// windows, and the entries where they fit.
+__host__ __device__ constexpr size_t grid_align(size_t x) { return (x + 15) & ~size_t(15); }
+constexpr uint32_t kGridScratchAt = (uint32_t)grid_align(sizeof(GridShared));
+constexpr uint32_t kGridColumnsAt = (uint32_t)grid_align(kGridScratchAt + kGridWarps * sizeof(WarpScratch));
 struct GridLayout {
-  size_t cols, q, states, v, ws, data;
+  uint32_t states, v, data, q;  // `q`: bytes at the end
 };
 __host__ __device__ inline GridLayout grid_layout(int32_t cols, int32_t own, int32_t cells, int cell) {
-  auto up = [](size_t x) { return (x + 15) & ~size_t(15); };
   GridLayout l;
-  size_t o = up(sizeof(GridShared));
-  l.cols = o; o = up(o + (size_t)cols * sizeof(GridCol));
-  l.q = o;    o = up(o + (size_t)cols * sizeof(uint64_t));
-  l.states = o; o = up(o + (size_t)own * sizeof(GridState));
-  l.v = o;    o = up(o + (size_t)cells * cell);
-  l.ws = o;   o = up(o + kGridWarps * sizeof(WarpScratch));
-  l.data = o;
+  l.states = (uint32_t)grid_align(kGridColumnsAt + (size_t)cols * sizeof(GridCol));
+  l.v = (uint32_t)grid_align(l.states + (size_t)own * sizeof(GridState));
+  l.data = (uint32_t)grid_align(l.v + (size_t)cells * cell);
+  l.q = (uint32_t)grid_align((size_t)cols * sizeof(uint64_t));
   return l;
 }
 
@@ -134,7 +139,7 @@ struct CoherentV {
   __device__ __forceinline__ uint32_t hi(int32_t r) const { return (uint32_t)(at(r) >> 32); }
 };
 
-// Barrier `n` (1, 2, ...) of the launch's CTAs: writes before it are visible
+// Barrier `n` (1, 2, ...) of the unit's CTAs: writes before it are visible
 // after it (read values written by other CTAs past L1). False when the wait
 // gave up or another CTA did.
 // Split in two: arrive (writes of the CTA before it), wait.
@@ -157,7 +162,7 @@ __device__ __forceinline__ bool grid_waiting(StepControl* ctl, long long t0) {
 __device__ __forceinline__ bool grid_sync(StepControl* ctl, uint32_t n, GridShared& S) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    const uint32_t target = n * gridDim.x;
+    const uint32_t target = n * (uint32_t)S.unit.ctas;
     grid_arrive(ctl);
     const long long t0 = clock64();
     int ok = 1;
@@ -174,13 +179,19 @@ __device__ __forceinline__ bool grid_sync(StepControl* ctl, uint32_t n, GridShar
 }
 
 struct GridTable {
-  GridCol* col;
-  uint64_t* q;
-  GridState* st;
+  uint32_t end;  // of shared memory
+  __device__ __forceinline__ GridCol& col(int i) const { return at_shared<GridCol>(kGridColumnsAt)[i]; }
+  __device__ __forceinline__ uint64_t& q(int lc) const { return *at_shared<uint64_t>(end - 8u - 8u * (uint32_t)lc); }
 };
 
+// This CTA's place among the unit's, and its part of the miss list.
+__device__ __forceinline__ int unit_rank(const GridShared& S) { return (int)blockIdx.x - S.unit.first; }
+__device__ __forceinline__ GridMiss* unit_misses(const GridShared& S) {
+  return S.unit.misses + (size_t)unit_rank(S) * S.unit.most_cols;
+}
+
 template <bool f32, int G>
-__device__ void build_grid_columns(const Problem& P, const GridTable& T, int n_chunks, int32_t max_col,
+__device__ void build_grid_columns(const Problem& P, const GridTable& T, GridState* st, int n_chunks, int32_t max_col,
                                    GridShared& S) {
   const int tid = threadIdx.x;
   const int32_t unit = max((max_col + 126 * G) / (127 * G), 1) * G;  // entries per length class
@@ -204,7 +215,7 @@ __device__ void build_grid_columns(const Problem& P, const GridTable& T, int n_c
     const int32_t jb = P.stateptr[s], je = P.stateptr[s + 1];
     const int at = (int)atomicAdd(&S.n_free, 1u);
     const int32_t lc = (int32_t)atomicAdd(&S.n_lc, (uint32_t)(je - jb));
-    T.st[at] = GridState{s, lc, lc + (je - jb)};
+    st[at] = GridState{s, lc, lc + (je - jb)};
     for (int32_t c = jb; c < je; ++c) atomicAdd(&S.hist[bucket(c, P.colptr[c + 1] - P.colptr[c])], 1u);
   }
   __syncthreads();
@@ -235,7 +246,7 @@ __device__ void build_grid_columns(const Problem& P, const GridTable& T, int n_c
   __syncthreads();
   if (tid == 0) S.n_own = (int32_t)S.n_free;
   for (int t = tid; t < (int)S.n_free; t += kGridThreads) {
-    const GridState g = T.st[t];
+    const GridState g = st[t];
     const int32_t s = g.s;
     int j = 0;
     while (j + 1 < n_chunks && !(s >= S.chunk_s0[j] && s - S.chunk_s0[j] < S.chunk_own[j + 1] - S.chunk_own[j])) ++j;
@@ -263,7 +274,7 @@ __device__ void build_grid_columns(const Problem& P, const GridTable& T, int n_c
       col.win = w;
       col.c = c;
       col.last = last >= w1 ? last : -1;
-      T.col[at] = col;
+      T.col(at) = col;
     }
   }
   __syncthreads();
@@ -279,14 +290,14 @@ __device__ void copy_grid_entries(const Problem& P, const GridTable& T, uint32_t
     uint32_t at = 0, e32 = 0;
     for (int base = 0; base < n_cols; base += 32) {
       const int i = base + lane;
-      const uint32_t k = i < n_cols ? (uint32_t)T.col[i].k : 0u;
+      const uint32_t k = i < n_cols ? (uint32_t)T.col(i).k : 0u;
       uint32_t incl = k;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(kFull, incl, o);
         if (lane >= o) incl += y;
       }
-      if (i < n_cols) T.q[i] = at + incl - k;
+      if (i < n_cols) T.q(i) = at + incl - k;
       const uint32_t sum = __shfl_sync(kFull, incl, 31);
       if (base < n32) e32 = at + __shfl_sync(kFull, incl, min(n32 - base, 32) - 1);
       at += sum;
@@ -305,8 +316,8 @@ __device__ void copy_grid_entries(const Problem& P, const GridTable& T, uint32_t
   if (!S.copied) return;
   const EntryCopy D = S.copy;
   for (int i = warp; i < n_cols; i += kGridWarps) {
-    const int32_t a = T.col[i].a, k = T.col[i].k, x = T.col[i].x;
-    const uint32_t at = (uint32_t)T.q[i];
+    const int32_t a = T.col(i).a, k = T.col(i).k, x = T.col(i).x;
+    const uint32_t at = (uint32_t)T.q(i);
     for (int32_t t = lane; t < k; t += 32) {
       at_shared<int32_t>(D.rows)[at + t] = P.rowval[a + t];
       if (!f32)
@@ -318,7 +329,7 @@ __device__ void copy_grid_entries(const Problem& P, const GridTable& T, uint32_t
     }
   }
   __syncthreads();
-  for (int i = tid; i < n_cols; i += kGridThreads) T.col[i].a = (int32_t)T.q[i];
+  for (int i = tid; i < n_cols; i += kGridThreads) T.col(i).a = (int32_t)T.q(i);
   __syncthreads();
 }
 
@@ -328,8 +339,7 @@ __device__ void copy_grid_entries(const Problem& P, const GridTable& T, uint32_t
 template <bool f32, bool w64, int G, bool pess, bool copied>
 __device__ __forceinline__ void grid_columns(const Problem& P, const GridTable& T,
                                              const Entries<typename PairOf<w64>::type, copied> src, int i0, int i1,
-                                             bool exact, const uint64_t* Vg, int lane, uint32_t* next, GridMiss* misses,
-                                             GridShared& S) {
+                                             bool exact, const uint64_t* Vg, int lane, uint32_t* next, GridShared& S) {
   typedef typename PairOf<w64>::type Pair;
   constexpr int NG = 32 / G;
   const int gi = lane / G, gl = lane % G;
@@ -339,7 +349,7 @@ __device__ __forceinline__ void grid_columns(const Problem& P, const GridTable& 
     base = i0 + __shfl_sync(kFull, base, 0);
     if (base >= i1) break;
     const int i = min(base + gi, i1 - 1);  // a group past the end reads the last column along
-    GridCol& c = T.col[i];
+    GridCol& c = T.col(i);
     const uint64_t rem = c.rem;
     const int32_t a = c.a, k = c.k, tried = c.e, hrow = c.hrow, x = c.x, last = c.last;
     const uint32_t lc = c.lc;
@@ -393,7 +403,7 @@ __device__ __forceinline__ void grid_columns(const Problem& P, const GridTable& 
     const bool mine = gl == 0 && base + gi < i1;
     const bool hit = tried >= 0 && (rem == 0 || (flt < r && part <= s.geq));
     if (mine && hit) {
-      T.q[lc & kLocalColumn] = s.acc + (w64 ? __umul64hi(vk, part) : mul_shr(vk >> 32, part, x));
+      T.q(lc & kLocalColumn) = s.acc + (w64 ? __umul64hi(vk, part) : mul_shr(vk >> 32, part, x));
       if (lc & kMoving) c.lc = lc & ~kMoving;
     }
     if (mine && !hit) {
@@ -409,7 +419,7 @@ __device__ __forceinline__ void grid_columns(const Problem& P, const GridTable& 
       m.neighbor = tried >= 0 && !(lc & kMoving) ? 1 : 0;
       m.hint = 0;
       m.pad = 0;
-      misses[atomicAdd(&S.n_miss, 1u)] = m;
+      unit_misses(S)[atomicAdd(&S.n_miss, 1u)] = m;
     }
   }
 }
@@ -430,7 +440,7 @@ template <bool f32, bool copied>
 __device__ __forceinline__ void settle_own(const Problem& P, const GridTable& T, const EntryCopy& D, GridMiss* at,
                                            const uint64_t* Vg, uint32_t scratch, int lane, const GridShared& S) {
   const GridMiss m = load_miss(at);
-  const GridCol& c = T.col[m.i];
+  const GridCol& c = T.col(m.i);
   const GridWindow w = S.win[c.win];
   const AnyV<f32> V{WindowV<f32>{w.off}, w.w0, w.len, Vg};
   const bool pess = P.pessimistic != 0, nb = m.neighbor != 0;
@@ -501,13 +511,15 @@ __device__ __forceinline__ void settle_few(const Problem& P, const GridTable& T,
 // its few (barrier `target`, waited for by one thread of the CTA), those that are
 // left anywhere, until a look at all lists finds none. False when the wait gave up.
 template <bool f32, bool copied>
-__device__ bool settle_misses(const StepLaunch& L, const GridPlan& R, const Problem& P, const GridTable& T,
-                              const EntryCopy& D, const uint64_t* Vg, uint32_t scratch, int k, uint32_t target,
-                              uint32_t own, int lane, int warp, GridShared& S) {
-  const int n_cta = (int)gridDim.x, me = (int)blockIdx.x;
-  uint32_t* listed = R.steal + (size_t)(k & 1) * 2 * n_cta;  // per CTA: misses listed
+__device__ bool settle_misses(const Problem& P, const GridTable& T, const EntryCopy& D, const uint64_t* Vg,
+                              uint32_t scratch, int k, uint32_t target, uint32_t own, int lane, int warp,
+                              GridShared& S) {
+  const GridUnit& U = S.unit;
+  StepControl* ctl = U.ctl;
+  const int n_cta = U.ctas, me = unit_rank(S);
+  uint32_t* listed = U.steal + (size_t)(k & 1) * 2 * n_cta;  // per CTA: misses listed
   uint32_t* taken = listed + n_cta;
-  GridMiss* mine = R.misses + (size_t)me * R.cap_cols;
+  GridMiss* mine = unit_misses(S);
   while (own) {
     uint32_t j = 0;
     if (lane == 0) j = atomicAdd(&taken[me], 1u);
@@ -519,13 +531,13 @@ __device__ bool settle_misses(const StepLaunch& L, const GridPlan& R, const Prob
   if (threadIdx.x == 0) {
     const long long t0 = clock64();
     int ok = 1;
-    for (uint32_t i = 0; !grid_arrived(L.ctl, target); ++i)
-      if ((i & 255) == 255 && !grid_waiting(L.ctl, t0)) {
+    for (uint32_t i = 0; !grid_arrived(ctl, target); ++i)
+      if ((i & 255) == 255 && !grid_waiting(ctl, t0)) {
         ok = 0;
         break;
       }
     S.ok = ok;
-    S.total = __ldcg(&L.ctl->misses[k & 3]);
+    S.total = __ldcg(&ctl->misses[k & 3]);
     __threadfence();
   }
   __syncthreads();
@@ -549,7 +561,7 @@ __device__ bool settle_misses(const StepLaunch& L, const GridPlan& R, const Prob
           j = __shfl_sync(kFull, j, 0);
           if (j >= many) break;
           found = true;
-          settle_other<f32>(P, R.misses + (size_t)victim * R.cap_cols + j, Vg, scratch, lane);
+          settle_other<f32>(P, U.misses + (size_t)victim * U.most_cols + j, Vg, scratch, lane);
         }
       }
     }
@@ -558,8 +570,7 @@ __device__ bool settle_misses(const StepLaunch& L, const GridPlan& R, const Prob
 }
 
 template <bool f32, int G, bool pess, bool copied>
-__device__ __forceinline__ int32_t grid_iterate(const StepLaunch& L, const Problem& P, const GridTable& T,
-                                                const GridLayout& lay, const GridPlan& R, int32_t k0, int32_t k1, GridShared& S) {
+__device__ __forceinline__ int32_t grid_iterate(const Problem& P, const GridTable& T, int32_t k0, int32_t k1, GridShared& S) {
   typedef typename std::conditional<f32, uint32_t, uint64_t>::type Cell;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const EntryCopy D = S.copy;
@@ -572,20 +583,18 @@ __device__ __forceinline__ int32_t grid_iterate(const StepLaunch& L, const Probl
     e32 = Entries<uint2, false>{P.rowval, P.lg32};
     e64 = Entries<ulonglong2, false>{P.rowval, f32 ? P.lgx : P.lg};
   }
-  const uint32_t scratch = (uint32_t)(lay.ws + warp * sizeof(WarpScratch));
+  const uint32_t scratch = kGridScratchAt + warp * (uint32_t)sizeof(WarpScratch);
   const bool infinite = P.infinite != 0, extra = infinite || P.policy_mode != 0;
-  const int n32 = S.n32, n_cols = S.n_cols, n_own = S.n_own, n_win = S.n_win;
-  Cell* cells = at_shared<Cell>((uint32_t)lay.v);
-  GridMiss* mine = R.misses + (size_t)blockIdx.x * R.cap_cols;
+  const int n32 = S.n32, n_cols = S.n_cols;
   uint32_t barrier = 0;
   int32_t k = k0;
   for (;; ++k) {
     const uint64_t* Vg = P.V[(k - 1) & 1];
     uint64_t* Vout = P.V[k & 1];
     // the windows of V_{k-1} (other CTAs wrote them: past L1)
-    for (int w = 0; w < n_win; ++w) {
+    for (int w = 0; w < S.n_win; ++w) {
       const unsigned long long* from = reinterpret_cast<const unsigned long long*>(Vg) + S.win[w].w0;
-      Cell* to = cells + S.win_at[w];
+      Cell* to = at_shared<Cell>(S.v) + S.win_at[w];
       for (int i = tid; i < S.win[w].len; i += kGridThreads) {
         const uint64_t v = __ldcg(from + i);
         to[i] = f32 ? (Cell)(v >> 32) : (Cell)v;
@@ -595,26 +604,28 @@ __device__ __forceinline__ int32_t grid_iterate(const StepLaunch& L, const Probl
     if (tid == 2) S.n_miss = S.taken = 0;
     __syncthreads();
     if (f32) {
-      grid_columns<f32, false, G, pess, copied>(P, T, e32, 0, n32, false, Vg, lane, &S.next[0], mine, S);
+      grid_columns<f32, false, G, pess, copied>(P, T, e32, 0, n32, false, Vg, lane, &S.next[0], S);
       if (n32 < n_cols)
-        grid_columns<f32, true, G, pess, copied>(P, T, e64, n32, n_cols, true, Vg, lane, &S.next[1], mine, S);
+        grid_columns<f32, true, G, pess, copied>(P, T, e64, n32, n_cols, true, Vg, lane, &S.next[1], S);
     } else {
-      grid_columns<f32, true, G, pess, copied>(P, T, e64, 0, n_cols, false, Vg, lane, &S.next[0], mine, S);
+      grid_columns<f32, true, G, pess, copied>(P, T, e64, 0, n_cols, false, Vg, lane, &S.next[0], S);
     }
     __syncthreads();
     const uint32_t n_miss = S.n_miss;
     // the states' new values, policy and residual
     const auto states = [&]() {
       unsigned long long dmax = 0;
+      const GridState* st = at_shared<GridState>(S.states);
+      const int n_own = S.n_own;
       for (int i = tid; i < n_own; i += kGridThreads) {
-        const GridState g = T.st[i];
+        const GridState g = st[i];
         const int32_t s = g.s;
         uint64_t bestq;
         int32_t best = 0;
-        if (R.single)
-          bestq = T.q[g.jb];
+        if (S.unit.single)
+          bestq = T.q(g.jb);
         else
-          best_action(P, g.jb, g.je, [&](int32_t c) { return T.q[c]; }, &bestq, &best);
+          best_action(P, g.jb, g.je, [&](int32_t c) { return T.q(c); }, &bestq, &best);
         const uint64_t vnew = free_state_value(P, s, bestq);
         Vout[s] = vnew;
         if (extra) {
@@ -636,18 +647,18 @@ __device__ __forceinline__ int32_t grid_iterate(const StepLaunch& L, const Probl
         if (tid == 0) {
           unsigned long long all = 0;
           for (int w = 0; w < kGridWarps; ++w) all = S.part[w] > all ? S.part[w] : all;
-          atomicMax(&L.ctl->resid[k & 3], all);
+          atomicMax(&S.unit.ctl->resid[k & 3], all);
         }
       }
     };
     // the columns' values and hints that the misses' records hold
     const auto collect = [&]() {
       for (uint32_t j = tid; j < n_miss; j += kGridThreads) {
-        const GridMiss m = load_miss(mine + j);
-        GridCol& c = T.col[m.i];
+        const GridMiss m = load_miss(unit_misses(S) + j);
+        GridCol& c = T.col(m.i);
         const uint32_t lc = c.lc & ~kMoving;
         const int32_t e = hint_entry(m.hint);
-        T.q[lc & kLocalColumn] = m.acc;
+        T.q(lc & kLocalColumn) = m.acc;
         c.lc = m.hint <= -2 ? lc | kMoving : lc;
         c.e = e;
         if (e >= 0) c.hrow = copied ? XRows{D.rows + c.a * 4u}[e] : __ldg(P.rowval + c.a + e);
@@ -656,7 +667,7 @@ __device__ __forceinline__ int32_t grid_iterate(const StepLaunch& L, const Probl
     };
     const uint32_t list = n_miss > kGridFewMisses ? n_miss : 0;
     if (n_miss && !list) {
-      settle_few<f32, copied>(P, T, D, mine, n_miss, Vg, scratch, lane, S);
+      settle_few<f32, copied>(P, T, D, unit_misses(S), n_miss, Vg, scratch, lane, S);
       __syncthreads();
       collect();
     }
@@ -665,28 +676,30 @@ __device__ __forceinline__ int32_t grid_iterate(const StepLaunch& L, const Probl
     ++barrier;
     if (tid == 0) {
       // this CTA's misses are listed (its part of the iteration is done if there are none)
-      uint32_t* steal = R.steal + (size_t)(k & 1) * 2 * gridDim.x;
-      uint32_t* next = R.steal + (size_t)((k + 1) & 1) * 2 * gridDim.x;
-      next[blockIdx.x] = next[gridDim.x + blockIdx.x] = 0;  // last read before the previous barrier
-      if (blockIdx.x == 0) {
-        L.ctl->resid[(k + 1) & 3] = 0;
-        L.ctl->misses[(k + 1) & 3] = 0;
+      const int n_cta = S.unit.ctas, me = unit_rank(S);
+      StepControl* ctl = S.unit.ctl;
+      uint32_t* steal = S.unit.steal + (size_t)(k & 1) * 2 * n_cta;
+      uint32_t* next = S.unit.steal + (size_t)((k + 1) & 1) * 2 * n_cta;
+      next[me] = next[n_cta + me] = 0;  // last read before the previous barrier
+      if (me == 0) {
+        ctl->resid[(k + 1) & 3] = 0;
+        ctl->misses[(k + 1) & 3] = 0;
       }
-      if (list) atomicAdd(&L.ctl->misses[k & 3], list);
-      steal[blockIdx.x] = list;
-      grid_arrive(L.ctl);
+      if (list) atomicAdd(&ctl->misses[k & 3], list);
+      steal[me] = list;
+      grid_arrive(ctl);
     }
-    if (!settle_misses<f32, copied>(L, R, P, T, D, Vg, scratch, k, barrier * gridDim.x, list, lane, warp, S)) return -1;
+    if (!settle_misses<f32, copied>(P, T, D, Vg, scratch, k, barrier * (uint32_t)S.unit.ctas, list, lane, warp, S)) return -1;
     if (S.total != 0) {
       // every miss is settled after one more barrier; their CTAs finish, and a last one ends the iteration
-      if (!grid_sync(L.ctl, ++barrier, S)) return -1;
+      if (!grid_sync(S.unit.ctl, ++barrier, S)) return -1;
       if (list) {
         collect();
         states();
       }
-      if (!grid_sync(L.ctl, ++barrier, S)) return -1;
+      if (!grid_sync(S.unit.ctl, ++barrier, S)) return -1;
     }
-    if (infinite && __ldcg(&L.ctl->resid[k & 3]) < P.eps_fix && !P.external_stop) break;
+    if (infinite && __ldcg(&S.unit.ctl->resid[k & 3]) < P.eps_fix && !P.external_stop) break;
     if (k == k1) break;
   }
   return k;
@@ -696,81 +709,92 @@ template <bool f32, int G>
 __global__ void __launch_bounds__(kGridThreads, 1) bellman_grid_kernel(StepLaunch L, GridPlan R, int32_t n_iters) {
   GridShared& S = *at_shared<GridShared>(0);
   constexpr int cell = f32 ? 4 : 8;
-  const GridLayout lay = grid_layout(R.cap_cols, R.cap_own, R.cap_cells, cell);
-  GridTable T;
-  T.col = at_shared<GridCol>((uint32_t)lay.cols);
-  T.q = at_shared<uint64_t>((uint32_t)lay.q);
-  T.st = at_shared<GridState>((uint32_t)lay.states);
   const int tid = threadIdx.x;
   const Problem& P = S.prob;
-  if (tid < (int)(sizeof(Problem) / 4))
-    reinterpret_cast<uint32_t*>(&S.prob)[tid] = reinterpret_cast<const uint32_t*>(L.probs)[tid];
-  IterState it = L.its[0];
-  const int32_t last = min(L.probs[0].horizon, it.iter + n_iters);
-  if (!it.done && last > it.iter) {
-    const int n_chunks = ((int)R.n_chunks - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    if (tid == 0) {
-      int32_t own = 0, cells = 0;
-      for (int j = 0; j < n_chunks; ++j) {
-        const int g = blockIdx.x + j * gridDim.x;
-        const int32_t a = R.chunk[g], b = R.chunk[g + 1];
-        S.chunk_s0[j] = a;
-        S.chunk_own[j] = own;
-        own += b - a;
-        if (R.one_window && j > 0) continue;
-        GridWindow w = R.one_window ? GridWindow{0, L.probs[0].n_states, 0} : R.win[g];
-        w.off = (int32_t)lay.v + (cells - w.w0) * cell;
-        S.win[j] = w;
-        S.win_at[j] = cells;
-        cells += w.len;
-      }
-      S.chunk_own[n_chunks] = own;
-      S.n_win = R.one_window ? min(1, n_chunks) : n_chunks;
-    }
+  const int2 todo = R.work[blockIdx.x];
+  for (int u = todo.x; u < todo.y; ++u) {
+    __syncthreads();  // the unit before is done with shared memory
+    if (tid < (int)(sizeof(GridUnit) / 4))
+      reinterpret_cast<uint32_t*>(&S.unit)[tid] = reinterpret_cast<const uint32_t*>(R.units + u)[tid];
     __syncthreads();
-    build_grid_columns<f32, G>(P, T, n_chunks, R.max_col, S);
-    copy_grid_entries<f32>(P, T, (uint32_t)lay.data, R.smem - (uint32_t)lay.data, S);
-    const int32_t k0 = it.iter + 1;
-    int32_t k;
-    if (S.copied)
-      k = P.pessimistic ? grid_iterate<f32, G, true, true>(L, P, T, lay, R, k0, last, S)
-                        : grid_iterate<f32, G, false, true>(L, P, T, lay, R, k0, last, S);
-    else
-      k = P.pessimistic ? grid_iterate<f32, G, true, false>(L, P, T, lay, R, k0, last, S)
-                        : grid_iterate<f32, G, false, false>(L, P, T, lay, R, k0, last, S);
-    if (k >= 0) {
-      it.iter = k;
-      const bool settled =
-          P.infinite && __ldcg(&L.ctl->resid[k & 3]) < P.eps_fix && !P.external_stop;
-      if (settled || k >= P.horizon) {
-        it.done = 1;
-        it.noconv = P.infinite && !settled ? 1 : 0;
+    const GridUnit& U = S.unit;
+    const GridLayout lay = grid_layout(U.most_cols, U.most_own, U.most_cells, cell);
+    const uint32_t end = R.smem & ~15u;
+    const GridTable T{end};
+    if (tid < (int)(sizeof(Problem) / 4))
+      reinterpret_cast<uint32_t*>(&S.prob)[tid] = reinterpret_cast<const uint32_t*>(L.probs + U.p)[tid];
+    __syncthreads();
+    StepControl* ctl = U.ctl;
+    const int n_cta = U.ctas;
+    IterState it = L.its[U.p];
+    const int32_t last = min(P.horizon, it.iter + (n_iters > 0 ? n_iters : U.iters));
+    if (!it.done && last > it.iter) {
+      const int me = unit_rank(S);
+      const int n_chunks = (U.n_chunks - me + n_cta - 1) / n_cta;
+      if (tid == 0) {
+        int32_t own = 0, cells = 0;
+        for (int j = 0; j < n_chunks; ++j) {
+          const int g = me + j * n_cta;
+          const int32_t a = U.chunk[g], b = U.chunk[g + 1];
+          S.chunk_s0[j] = a;
+          S.chunk_own[j] = own;
+          own += b - a;
+          if (U.one_window && j > 0) continue;
+          GridWindow w = U.one_window ? GridWindow{0, P.n_states, 0} : U.win[g];
+          w.off = (int32_t)lay.v + (cells - w.w0) * cell;
+          S.win[j] = w;
+          S.win_at[j] = cells;
+          cells += w.len;
+        }
+        S.chunk_own[n_chunks] = own;
+      S.states = lay.states;
+      S.v = lay.v;
+        S.n_win = U.one_window ? min(1, n_chunks) : n_chunks;
       }
-      // hints back to the session's state
-      for (int i = tid; i < S.n_cols; i += kGridThreads) {
-        const GridCol& c = T.col[i];
-        if (c.rem == 0) continue;
-        P.hint[c.c] = c.lc & kMoving ? -2 - c.e : c.e;
+      __syncthreads();
+      build_grid_columns<f32, G>(P, T, at_shared<GridState>(lay.states), n_chunks, U.max_col, S);
+      copy_grid_entries<f32>(P, T, lay.data, end - lay.q - lay.data, S);
+      const int32_t k0 = it.iter + 1;
+      int32_t k;
+      if (S.copied)
+        k = P.pessimistic ? grid_iterate<f32, G, true, true>(P, T, k0, last, S)
+                          : grid_iterate<f32, G, false, true>(P, T, k0, last, S);
+      else
+        k = P.pessimistic ? grid_iterate<f32, G, true, false>(P, T, k0, last, S)
+                          : grid_iterate<f32, G, false, false>(P, T, k0, last, S);
+      if (k >= 0) {
+        it.iter = k;
+        const bool settled = P.infinite && __ldcg(&ctl->resid[k & 3]) < P.eps_fix && !P.external_stop;
+        if (settled || k >= P.horizon) {
+          it.done = 1;
+          it.noconv = P.infinite && !settled ? 1 : 0;
+        }
+        // hints back to the problem's state
+        for (int i = tid; i < S.n_cols; i += kGridThreads) {
+          const GridCol& c = T.col(i);
+          if (c.rem == 0) continue;
+          P.hint[c.c] = c.lc & kMoving ? -2 - c.e : c.e;
+        }
       }
+    } else {
+      it.done = 1;  // horizon 0: nothing to run
     }
-  } else {
-    it.done = 1;  // horizon 0: nothing to run
-  }
-  if (it.done) it.k_final = it.iter;
-  __syncthreads();
-  // the last CTA writes the iteration state and resets the launch's counters
-  // (every CTA has read them by then)
-  if (tid == 0) {
-    __threadfence();
-    if (atomicAdd(&L.ctl->finished, 1u) == gridDim.x - 1u) {
+    if (it.done) it.k_final = it.iter;
+    __syncthreads();
+    // the unit's last CTA writes the iteration state and resets the unit's counters
+    // (every CTA has read them by then)
+    if (tid == 0) {
       __threadfence();
-      it.resmax = 0;
-      L.its[0] = it;
-      L.ctl->finished = 0;
-      L.ctl->arrived = 0;
-      for (int i = 0; i < 4; ++i) {
-        L.ctl->resid[i] = 0;
-        L.ctl->misses[i] = 0;
+      if (atomicAdd(&ctl->finished, 1u) == (uint32_t)n_cta - 1u) {
+        __threadfence();
+        it.resmax = 0;
+        L.its[U.p] = it;
+        ctl->finished = 0;
+        ctl->arrived = 0;
+        for (int i = 0; i < 4; ++i) {
+          ctl->resid[i] = 0;
+          ctl->misses[i] = 0;
+        }
       }
     }
   }
@@ -785,8 +809,75 @@ GridKernel grid_kernel(const GridPlan& R) {
 
 }  // namespace
 
-size_t grid_bytes(int32_t cols, int32_t own, int32_t cells, bool f32) {
-  return grid_layout(cols, own, cells, f32 ? 4 : 8).data;
+size_t grid_bytes(const GridCut& c, bool f32) {
+  const GridLayout l = grid_layout(c.most_cols, c.most_own, c.most_cells, f32 ? 4 : 8);
+  return (size_t)l.data + l.q;
+}
+
+// Cuts the states of a model (`fx`: those the property fixes) into chunks for
+// `ctas` CTAs. False when no CTA's share fits.
+bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut& out) {
+  const bool f32 = m->lg32 != nullptr;
+  const int32_t n = m->n_states;
+  const int32_t* sp = m->h_stateptr.data();
+  const int32_t* cp = m->h_colptr.data();
+  if (m->h_span.empty() || m->nnz >= kGridMostEntries) return false;
+  auto cost = [&](int32_t s) -> int64_t { return fx[s] ? 1 : cp[sp[s + 1]] - cp[sp[s]] + 24 * (sp[s + 1] - sp[s]); };
+  int64_t total = 0;
+  for (int32_t s = 0; s < n; ++s) total += cost(s);
+  // Chunks per CTA: more of them spread the regions where thresholds move (40,000
+  // states of 2 actions, 160 MB: 6.8 ms with 8, 5.4 with 16), but each has its own
+  // window to load (20,000 states of 40 entries: 1.6 ms with 8, 1.9 with 16): one
+  // for every 24 columns, and at most 96 KB of windows. One CTA alone takes all.
+  int per = ctas == 1 ? 1
+                      : (int)std::min<int64_t>(kGridMaxChunks, std::max<int64_t>(1, m->n_cols / (24 * (int64_t)ctas)));
+  std::vector<int64_t> cells, cols, own, ent;
+  int64_t most_cells = 0;
+  for (;; per = (per + 1) / 2) {
+    const int32_t nc = per * ctas;
+    out.chunk.assign(nc + 1, 0);
+    out.win.assign(nc, GridWindow{});
+    cells.assign(ctas, 0);
+    cols.assign(ctas, 0);
+    own.assign(ctas, 0);
+    ent.assign(ctas, 0);
+    int64_t done = 0;
+    int32_t s = 0;
+    for (int32_t g = 0; g < nc; ++g) {
+      // states of about equal work, and their window: all their destinations, or
+      // all but the columns' last ones when those alone would stretch it
+      const int c = g % ctas;
+      int32_t lo = n, hi = -1, inner = -1;
+      for (; s < n && (g == nc - 1 || done * nc < total * (g + 1)); ++s) {
+        done += cost(s);
+        lo = std::min(lo, m->h_span[s].x);
+        hi = std::max(hi, m->h_span[s].y);
+        inner = std::max(inner, m->h_span[s].z);
+        if (fx[s]) continue;
+        cols[c] += sp[s + 1] - sp[s];
+        own[c] += 1;
+        ent[c] += cp[sp[s + 1]] - cp[sp[s]];
+      }
+      out.chunk[g + 1] = s;
+      if (hi < 0) lo = hi = 0;
+      inner = std::max(inner, lo);
+      const int64_t all = (int64_t)hi - lo + 1, most = (int64_t)inner - lo + 1;
+      out.win[g] = GridWindow{lo, (int32_t)(all > 2 * most + 64 ? most : all), 0};
+      cells[c] += out.win[g].len;
+    }
+    most_cells = *std::max_element(cells.begin(), cells.end());
+    if (per == 1 || most_cells * (f32 ? 4 : 8) <= 96 * 1024 || most_cells >= n) break;
+  }
+  out.one_window = most_cells >= n ? 1 : 0;
+  most_cells = std::min<int64_t>(most_cells, n);
+  const int64_t most_cols = *std::max_element(cols.begin(), cols.end());
+  const int64_t most_own = *std::max_element(own.begin(), own.end());
+  if (most_cells > 60000 || most_cols > 5000 || most_own > 60000) return false;
+  out.most_cells = (int32_t)most_cells;
+  out.most_cols = (int32_t)most_cols;
+  out.most_own = (int32_t)most_own;
+  out.entries = *std::max_element(ent.begin(), ent.end());
+  return grid_bytes(out, f32) <= kResidentSmem;
 }
 
 cudaError_t grid_prepare(const GridPlan& R) {
@@ -797,9 +888,10 @@ cudaError_t grid_prepare(const GridPlan& R) {
   return e == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : e;
 }
 
+// `n_iters` 0: each unit's own number of iterations.
 cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t n_iters, cudaStream_t st) {
-  if (n_iters <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(R.steal, 0, sizeof(uint32_t) * 4 * (size_t)R.grid, st);
+  if (n_iters < 0) return cudaSuccess;
+  cudaError_t e = cudaMemsetAsync(R.steal, 0, sizeof(uint32_t) * 4 * (size_t)R.steal_ctas, st);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t c;
   std::memset(&c, 0, sizeof(c));

@@ -317,20 +317,40 @@ struct alignas(16) GridMiss {
   int32_t hint;
   int32_t pad;
 };
-struct GridPlan {
+// One problem of a launch, and the CTAs that run it.
+struct GridUnit {
   const int32_t* chunk;    // n_chunks + 1 state boundaries
   const GridWindow* win;   // per chunk
-  GridMiss* misses;        // cap_cols per CTA
+  GridMiss* misses;        // most_cols per CTA
   uint32_t* steal;         // by iteration parity, per CTA: misses listed, misses taken
-  int32_t n_chunks;        // 0: not taken
+  StepControl* ctl;        // the unit's barriers
+  int32_t p;               // problem
+  int32_t n_chunks;
   int32_t one_window;      // every CTA keeps all values (the windows' sum would be no smaller)
+  int32_t first, ctas;     // CTAs [first, first + ctas)
+  int32_t single;          // every state has one action
+  int32_t most_cols, most_own, most_cells;  // of one CTA
+  int32_t max_col;
+  int32_t iters;           // iterations in this launch, when the launch does not say
+  int32_t pad;
+};
+struct GridPlan {
+  const GridUnit* units;
+  const int2* work;        // per CTA: its units [x, y), one after the other (units of several CTAs: one)
+  uint32_t* steal;         // all units'
+  int32_t n_units;         // 0: not taken
+  int32_t steal_ctas;      // the units' CTAs together
   int32_t grid;            // CTAs
   int32_t group;           // lanes to a column
   int32_t f32;
-  int32_t single;          // every state has one action
-  int32_t cap_cols, cap_own, cap_cells;  // of one CTA
-  int32_t max_col;
   uint32_t smem;
+};
+// A model cut for a number of CTAs (plan_grid_unit).
+struct GridCut {
+  std::vector<int32_t> chunk;
+  std::vector<GridWindow> win;
+  int32_t one_window = 0, most_cols = 0, most_own = 0, most_cells = 0;  // most of one CTA
+  int64_t entries = 0;                                                  // likewise
 };
 
 // NVTX range for the host-side phases (model upload, session steps, server
@@ -363,7 +383,8 @@ cudaError_t resident_prepare(ResidentPlan& R);
 cudaError_t launch_bellman_resident(const StepLaunch& L, const ResidentPlan& R, int32_t n_iters, cudaStream_t st);
 // grid.cu
 // Shared memory of one CTA.
-size_t grid_bytes(int32_t cols, int32_t own, int32_t cells, bool f32);
+size_t grid_bytes(const GridCut& c, bool f32);
+bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut& out);
 cudaError_t grid_prepare(const GridPlan& R);
 cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t n_iters, cudaStream_t st);
 // CTAs of the persistent tiled kernel: one per SM.
@@ -444,7 +465,7 @@ struct Session {
   // Step calls by rule: the resident kernel's plan (n_units 0: not taken).
   ResidentPlan resident{};
   imdp_status plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st);
-  GridPlan whole{};  // the grid kernel's (n_chunks 0: not taken)
+  GridPlan whole{};  // the grid kernel's (n_units 0: not taken)
   imdp_status plan_grid(cudaStream_t st);
   SideStream side;  // created when the session has both tiles and wide states
   LaunchConfig cfg;  // launch configuration (rule, set_launch or the autotuner)

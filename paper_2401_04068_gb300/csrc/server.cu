@@ -81,6 +81,23 @@ class Arena {
   std::map<size_t, size_t> free_;
 };
 
+// Requests running together by rule share launches of the grid kernel: every
+// request gets CTAs in proportion to the work it has left, so that all end at
+// about the same time, and small ones are run by one CTA one after the other.
+// Per-iteration launches of the direct kernel take what the launch and its last
+// wave take, 500 times over, while a few large requests hold most of the work
+// (64 requests of 50 to 4000 states, 100 to 500 iterations: 49.3 ms,
+// 30.2 with shared launches; 19 requests 20.6 and 10.1). Bound by the misses of the
+// first iterations (a launch of 2 ms of steady iterations takes 6) and by 4 ms of
+// admission and results on the host.
+constexpr int32_t kGuessedIterations = 200;
+// Transitions (and 40 for a column) an SM takes per second: the grid kernel's
+// rate on models of 100 and more transitions a column.
+constexpr double kEntriesPerSecond = 2.4e9;
+// A launch lasts about this long: requests that arrive wait for it, and a launch
+// has tables to build (20 to 40 us) and its end to be noticed (50 us).
+constexpr double kQuantumSeconds = 2e-3;
+
 struct Request {
   uint64_t ticket = 0;
   DevModel* model = nullptr;
@@ -95,8 +112,23 @@ struct Request {
   int32_t k = 0;
   imdp_status status = IMDP_EPENDING;
   bool done = false;
-  std::vector<Tile> tiles;     // tile plan under the server's launch configuration (fixed states left out)
+  std::vector<uint8_t> fixed;  // per state: 1 reach, 2 avoid
+  LaunchConfig cfg;            // the server's when the request was admitted
+  bool planned = false;        // the two below are set (on the first per-iteration launch)
+  std::vector<Tile> tiles;     // tile plan under that configuration (fixed states left out)
   std::vector<int32_t> wide;   // wide states
+  int32_t least = 1;           // CTAs the grid kernel needs for it, as far as known
+  // iterations left (an infinite horizon: a guess, it ends by itself), and what
+  // one of them costs the grid kernel on one SM
+  int32_t left() const {
+    const int32_t cap = spec.infinite_time ? (spec.horizon > 0 ? spec.horizon : 1000000) : spec.horizon;
+    const int32_t n = std::max(cap - k, 1);
+    return spec.infinite_time ? std::min(n, kGuessedIterations) : n;
+  }
+  double seconds(int ctas) const {
+    const double work = (double)model->nnz + 40.0 * model->n_cols;
+    return (ctas > 1 ? 6.5e-6 : 4e-6) + work / (ctas * kEntriesPerSecond);
+  }
 };
 
 size_t working_bytes(const DevModel* m, const imdp_spec* sp) {
@@ -213,17 +245,13 @@ struct Server {
     P.property = sp->property;
     P.infinite = sp->infinite_time ? 1 : 0;
     P.horizon = sp->infinite_time ? (sp->horizon > 0 ? sp->horizon : 1000000) : sp->horizon;
-    std::vector<uint8_t> f((size_t)n, 0);
+    std::vector<uint8_t>& f = r->fixed;
+    f.assign((size_t)n, 0);
     if (sp->property != IMDP_REWARD) {
       for (int32_t v : r->reach) f[v] = 1;
       for (int32_t v : r->avoid) f[v] = 2;
     }
-    {
-      const LaunchConfig rc = resolve_launch(StepLaunch{}, &cfg);
-      r->tiles.clear();
-      r->wide.clear();
-      plan_tiles(m, 0, r->tiles, r->wide, rc.tile_entries, rc.wide_col, f.data());
-    }
+    r->cfg = cfg;
     cudaError_t e = cudaMemsetAsync(mask, 0, padded_u8(n), stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(mask, f.data(), n, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(hints, 0xff, padded_i32(m->n_cols) * sizeof(int32_t), stream);
@@ -280,6 +308,11 @@ struct Server {
     for (int32_t s = 0; s < count; ++s) {
       Request* r = slots[s];
       if (!r) continue;
+      if (!r->planned) {
+        const LaunchConfig rc = resolve_launch(StepLaunch{}, &r->cfg);
+        plan_tiles(r->model, 0, r->tiles, r->wide, rc.tile_entries, rc.wide_col, r->fixed.data());
+        r->planned = true;
+      }
       const size_t at = tiles.size();
       tiles.insert(tiles.end(), r->tiles.begin(), r->tiles.end());
       for (size_t t = at; t < tiles.size(); ++t) {
@@ -315,8 +348,6 @@ struct Server {
       e = cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess && !wide.empty())
       e = cudaMemcpyAsync(d_wide, wide.data(), sizeof(int2) * wide.size(), cudaMemcpyHostToDevice, stream);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(d_probs, probs_h.data(), sizeof(Problem) * count, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) return cuda_status(e, "server tables");
     n_tiles = (int32_t)tiles.size();
@@ -331,6 +362,247 @@ struct Server {
   SideStream side;
   int2* d_wide = nullptr;
   size_t wide_cap = 0;
+
+  // The grid kernel's plan for the running requests, in a block of the arena
+  // (so it counts against the budget; it is given back before requests are admitted).
+  GridPlan gplan{};
+  size_t g_off = 0, g_bytes = 0;
+  std::vector<GridUnit> g_units;  // by CTA; the units of one CTA behind one another
+  std::vector<int2> g_work;       // per CTA: its units
+  std::vector<Request*> g_reqs;   // per unit
+  uint64_t blocked = 0;           // the ticket that waits for budget although no plan held any
+  GridUnit* d_gunits = nullptr;
+  int2* d_gwork = nullptr;
+  StepControl* d_gctl = nullptr;
+
+  void drop_grid() {
+    if (g_bytes) arena.release(g_off, g_bytes);
+    g_bytes = 0;
+    gplan = GridPlan{};
+  }
+
+  // CTAs for every request so that each ends within T; the small ones in bins.
+  struct Share {
+    std::vector<std::pair<Request*, int>> wide;  // request, CTAs
+    std::vector<std::vector<Request*>> bins;     // one CTA each
+  };
+  static bool share(const std::vector<Request*>& rs, double T, int grid, Share& out) {
+    out.wide.clear();
+    out.bins.clear();
+    std::vector<double> load;
+    int used = 0;
+    for (Request* r : rs) {  // longest first
+      const double n = r->left(), one = n * r->seconds(1);
+      if (r->least == 1 && one <= T) {
+        size_t b = 0;
+        while (b < load.size() && load[b] + one > T) ++b;
+        if (b == load.size()) {
+          load.push_back(0.0);
+          out.bins.emplace_back();
+        }
+        load[b] += one;
+        out.bins[b].push_back(r);
+      } else {
+        const double fixed = n * 6.5e-6, rest = n * (r->seconds(2) - 6.5e-6) * 2.0;
+        if (T <= fixed) return false;
+        const double c = std::ceil(rest / (T - fixed));
+        if (c > grid) return false;
+        const int ctas = std::max({(int)c, r->least, 2});
+        out.wide.emplace_back(r, ctas);
+        used += ctas;
+      }
+      if (used + (int)out.bins.size() > grid) return false;
+    }
+    return true;
+  }
+
+  // Plans the running requests for the grid kernel (called with mu held: the
+  // arena). False when they do not fit it together.
+  bool plan_grid(int32_t count) {
+    drop_grid();
+    std::vector<Request*> rs;
+    int64_t nnz = 0, cols = 0;
+    for (int32_t s = 0; s < count; ++s)
+      if (slots[s]) {
+        rs.push_back(slots[s]);
+        nnz += slots[s]->model->nnz;
+        cols += slots[s]->model->n_cols;
+      }
+    const int grid = bellman_grid();
+    const bool f32 = !rs.empty() && rs[0]->model->lg32;
+    for (const Request* r : rs)
+      if ((r->model->lg32 != nullptr) != f32 || r->model->nnz >= kGridMostEntries) return false;
+    if (rs.empty()) return false;
+    std::stable_sort(rs.begin(), rs.end(), [](const Request* a, const Request* b) {
+      return a->left() * a->seconds(1) > b->left() * b->seconds(1);
+    });
+    Share best, now;
+    std::vector<GridCut> cuts;
+    for (int attempt = 0;; ++attempt) {
+      double hi = 0.0, lo = 0.0;
+      for (const Request* r : rs) hi += r->left() * r->seconds(1);
+      if (!share(rs, hi, grid, best)) return false;  // the least that the requests need is too much
+      for (int i = 0; i < 20; ++i) {
+        const double mid = 0.5 * (lo + hi);
+        if (share(rs, mid, grid, now)) {
+          hi = mid;
+          std::swap(best, now);
+        } else {
+          lo = mid;
+        }
+      }
+      cuts.assign(rs.size(), GridCut{});
+      bool ok = true;
+      size_t i = 0;
+      auto cut = [&](Request* r, int ctas) {
+        if (!plan_grid_unit(r->model, r->fixed.data(), ctas, cuts[i++])) {
+          r->least = ctas + std::max(1, ctas / 2);
+          ok = false;
+        }
+      };
+      for (auto& w : best.wide) cut(w.first, w.second);
+      for (auto& b : best.bins) {
+        // the one that ends first runs first
+        std::stable_sort(b.begin(), b.end(), [](const Request* x, const Request* y) {
+          return x->left() * x->seconds(1) < y->left() * y->seconds(1);
+        });
+        for (Request* r : b) cut(r, 1);
+      }
+      if (ok) break;
+      if (attempt == 8) return false;
+    }
+    // units, and where their tables lie in the block
+    g_units.clear();
+    g_work.clear();
+    g_reqs.clear();
+    size_t at = 0, misses = 0, chunks = 0;
+    auto take = [&](size_t bytes) {
+      const size_t o = at;
+      at += (bytes + 255) & ~size_t(255);
+      return o;
+    };
+    int32_t steal_ctas = 0;
+    bool copy = true;
+    size_t need = 0, all = 0;
+    auto unit = [&](Request* r, int first, int ctas) {
+      const GridCut& c = cuts[g_units.size()];
+      GridUnit u{};
+      u.p = r->slot;
+      u.n_chunks = (int32_t)c.win.size();
+      u.one_window = c.one_window;
+      u.first = first;
+      u.ctas = ctas;
+      u.single = r->model->n_cols == r->model->n_states ? 1 : 0;
+      u.most_cols = c.most_cols;
+      u.most_own = c.most_own;
+      u.most_cells = c.most_cells;
+      u.max_col = r->model->max_col;
+      g_units.push_back(u);
+      g_reqs.push_back(r);
+      steal_ctas += ctas;
+      chunks += c.chunk.size();
+      misses += (size_t)ctas * c.most_cols;
+      const size_t mine = grid_bytes(c, f32), with = mine + 64 + 20 * (size_t)c.entries;
+      need = std::max(need, mine);
+      all = std::max(all, with);
+      copy = copy && with <= kResidentSmem;
+    };
+    int first = 0;
+    for (auto& w : best.wide) {
+      for (int c = 0; c < w.second; ++c) g_work.push_back(make_int2((int)g_units.size(), (int)g_units.size() + 1));
+      unit(w.first, first, w.second);
+      first += w.second;
+    }
+    for (auto& b : best.bins) {
+      const int u0 = (int)g_units.size();
+      for (Request* r : b) unit(r, first, 1);
+      g_work.push_back(make_int2(u0, (int)g_units.size()));
+      ++first;
+    }
+    const size_t n = g_units.size();
+    const size_t o_units = take(n * sizeof(GridUnit)), o_work = take(g_work.size() * sizeof(int2)),
+                 o_ctl = take(n * sizeof(StepControl)), o_steal = take(4 * sizeof(uint32_t) * (size_t)steal_ctas),
+                 o_chunk = take(chunks * sizeof(int32_t)), o_win = take(chunks * sizeof(GridWindow)),
+                 o_miss = take(misses * sizeof(GridMiss));
+    size_t off;
+    if (!arena.alloc(at, &off)) return false;  // no room in the budget: per-iteration launches
+    g_off = off;
+    g_bytes = at;
+    unsigned char* block = base + off;
+    gplan.units = d_gunits = (GridUnit*)(block + o_units);
+    gplan.work = d_gwork = (int2*)(block + o_work);
+    d_gctl = (StepControl*)(block + o_ctl);
+    gplan.steal = (uint32_t*)(block + o_steal);
+    gplan.steal_ctas = steal_ctas;
+    gplan.grid = first;
+    gplan.group = nnz >= 256 * cols || cols < 48 * (int64_t)first ? 32 : 8;
+    gplan.f32 = f32 ? 1 : 0;
+    gplan.smem = (uint32_t)((copy ? all : need) + 15) & ~15u;
+    std::vector<int32_t> ch;
+    std::vector<GridWindow> wn;
+    ch.reserve(chunks);
+    wn.reserve(chunks);
+    GridMiss* miss = (GridMiss*)(block + o_miss);
+    uint32_t* steal = gplan.steal;
+    for (size_t i = 0; i < n; ++i) {
+      GridUnit& u = g_units[i];
+      const GridCut& c = cuts[i];
+      u.chunk = (int32_t*)(block + o_chunk) + ch.size();
+      u.win = (GridWindow*)(block + o_win) + wn.size();
+      ch.insert(ch.end(), c.chunk.begin(), c.chunk.end());
+      wn.insert(wn.end(), c.win.begin(), c.win.end());
+      u.misses = miss;
+      miss += (size_t)u.ctas * u.most_cols;
+      u.steal = steal;
+      steal += 4 * (size_t)u.ctas;
+      u.ctl = d_gctl + i;
+    }
+    cudaError_t e = grid_prepare(gplan);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_gctl, 0, n * sizeof(StepControl), stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync((void*)g_units[0].chunk, ch.data(), ch.size() * sizeof(int32_t), cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync((void*)g_units[0].win, wn.data(), wn.size() * sizeof(GridWindow), cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);  // the host vectors go out of scope
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      drop_grid();
+      return false;
+    }
+    gplan.n_units = (int32_t)n;
+    return true;
+  }
+
+  // Iterations of every unit in the next launch, about a quantum for each CTA;
+  // returns the CTAs that still have work.
+  int plan_quantum(std::vector<int2>& work) {
+    work.assign(g_work.size(), make_int2(0, 0));
+    std::vector<double> left(g_work.size(), 0.0);
+    double longest = 0.0;
+    auto per = [&](int u) { return g_reqs[u]->seconds(g_units[u].ctas); };
+    for (size_t c = 0; c < g_work.size(); ++c) {
+      for (int u = g_work[c].x; u < g_work[c].y; ++u)
+        if (g_reqs[u]) left[c] += g_reqs[u]->left() * per(u);
+      longest = std::max(longest, left[c]);
+    }
+    const double f = longest > kQuantumSeconds ? kQuantumSeconds / longest : 1.0;
+    int busy = 0;
+    for (size_t c = 0; c < g_work.size(); ++c) {
+      double budget = f * left[c];
+      int2& w = work[c];
+      for (int u = g_work[c].x; u < g_work[c].y && (w.y == 0 || budget > 1e-7); ++u) {
+        Request* r = g_reqs[u];
+        if (!r) continue;
+        const int32_t n = (int32_t)std::min<double>(r->left(), std::ceil(budget / per(u) - 1e-9));
+        g_units[u].iters = std::max(n, 1);
+        budget -= n * per(u);
+        if (w.y == 0) w.x = u;
+        w.y = u + 1;
+      }
+      busy += w.y > 0 ? 1 : 0;
+    }
+    return busy;
+  }
 
   void retire(Request* r, const IterState& it) {
     const DevModel* m = r->model;
@@ -351,6 +623,9 @@ struct Server {
     r->finished = Clock::now();
     std::lock_guard<std::mutex> lk(mu);
     arena.release(r->off, r->bytes);
+    for (Request*& g : g_reqs)
+      if (g == r) g = nullptr;
+    blocked = 0;
     slots[r->slot] = nullptr;
     std::memset(&probs_h[r->slot], 0, sizeof(Problem));
     r->slot = -1;
@@ -361,7 +636,11 @@ struct Server {
   void run() {
     cudaSetDevice(device);
     std::vector<IterState> its;
+    std::vector<StepControl> ctls;
+    std::vector<int2> work;
     int32_t count = 0;  // slots [0, count) are in the launch
+    bool stale = true;  // the per-iteration launches' tables are older than the slots
+    bool fits = true;   // the running requests fit the grid kernel together, as far as known
     while (true) {
       bool changed = false;
       const Clock::time_point h0 = Clock::now();
@@ -383,7 +662,13 @@ struct Server {
             }
           if (slot < 0) break;
           Request* r = queue.front();
-          if (!admit(r, slot)) break;  // wait for budget
+          if (!admit(r, slot)) {
+            // the grid kernel's plan makes room, once for a request that then still has to wait
+            if (!g_bytes || blocked == r->ticket) break;
+            drop_grid();
+            blocked = r->ticket;
+            continue;
+          }
           queue.pop_front();
           changed = true;
         }
@@ -392,9 +677,30 @@ struct Server {
       for (int s = 0; s < max_active; ++s)
         if (slots[s]) hi = s + 1;
       if (hi == 0) continue;
+      cudaError_t e = cudaSuccess;
+      LaunchConfig lc;
+      bool grid_kernel = false;
       if (changed || hi != count) {
         // slots without a request keep done = 1 (set at creation, kept on retire)
+        stale = true;
+        fits = fits || changed;
         count = hi;
+        e = cudaMemcpyAsync(d_probs, probs_h.data(), sizeof(Problem) * count, cudaMemcpyHostToDevice, stream);
+      }
+      {
+        std::lock_guard<std::mutex> lk(mu);
+        lc = cfg;
+        if (lc.kernel == kKernelRule && fits) {
+          // planned again when a quarter of the CTAs have run out of work
+          grid_kernel = gplan.n_units > 0 && !changed && plan_quantum(work) * 4 > gplan.grid * 3;
+          if (!grid_kernel) {
+            grid_kernel = fits = plan_grid(count);
+            if (grid_kernel) plan_quantum(work);
+          }
+        }
+        if (!grid_kernel) drop_grid();
+      }
+      if (!grid_kernel && stale && e == cudaSuccess) {
         const imdp_status st = upload_tables(count);
         if (st != IMDP_OK) {
           std::lock_guard<std::mutex> lk(mu);
@@ -407,6 +713,7 @@ struct Server {
           cv.notify_all();
           return;
         }
+        stale = false;
       }
       pending_host_ms = std::chrono::duration<double, std::milli>(Clock::now() - h0).count();
       StepLaunch L{};
@@ -424,25 +731,32 @@ struct Server {
       L.n_wide = n_wide;
       const int grid = bellman_grid();
       TraceRange trace("imdp server chunk");
-      LaunchConfig lc;
-      {
-        std::lock_guard<std::mutex> lk(mu);
-        lc = cfg;
-      }
       const Clock::time_point w0 = Clock::now();
-      cudaError_t e = cudaSuccess;
-      if (!ev0) {
+      if (!ev0 && e == cudaSuccess) {
         e = cudaEventCreate(&ev0);
         if (e == cudaSuccess) e = cudaEventCreate(&ev1);
       }
+      if (grid_kernel && e == cudaSuccess) {
+        e = cudaMemcpyAsync(d_gunits, g_units.data(), sizeof(GridUnit) * g_units.size(), cudaMemcpyHostToDevice, stream);
+        if (e == cudaSuccess)
+          e = cudaMemcpyAsync(d_gwork, work.data(), sizeof(int2) * work.size(), cudaMemcpyHostToDevice, stream);
+      }
       if (e == cudaSuccess) e = cudaEventRecord(ev0, stream);
-      for (int i = 0; i < chunk && e == cudaSuccess; ++i) e = launch_bellman_step(L, grid, stream, &side, &lc);
+      if (grid_kernel) {
+        if (e == cudaSuccess) e = launch_bellman_grid(L, gplan, 0, stream);
+      } else {
+        for (int i = 0; i < chunk && e == cudaSuccess; ++i) e = launch_bellman_step(L, grid, stream, &side, &lc);
+      }
       if (e == cudaSuccess) e = cudaEventRecord(ev1, stream);
       its.resize(count);
       StepControl c{};
       if (e == cudaSuccess) e = cudaMemcpyAsync(its.data(), d_its, sizeof(IterState) * count, cudaMemcpyDeviceToHost, stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(&c, d_ctl, sizeof(c), cudaMemcpyDeviceToHost, stream);
+      ctls.resize(grid_kernel ? g_units.size() : 0);
+      if (e == cudaSuccess && !grid_kernel) e = cudaMemcpyAsync(&c, d_ctl, sizeof(c), cudaMemcpyDeviceToHost, stream);
+      if (e == cudaSuccess && grid_kernel)
+        e = cudaMemcpyAsync(ctls.data(), d_gctl, sizeof(StepControl) * ctls.size(), cudaMemcpyDeviceToHost, stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+      for (const StepControl& g : ctls) c.error |= g.error;
       if (e != cudaSuccess || c.error) {
         std::lock_guard<std::mutex> lk(mu);
         fatal = e != cudaSuccess ? cuda_status(e, "server step") : IMDP_ETIMEOUT;
@@ -460,7 +774,11 @@ struct Server {
       for (int s = 0; s < count; ++s) {
         Request* r = slots[s];
         active += r ? 1 : 0;
-        if (r && its[s].done) retire(r, its[s]);
+        if (r) r->k = its[s].iter;
+        if (r && its[s].done) {
+          retire(r, its[s]);
+          fits = true;
+        }
       }
       {
         std::lock_guard<std::mutex> lk(mu);

@@ -496,96 +496,51 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
 imdp_status Session::plan_grid(cudaStream_t st) {
   whole = GridPlan{};
   const DevModel* m = models[0];
-  if (L.tiny_ok || resident.n_units > 0 || count != 1 || m->h_span.empty() || m->nnz >= kGridMostEntries) return IMDP_OK;
+  GridCut cut;
+  if (L.tiny_ok || resident.n_units > 0 || count != 1 || !plan_grid_unit(m, fixed_h.data(), grid, cut)) return IMDP_OK;
   const bool f32 = m->lg32 != nullptr;
-  const int32_t n = m->n_states;
-  const int32_t* sp = m->h_stateptr.data();
-  const int32_t* cp = m->h_colptr.data();
-  const uint8_t* fx = fixed_h.data();
-  auto cost = [&](int32_t s) -> int64_t { return fx[s] ? 1 : cp[sp[s + 1]] - cp[sp[s]] + 24 * (sp[s + 1] - sp[s]); };
-  int64_t total = 0;
-  for (int32_t s = 0; s < n; ++s) total += cost(s);
-  // Chunks per CTA: more of them spread the regions where thresholds move (40,000
-  // states of 2 actions, 160 MB: 6.8 ms with 8, 5.4 with 16), but each has its own
-  // window to load (20,000 states of 40 entries: 1.6 ms with 8, 1.9 with 16): one
-  // for every 24 columns, and at most 96 KB of windows.
-  int per = (int)std::min<int64_t>(kGridMaxChunks, std::max<int64_t>(1, m->n_cols / (24 * (int64_t)grid)));
-  std::vector<int32_t> chunk;
-  std::vector<GridWindow> win;
-  std::vector<int64_t> cells, cols, own, ent;
-  int64_t cap_cells = 0;
-  int32_t nc = 0;
-  for (;; per = (per + 1) / 2) {
-    nc = per * grid;
-    chunk.assign(nc + 1, 0);
-    win.assign(nc, GridWindow{});
-    cells.assign(grid, 0);
-    cols.assign(grid, 0);
-    own.assign(grid, 0);
-    ent.assign(grid, 0);
-    int64_t done = 0;
-    int32_t s = 0;
-    for (int32_t g = 0; g < nc; ++g) {
-      // states of about equal work, and their window: all their destinations, or
-      // all but the columns' last ones when those alone would stretch it
-      const int c = g % grid;
-      int32_t lo = n, hi = -1, inner = -1;
-      for (; s < n && (g == nc - 1 || done * nc < total * (g + 1)); ++s) {
-        done += cost(s);
-        lo = std::min(lo, m->h_span[s].x);
-        hi = std::max(hi, m->h_span[s].y);
-        inner = std::max(inner, m->h_span[s].z);
-        if (fx[s]) continue;
-        cols[c] += sp[s + 1] - sp[s];
-        own[c] += 1;
-        ent[c] += cp[sp[s + 1]] - cp[sp[s]];
-      }
-      chunk[g + 1] = s;
-      if (hi < 0) lo = hi = 0;
-      inner = std::max(inner, lo);
-      const int64_t all = (int64_t)hi - lo + 1, most = (int64_t)inner - lo + 1;
-      win[g] = GridWindow{lo, (int32_t)(all > 2 * most + 64 ? most : all), 0};
-      cells[c] += win[g].len;
-    }
-    cap_cells = *std::max_element(cells.begin(), cells.end());
-    if (per == 1 || cap_cells * (f32 ? 4 : 8) <= 96 * 1024 || cap_cells >= n) break;
-  }
-  whole.one_window = cap_cells >= n ? 1 : 0;
-  cap_cells = std::min<int64_t>(cap_cells, n);
-  const int64_t cap_cols = *std::max_element(cols.begin(), cols.end());
-  const int64_t cap_own = *std::max_element(own.begin(), own.end());
-  if (cap_cells > 60000 || cap_cols > 5000 || cap_own > 60000) return IMDP_OK;
-  const size_t need = grid_bytes((int32_t)cap_cols, (int32_t)cap_own, (int32_t)cap_cells, f32);
-  if (need > kResidentSmem) return IMDP_OK;
-  const size_t all = need + 64 + 20 * (size_t)*std::max_element(ent.begin(), ent.end());
-  whole.smem = (uint32_t)(all <= kResidentSmem ? all : need);
-  whole.cap_cols = (int32_t)cap_cols;
-  whole.cap_own = (int32_t)cap_own;
-  whole.cap_cells = (int32_t)cap_cells;
-  whole.grid = grid;
+  const size_t need = grid_bytes(cut, f32), all = need + 64 + 20 * (size_t)cut.entries;
+  whole.smem = (uint32_t)((all <= kResidentSmem ? all : need) + 15) & ~15u;
+  whole.grid = whole.steal_ctas = grid;
   whole.group = m->nnz >= 256 * (int64_t)m->n_cols || m->n_cols < 48 * (int64_t)grid ? 32 : 8;
   whole.f32 = f32 ? 1 : 0;
-  whole.single = m->n_cols == n ? 1 : 0;
-  whole.max_col = m->max_col;
   if (grid_prepare(whole) != cudaSuccess) {
     cudaGetLastError();
     return IMDP_OK;
   }
-  int32_t* dc = alloc<int32_t>(chunk.size());
-  GridWindow* dw = alloc<GridWindow>(win.size());
-  whole.misses = alloc<GridMiss>((size_t)grid * cap_cols);
-  whole.steal = alloc<uint32_t>(4 * (size_t)grid);
-  if (!dc || !dw || !whole.misses || !whole.steal) {
+  int32_t* dc = alloc<int32_t>(cut.chunk.size());
+  GridWindow* dw = alloc<GridWindow>(cut.win.size());
+  GridUnit* du = alloc<GridUnit>(1);
+  int2* work = alloc<int2>(grid);
+  GridUnit u{};
+  u.misses = alloc<GridMiss>((size_t)grid * cut.most_cols);
+  u.steal = whole.steal = alloc<uint32_t>(4 * (size_t)grid);
+  if (!dc || !dw || !du || !work || !u.misses || !u.steal) {
     set_error("device allocation failed (session)");
     return IMDP_ENOMEM;
   }
-  cudaError_t e = cudaMemcpyAsync(dc, chunk.data(), sizeof(int32_t) * chunk.size(), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dw, win.data(), sizeof(GridWindow) * win.size(), cudaMemcpyHostToDevice, st);
+  u.chunk = dc;
+  u.win = dw;
+  u.ctl = ctl;
+  u.n_chunks = (int32_t)cut.win.size();
+  u.one_window = cut.one_window;
+  u.ctas = grid;
+  u.single = m->n_cols == m->n_states ? 1 : 0;
+  u.most_cols = cut.most_cols;
+  u.most_own = cut.most_own;
+  u.most_cells = cut.most_cells;
+  u.max_col = m->max_col;
+  const std::vector<int2> all_of_one(grid, make_int2(0, 1));
+  cudaError_t e = cudaMemcpyAsync(dc, cut.chunk.data(), sizeof(int32_t) * cut.chunk.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(dw, cut.win.data(), sizeof(GridWindow) * cut.win.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(du, &u, sizeof(u), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(work, all_of_one.data(), sizeof(int2) * grid, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host vectors go out of scope
   if (e != cudaSuccess) return cuda_status(e, "session plan");
-  whole.chunk = dc;
-  whole.win = dw;
-  whole.n_chunks = nc;
+  whole.units = du;
+  whole.work = work;
+  whole.n_units = 1;
   return IMDP_OK;
 }
 
@@ -801,7 +756,7 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
     launched_since_reset += n;
     return IMDP_OK;
   }
-  if (cfg.kernel == kKernelRule && n >= kResidentSteps && (resident.n_units > 0 || whole.n_chunks > 0)) {
+  if (cfg.kernel == kKernelRule && n >= kResidentSteps && (resident.n_units > 0 || whole.n_units > 0)) {
     // by rule: all n iterations in one launch of the resident or the grid kernel,
     // or in several of about half a second, so that a long call does not hold the
     // SMs that another stream's grid kernel waits for
