@@ -293,8 +293,7 @@ IMDP_API void imdp_session_destroy(imdp_session* s);
  * Launch configuration of a session's Bellman step (no counterpart in the
  * paper, whose GPU kernels have one fixed shape). Every configuration computes
  * the same words; they differ in speed only. Zero fields mean "by rule".
- *   kernel        0 by rule: the single-CTA kernel for a session of one small
- *                 problem; else step calls of 4 or more iterations run them in one
+ *   kernel        0 by rule: step calls of 4 or more iterations run them in one
  *                 launch of the resident kernel where its values fit shared memory
  *                 and its cost model says it pays (no state slices, one storage
  *                 format): every problem, or every part of one finite-horizon
@@ -304,15 +303,16 @@ IMDP_API void imdp_session_destroy(imdp_session* s);
  *                 kernel, whose CTAs each keep the values their states need on chip
  *                 and wait for one another after every iteration. Everything else
  *                 runs one iteration per launch (what imdp_session_get_launch
- *                 reports), from the shape of the session's problems (the
+ *                 reports): the single-CTA kernel for a session of one small
+ *                 problem; else, from the shape of the session's problems (the
  *                 autotuner's choices on GB300 for the benchmark shapes), direct
  *                 with 3 CTAs per SM and 1024-entry tiles when their columns hold
  *                 256 or more transitions on average, otherwise slice with 3 CTAs
  *                 per SM (4 when every problem has 32-bit storage) when every
  *                 model already has its slice layout (see 4 below: building it
  *                 costs about as many iterations' time as a few hundred save),
- *                 otherwise ring (the server's rule is the single-CTA kernel or
- *                 ring);
+ *                 otherwise ring (the server's rule is the grid kernel, several
+ *                 requests in one launch, or ring);
  *                 1 ring: a producer warp bulk-copies tiles of
  *                 consecutive states into a three-stage shared-memory ring for
  *                 consumer warps; 2 direct: every warp takes the next tile and
@@ -481,9 +481,11 @@ IMDP_API imdp_status imdp_session_restore(imdp_session* s, int32_t index, const 
  * Continuous-batching server. Requests (a resident model plus a specification)
  * share the Bellman launches of one slotted batch run by a worker thread: a
  * request is admitted when a slot (up to 1024) and enough of the server's device
- * memory budget are free, joins the running batch between chunks of 8
- * iterations, and retires on its own horizon or convergence test. Each result
- * equals what imdp_value_iteration returns for the same request alone.
+ * memory budget are free, joins the running batch between launches (by rule
+ * about 2 ms of iterations of all requests in one launch of the grid kernel, or
+ * chunks of 8 per-iteration launches), and retires on its own horizon or
+ * convergence test. Each result equals what imdp_value_iteration returns for the
+ * same request alone.
  *   hbm_budget   bytes of device memory for per-request state (values, masks,
  *                hints, outputs); allocated once at creation (>= 1 MiB)
  * Thread-safe: submit/poll/wait may be called from any thread. Models must

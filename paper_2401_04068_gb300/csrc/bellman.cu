@@ -916,7 +916,10 @@ __global__ void __launch_bounds__(32 * NW, MINB) bellman_slice_kernel(StepLaunch
 // launch of the tiled kernels. The columns run the same exact routines (V read
 // from shared memory), so the words are those of the tiled kernels. This
 // removes the per-iteration launch (a few microseconds each, more than the
-// work of such a problem).
+// work of such a problem). A chain of dependent steps, a column per warp at a
+// time, bounds it: step calls of four or more iterations take the resident kernel
+// (200 iterations of 5 columns 322 us here and 240 there, 200 columns of 12 entries
+// 5836 and 439), shorter ones would not pay for building its tables.
 constexpr int kTinyWarps = 4;
 
 struct TinyLayout {

@@ -341,7 +341,6 @@ imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<
 
 imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st) {
   resident = ResidentPlan{};
-  if (L.tiny_ok) return IMDP_OK;
   bool any32 = false, any64 = false;
   for (const DevModel* m : models) {
     if (is_slice(m)) return IMDP_OK;
@@ -404,16 +403,24 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
   while (c < kMaxCluster && ((int64_t)n_units * c < grid || unit_bytes * (grid / c) > 200e6 ||
                              (double)most / c > 1.7 * (double)work / grid))
     c *= 2;
+  // Small units: at least 7 columns to a CTA (200 iterations of 12 columns 276 us
+  // with one CTA, 310 with 4; 20 columns 330 with 2 or 4; 200 columns of 12 entries
+  // 690 / 525 / 457 with 1 / 2 / 16).
+  while (c > 1 && cols < 7 * (int64_t)c * n_units) c /= 2;
+  const bool alone = count == 1 && n_units == 1;
   // Two CTAs of an SM overlap each other's barriers while both their units stay
   // in L2 (4096 parts of 0.3 MB on 32-bit storage: 68 ms against 74 with one).
   const bool two = n_units * (int64_t)c >= 2 * grid && unit_bytes * (2 * grid / c) <= 100e6;
-  resident.threads = two ? kResidentThreads / 2 : kResidentThreads;
+  // Half the warps also where they hold a CTA's few short columns: their barriers
+  // are cheaper (5 columns 238 us against 251, 600 columns 607 against 799).
+  const bool few = alone && cols <= 48 * c && entries <= 32 * cols;
+  resident.threads = two || few ? kResidentThreads / 2 : kResidentThreads;
   // Seconds an iteration takes: per-iteration launches about 10 us and 0.64
   // transitions a cycle and SM, this kernel about 3 us and 1.17 on the SMs it
   // covers, the grid kernel (one problem only) about 6.5 us and 1 on all.
   const double sms = std::min<double>(grid, (double)n_units * c), hz = 1.9e9, e = (double)entries;
   double other = 10e-6 + e / (0.64 * grid * hz);
-  if (count == 1 && n_units == 1) other = std::min(other, 6.5e-6 + e / (1.0 * grid * hz));
+  if (alone) other = std::min(other, 6.5e-6 + e / (1.0 * grid * hz));
   if (3e-6 + e / (1.17 * sms * hz) > other) return IMDP_OK;
   // ranks of a unit: contiguous states of about equal work
   std::vector<int32_t> bounds;
@@ -748,15 +755,16 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
   if (n <= 0) return IMDP_OK;
   TraceRange trace("imdp session step");
   cudaError_t e = cudaSuccess;
-  if (resolve_launch(L, &cfg).kernel == kKernelTiny) {
-    // one small problem: all n iterations in one launch of one CTA
+  const bool long_step = cfg.kernel == kKernelRule && n >= kResidentSteps && (resident.n_units > 0 || whole.n_units > 0);
+  if (!long_step && resolve_launch(L, &cfg).kernel == kKernelTiny) {
+    // one small problem, few iterations: all of them in one launch of one CTA
     e = launch_bellman_tiny(L, n, models[0]->lg32 != nullptr, st);
     if (e != cudaSuccess) return cuda_status(e, "bellman step");
     launches += n;
     launched_since_reset += n;
     return IMDP_OK;
   }
-  if (cfg.kernel == kKernelRule && n >= kResidentSteps && (resident.n_units > 0 || whole.n_units > 0)) {
+  if (long_step) {
     // by rule: all n iterations in one launch of the resident or the grid kernel,
     // or in several of about half a second, so that a long call does not hold the
     // SMs that another stream's grid kernel waits for

@@ -167,3 +167,21 @@ def test_one_large_problem(shape, case):
         _, oV, _, _, _ = run_oracle(m, **kw)
         assert float(np.max(np.abs(ref[0][0].astype(np.float64) / 2.0 ** 63 - oV))) <= TOL_F64
     model.close()
+
+
+# the smallest problems (one CTA, half its warps, or a few CTAs) and step calls
+# too short for a resident launch in between (the single-CTA kernel)
+@pytest.mark.parametrize("shape", [(1, 1, 1), (5, 1, 5), (7, 3, 4), (64, 1, 12), (330, 3, 4), (1000, 1, 3)])
+@pytest.mark.parametrize("storage", ["f64", "f32"])
+def test_small_problem(shape, storage):
+    n, a, k = shape
+    m = banded_imdp(n, a, n * a * (min(k, n) + 1) + 1, eps=0.1, seed=n)
+    model = g.create_model(m, dtype=g.IMDP_F32 if storage == "f32" else g.IMDP_F64)
+    for kw in (dict(horizon=23, reach=m.goal), dict(infinite_time=True, eps=1e-5, horizon=90, reach=m.goal),
+               dict(horizon=23, reach=m.goal, pessimistic=False, maximize=False)):
+        spec = [g.make_spec(**kw)]
+        policy = "infinite_time" not in kw
+        ref = _run([model], [m], spec, g.KERNEL_RING, policy=policy)
+        _same(ref, _run([model], [m], spec, g.KERNEL_RULE, policy=policy))
+        _same(ref, _run([model], [m], spec, g.KERNEL_RULE, steps=(3, 5, 1, 4, 2, 90), policy=policy))
+    model.close()
