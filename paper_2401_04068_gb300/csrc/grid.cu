@@ -85,7 +85,7 @@ struct GridShared {
 // windows, and the entries where they fit.
 __host__ __device__ constexpr size_t grid_align(size_t x) { return (x + 15) & ~size_t(15); }
 constexpr uint32_t kGridScratchAt = (uint32_t)grid_align(sizeof(GridShared));
-constexpr uint32_t kGridColumnsAt = (uint32_t)grid_align(kGridScratchAt + kGridWarps * sizeof(WarpScratch));
+constexpr uint32_t kGridColumnsAt = (uint32_t)grid_align(kGridScratchAt + kGridWarps * sizeof(SettleScratch));
 struct GridLayout {
   uint32_t states, v, data, q;  // `q`: bytes at the end
 };
@@ -436,9 +436,9 @@ __device__ __forceinline__ GridMiss load_miss(const GridMiss* p) {
 
 // Settles one missed column; its value and hint go to its record. `own`: the
 // CTA's own column (its table, windows and copy), else another CTA's.
-template <bool f32, bool copied>
+template <bool f32, bool copied, bool team>
 __device__ __forceinline__ void settle_own(const Problem& P, const GridTable& T, const EntryCopy& D, GridMiss* at,
-                                           const uint64_t* Vg, uint32_t scratch, int lane, const GridShared& S) {
+                                           const uint64_t* Vg, const Team& W, int lane, const GridShared& S) {
   const GridMiss m = load_miss(at);
   const GridCol& c = T.col(m.i);
   const GridWindow w = S.win[c.win];
@@ -450,21 +450,21 @@ __device__ __forceinline__ void settle_own(const Problem& P, const GridTable& T,
   if constexpr (copied) {
     const XRows rows{D.rows + a * 4u};
     if (f32 && m.i < S.n32)
-      q = missed_column<true, 3, kSettleTrips>(rows, Bounds<true, 3>{D.pairs + a * 8u, 32 - x}, m.k, m.rem, V, pess, nb, m.vk, m.acc,
-                                 m.flt, m.geq, scratch, w.w0, lane, &ho);
+      q = missed_column<true, 3, kSettleTrips, team>(rows, Bounds<true, 3>{D.pairs + a * 8u, 32 - x}, m.k, m.rem, V, pess, nb, m.vk, m.acc,
+                                 m.flt, m.geq, W, w.w0, lane, &ho);
     else
-      q = missed_column<false, 3, kSettleTrips>(rows, Bounds<false, 3>{(f32 ? D.exact : D.pairs) + a * 16u, 0}, m.k, m.rem, V, pess, nb,
-                                  m.vk, m.acc, m.flt, m.geq, scratch, w.w0, lane, &ho);
+      q = missed_column<false, 3, kSettleTrips, team>(rows, Bounds<false, 3>{(f32 ? D.exact : D.pairs) + a * 16u, 0}, m.k, m.rem, V, pess, nb,
+                                  m.vk, m.acc, m.flt, m.geq, W, w.w0, lane, &ho);
   } else {
     const GRows rows{P.rowval + a};
     if (f32 && m.i < S.n32)
-      q = missed_column<true, 1, kSettleTrips>(rows, Bounds<true, 1>{P.lg32 + a, 32 - x}, m.k, m.rem, V, pess, nb, m.vk, m.acc, m.flt,
-                                 m.geq, scratch, w.w0, lane, &ho);
+      q = missed_column<true, 1, kSettleTrips, team>(rows, Bounds<true, 1>{P.lg32 + a, 32 - x}, m.k, m.rem, V, pess, nb, m.vk, m.acc, m.flt,
+                                 m.geq, W, w.w0, lane, &ho);
     else
-      q = missed_column<false, 1, kSettleTrips>(rows, Bounds<false, 1>{f32 ? P.lgx + x : P.lg + a, 0}, m.k, m.rem, V, pess, nb, m.vk,
-                                  m.acc, m.flt, m.geq, scratch, w.w0, lane, &ho);
+      q = missed_column<false, 1, kSettleTrips, team>(rows, Bounds<false, 1>{f32 ? P.lgx + x : P.lg + a, 0}, m.k, m.rem, V, pess, nb, m.vk,
+                                  m.acc, m.flt, m.geq, W, w.w0, lane, &ho);
   }
-  if (lane == 0) {
+  if (lane == 0 && (!team || W.rank == 0)) {
     at->acc = q;
     at->hint = ho;
   }
@@ -481,11 +481,11 @@ __device__ __forceinline__ void settle_other(const Problem& P, GridMiss* at, con
   uint64_t q;
   if (f32 && P.xoff) x = __ldg(P.xoff + m.c);
   if (f32 && x < 0)
-    q = missed_column<true, 1, kSettleTrips>(rows, Bounds<true, 1>{P.lg32 + a, 32 - __ldg(P.shift + m.c)}, m.k, m.rem, V, pess, nb,
-                               m.vk, m.acc, m.flt, m.geq, scratch, 0, lane, &ho);
+    q = missed_column<true, 1, kSettleTrips, false>(rows, Bounds<true, 1>{P.lg32 + a, 32 - __ldg(P.shift + m.c)}, m.k, m.rem, V, pess, nb,
+                               m.vk, m.acc, m.flt, m.geq, Team{1, 0, 0, scratch}, 0, lane, &ho);
   else
-    q = missed_column<false, 1, kSettleTrips>(rows, Bounds<false, 1>{f32 ? P.lgx + x : P.lg + a, 0}, m.k, m.rem, V, pess, nb, m.vk,
-                                m.acc, m.flt, m.geq, scratch, 0, lane, &ho);
+    q = missed_column<false, 1, kSettleTrips, false>(rows, Bounds<false, 1>{f32 ? P.lgx + x : P.lg + a, 0}, m.k, m.rem, V, pess, nb, m.vk,
+                                m.acc, m.flt, m.geq, Team{1, 0, 0, scratch}, 0, lane, &ho);
   if (lane == 0) {
     at->acc = q;
     at->hint = ho;
@@ -502,8 +502,21 @@ __device__ __forceinline__ void settle_few(const Problem& P, const GridTable& T,
     if (lane == 0) j = atomicAdd(&S.taken, 1u);
     j = __shfl_sync(kFull, j, 0);
     if (j >= n) break;
-    settle_own<f32, copied>(P, T, D, mine + j, Vg, scratch, lane, S);
+    settle_own<f32, copied, false>(P, T, D, mine + j, Vg, Team{1, 0, 0, scratch}, lane, S);
   }
+}
+
+// The same by teams of `size` warps. Not inlined: its registers stay out of the
+// column loop.
+template <bool f32, bool copied>
+__device__ __noinline__ void settle_teams(const GridTable T, uint32_t n, const uint64_t* Vg, int size) {
+  GridShared& S = *at_shared<GridShared>(0);
+  const EntryCopy D = S.copy;
+  GridMiss* mine = unit_misses(S);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, at = warp / size;
+  const Team W{size, warp % size, 1 + at, kGridScratchAt + (uint32_t)(at * size * sizeof(SettleScratch))};
+  for (uint32_t j = at; j < n; j += kGridWarps / size)
+    settle_own<f32, copied, true>(S.prob, T, D, mine + j, Vg, W, lane, S);
 }
 
 // Missed columns of this iteration, of the CTAs that listed them (`own` of this
@@ -525,7 +538,7 @@ __device__ bool settle_misses(const Problem& P, const GridTable& T, const EntryC
     if (lane == 0) j = atomicAdd(&taken[me], 1u);
     j = __shfl_sync(kFull, j, 0);
     if (j >= own) break;
-    settle_own<f32, copied>(P, T, D, mine + j, Vg, scratch, lane, S);
+    settle_own<f32, copied, false>(P, T, D, mine + j, Vg, Team{1, 0, 0, scratch}, lane, S);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -583,7 +596,7 @@ __device__ __forceinline__ int32_t grid_iterate(const Problem& P, const GridTabl
     e32 = Entries<uint2, false>{P.rowval, P.lg32};
     e64 = Entries<ulonglong2, false>{P.rowval, f32 ? P.lgx : P.lg};
   }
-  const uint32_t scratch = kGridScratchAt + warp * (uint32_t)sizeof(WarpScratch);
+  const uint32_t scratch = kGridScratchAt + warp * (uint32_t)sizeof(SettleScratch);
   const bool infinite = P.infinite != 0, extra = infinite || P.policy_mode != 0;
   const int n32 = S.n32, n_cols = S.n_cols;
   uint32_t barrier = 0;
@@ -677,7 +690,11 @@ __device__ __forceinline__ int32_t grid_iterate(const Problem& P, const GridTabl
     };
     const uint32_t list = n_miss > kGridFewMisses ? n_miss : 0;
     if (n_miss && !list) {
-      settle_few<f32, copied>(P, T, D, unit_misses(S), n_miss, Vg, scratch, lane, S);
+      const int size = team_size(n_miss, S.unit.max_col, kGridWarps);
+      if (size > 1)
+        settle_teams<f32, copied>(T, n_miss, Vg, size);
+      else
+        settle_few<f32, copied>(P, T, D, unit_misses(S), n_miss, Vg, scratch, lane, S);
       __syncthreads();
       collect();
     }

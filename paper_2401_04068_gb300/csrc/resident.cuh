@@ -338,6 +338,43 @@ __device__ __forceinline__ ulonglong2 settle_pair(const Bounds<f32, 3>& lg, int 
   return ok ? lg[i] : make_ulonglong2(0, 0);
 }
 
+// What a warp needs to settle a column, and what the warps of a team exchange.
+struct SettleScratch {
+  WarpScratch ws;
+  unsigned long long x[2][4];  // by parity of the exchange: this warp's partial results
+  uint32_t pos;                // the team's candidates
+};
+
+// Warps that settle one column together: `size` of them (the first one's scratch
+// at `scratch`, the others' behind it), this one's rank, and a barrier of their own.
+struct Team {
+  int size, rank, bar;
+  uint32_t scratch;
+  __device__ __forceinline__ SettleScratch* of(int r) const {
+    return at_shared<SettleScratch>(scratch + (uint32_t)(r * sizeof(SettleScratch)));
+  }
+  __device__ __forceinline__ void sync() const {
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(32 * size) : "memory");
+  }
+};
+
+// The team size for `n` missed columns of up to `k` entries on `warps` warps. One
+// warp takes 60 cycles for an entry (its passes together) and 6,000 besides, most
+// of it waiting for one instruction after the other, so columns that are fewer
+// than the warps are shared out; a team's exchanges cost about 6,000 more.
+__device__ __forceinline__ int team_size(uint32_t n, int32_t k, int warps) {
+  int best = 1;
+  uint32_t least = (n + warps - 1) / warps * (45u * (uint32_t)k + 4500u);  // (less a quarter: teams have to pay)
+  for (int t = 2; t <= 8 && warps % t == 0; t *= 2) {
+    const uint32_t cost = (n * t + warps - 1) / warps * (60u * (uint32_t)k / t + 12000u);
+    if (cost < least) {
+      least = cost;
+      best = t;
+    }
+  }
+  return best;
+}
+
 // A column whose warm start failed (or that had no hint), by the whole warp: the
 // neighbour check, then the threshold search (the sequence of column_q, to the
 // bit). The passes of column_neighbor and column_search load one entry a lane,
@@ -346,12 +383,42 @@ __device__ __forceinline__ ulonglong2 settle_pair(const Bounds<f32, 3>& lg, int 
 // takes keys only (its key's entries are looked up by a second one) and leaves
 // the key range for the search. Not inlined: the search's registers stay out of
 // the warm pass. `none`: any state that V holds.
-template <bool f32, int gmem, int U, class VA>
+//
+// `team`: by the warps of T, trips dealt round. Their partial results meet in
+// shared memory; sums are exact or saturate alike in any order, and candidates are
+// ordered by entry, so the words are those of one warp. Grid kernel,
+// one warp a column and teams where they pay: cartpole_960 2.54 -> 2.18 ms,
+// cartpole_3840 12.8 -> 11.5, 1,712 states of 657 entries 2.13 -> 1.66. The resident
+// kernel has columns enough for its warps and its column loop slows down beside the
+// second copy of this (4096 pendulum parts 65.2 -> 69.2 ms), so it has one warp each.
+template <bool f32, int gmem, int U, bool team, class VA>
 __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type rows, const Bounds<f32, gmem> lg,
                                                int32_t k, uint64_t rem, const VA V, bool pess, bool neighbor,
-                                               uint64_t vk, uint64_t wacc, uint64_t flt, uint64_t geq, uint32_t scratch,
+                                               uint64_t vk, uint64_t wacc, uint64_t flt, uint64_t geq, const Team T,
                                                int32_t none, int lane, int32_t* hint_out) {
-  WarpScratch* ws = at_shared<WarpScratch>(scratch);
+  WarpScratch* ws = &T.of(0)->ws;
+  const int size = team ? T.size : 1, rank = team ? T.rank : 0;
+  const int step = 32 * size;  // entries from one trip of a warp to its next
+  int parity = 0;
+  if (team && rank == 0 && lane == 0) T.of(0)->pos = 0;
+  // the team's partial results of every warp, one warp's on each of the first lanes
+  const auto exchange = [&](uint64_t& a, uint64_t& b, uint64_t& c, uint64_t& d) {
+    if (lane == 0) {
+      unsigned long long* x = T.of(rank)->x[parity];
+      x[0] = a;
+      x[1] = b;
+      x[2] = c;
+      x[3] = d;
+    }
+    T.sync();
+    const unsigned long long* x = T.of(min(lane, size - 1))->x[parity];
+    a = x[0];
+    b = x[1];
+    c = x[2];
+    d = x[3];
+    parity ^= 1;
+  };
+  const bool peer = lane < size;  // this lane holds a warp's result after an exchange
   const auto key_of = [&](int32_t r) -> uint64_t {
     const uint64_t v = V.at(r);
     return pess ? v : kOne - v;
@@ -359,13 +426,13 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
   const auto value = [&](uint64_t x) { return pess ? x : kOne - x; };
   // calls f(entry, key) for every entry, a lane's in ascending order
   const auto keys = [&](const auto& f) {
-    for (int base = lane; base < k; base += 32 * U) {
+    for (int base = 32 * rank + lane; base < k; base += step * U) {
       int32_t r[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) r[u] = settle_row(rows, base + 32 * u, base + 32 * u < k, none);
+      for (int u = 0; u < U; ++u) r[u] = settle_row(rows, base + step * u, base + step * u < k, none);
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (base + 32 * u < k) f(base + 32 * u, key_of(r[u]));
+        if (base + step * u < k) f(base + step * u, key_of(r[u]));
     }
   };
   if (f32 && neighbor) {
@@ -384,7 +451,16 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
       have = true;
     }
   });
-  if (neighbor && !(down && flt >= kOne) && __any_sync(kFull, have)) {
+  bool some = __any_sync(kFull, have);
+  if (team) {
+    uint64_t h = some ? 1 : 0;
+    if (neighbor) near = down ? warp_max_u64(near) : warp_min_u64(near);
+    cmin = warp_min_u64(cmin);
+    cmax = warp_max_u64(cmax);
+    exchange(cmin, cmax, near, h);
+    some = __any_sync(kFull, peer && h != 0);
+  }
+  if (neighbor && !(down && flt >= kOne) && some) {
     const uint64_t tgt = down ? warp_max_u64(near) : warp_min_u64(near);
     uint64_t gs = 0, ds = 0, dk = 0;
     int first = -1;
@@ -401,13 +477,27 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
         }
       }
     });
-    const uint64_t G = warp_sum_sat(gs), D = warp_sum_u64(ds);
-    const int32_t h = __shfl_sync(kFull, first, __ffs(__ballot_sync(kFull, first >= 0)) - 1);
+    uint64_t G = warp_sum_sat(gs), D = warp_sum_u64(ds);
+    int32_t h = first;
+    if (team) {
+      // of the key's entries the one that a single warp's lowest lane sees first
+      uint64_t c = __reduce_min_sync(kFull, first >= 0 ? ((unsigned)lane << 26) | ((unsigned)first >> 5) : ~0u);
+      dk = warp_sum_u64(dk);
+      exchange(G, D, dk, c);
+      G = warp_sum_sat(peer ? G : 0);
+      D = warp_sum_u64(peer ? D : 0);
+      if (!peer) dk = 0;
+      const unsigned code = __reduce_min_sync(kFull, (unsigned)c);
+      h = (int32_t)(((code & 0x3ffffffu) << 5) | (code >> 26));
+    } else {
+      h = __shfl_sync(kFull, first, __ffs(__ballot_sync(kFull, first >= 0)) - 1);
+    }
     const uint64_t vt = value(tgt);
     if (down) {
       const uint64_t fl = flt - G;
       if (fl < rem) {
         *hint_out = h;
+        if (team) T.sync();  // the scratch is free
         return wacc - D + __umul64hi(vt, rem - fl);
       }
     } else {
@@ -415,6 +505,7 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
       const uint64_t fl = flt + geq;
       if (sat_add(fl, G) >= rem) {
         *hint_out = h;
+        if (team) T.sync();
         return wacc + DK + __umul64hi(vt, rem - fl);
       }
     }
@@ -436,26 +527,31 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
     }
     const int bits = 64 - __clzll((long long)(cmax - cmin));
     const int shift = bits > 6 ? bits - 6 : 0;
-    ws->hl[lane] = 0;
-    ws->hl[lane + 32] = 0;
-    ws->hh[lane] = 0;
-    ws->hh[lane + 32] = 0;
-    ws->hc[lane] = 0;
-    ws->hc[lane + 32] = 0;
-    if (lane == 0) ws->hsat[0] = ws->hsat[1] = 0;
-    __syncwarp();
-    for (int base = lane; base < k; base += 32 * U) {
+    if (!team || rank == 0) {
+      ws->hl[lane] = 0;
+      ws->hl[lane + 32] = 0;
+      ws->hh[lane] = 0;
+      ws->hh[lane + 32] = 0;
+      ws->hc[lane] = 0;
+      ws->hc[lane + 32] = 0;
+      if (lane == 0) ws->hsat[0] = ws->hsat[1] = 0;
+    }
+    if (team)
+      T.sync();
+    else
+      __syncwarp();
+    for (int base = 32 * rank + lane; base < k; base += step * U) {
       int32_t r[U];
       uint64_t g[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int i = base + 32 * u;
+        const int i = base + step * u;
         r[u] = settle_row(rows, i, i < k, none);
         g[u] = settle_pair(lg, i, i < k).y;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        if (base + 32 * u >= k) break;
+        if (base + step * u >= k) break;
         const uint64_t x = key_of(r[u]);
         if (x >= lo && x <= hi) {
           const int b = (int)((x - cmin) >> shift);
@@ -471,7 +567,10 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
         }
       }
     }
-    __syncwarp();
+    if (team)
+      T.sync();
+    else
+      __syncwarp();
     const unsigned sat = ws->hsat[lane >> 4];
     const uint64_t h0 = ((sat >> ((2 * lane) & 31)) & 1u) ? ~0ull
                                                           : (((uint64_t)ws->hh[2 * lane] << 32) | ws->hl[2 * lane]);
@@ -490,7 +589,10 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
     const int b = __shfl_sync(kFull, low ? 2 * lane : 2 * lane + 1, L);
     fb = __shfl_sync(kFull, low ? sat_add(fb, ex) : i0, L);
     const unsigned cnt = ws->hc[b];
-    __syncwarp();
+    if (team)
+      T.sync();  // every warp has read the histogram
+    else
+      __syncwarp();
     lo = cmin + ((uint64_t)b << shift);
     const uint64_t top = lo + ((1ull << shift) - 1ull);
     hi = top < cmax ? top : cmax;
@@ -504,32 +606,42 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
     });
     cmin = warp_min_u64(a);
     cmax = warp_max_u64(z);
+    if (team) {
+      uint64_t u0 = 0, u1 = 0;
+      exchange(cmin, cmax, u0, u1);
+      cmin = warp_min_u64(cmin);
+      cmax = warp_max_u64(cmax);
+    }
   }
   uint64_t acc = 0, gsum = 0;
   unsigned pos = 0;
   int first_cand = -1;
   const unsigned lt = (1u << lane) - 1u;
-  for (int base = 0; base < k; base += 32 * U) {
+  for (int base = 32 * rank; base < k; base += step * U) {
     int32_t r[U];
     ulonglong2 b[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = base + 32 * u + lane;
+      const int i = base + step * u + lane;
       r[u] = settle_row(rows, i, i < k, none);
       b[u] = settle_pair(lg, i, i < k);
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (base + 32 * u >= k) break;
-      const int i = base + 32 * u + lane;
+      if (base + step * u >= k) break;
+      const int i = base + step * u + lane;
       const bool valid = i < k;
       const uint64_t x = key_of(r[u]);
       const bool below = all_below || x < lo;
       const bool cand = valid && !all_below && x >= lo && x <= hi;
       acc = mul_hi_add(value(x), below ? b[u].x + b[u].y : b[u].x, acc);  // past the end: a zero pair
       const unsigned m = __ballot_sync(kFull, cand);
-      if (m && first_cand < 0) first_cand = base + 32 * u + __ffs(m) - 1;
+      if (m && first_cand < 0) first_cand = base + step * u + __ffs(m) - 1;
       if (!uniform) {
+        if (team && m) {
+          if (lane == 0) pos = atomicAdd(&T.of(0)->pos, (unsigned)__popc(m));
+          pos = __shfl_sync(kFull, pos, 0);
+        }
         if (cand) {
           const unsigned at = min(pos + __popc(m & lt), 31u);
           ws->ck[at] = x;
@@ -543,8 +655,18 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
     }
   }
   acc = warp_sum_u64(acc);
+  if (team) {
+    uint64_t f = (unsigned)first_cand, u1 = 0;
+    if (uniform) gsum = warp_sum_sat(gsum);
+    exchange(acc, gsum, f, u1);  // (and every warp's candidates are listed)
+    acc = warp_sum_u64(peer ? acc : 0);
+    if (!peer) gsum = 0;
+    first_cand = (int)__reduce_min_sync(kFull, (unsigned)f);
+    pos = T.of(0)->pos;
+  }
   if (all_below) {
     *hint_out = -1;
+    if (team) T.sync();
     return acc;
   }
   pos = min(pos, 32u);
@@ -552,6 +674,7 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
   if (uniform) {
     const uint64_t g = warp_sum_sat(gsum);
     *hint_out = first_cand >= 0 ? -2 - first_cand : -1;
+    if (team) T.sync();
     return acc + __umul64hi(value(lo), g < r2 ? g : r2);
   }
   __syncwarp();
@@ -562,7 +685,7 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
     uint64_t before = 0;
     for (unsigned j = 0; j < pos; ++j) {
       const uint64_t kj = ws->ck[j];
-      if (kj < ki || (kj == ki && j < (unsigned)lane)) before = sat_add(before, ws->cg[j]);
+      if (kj < ki || (kj == ki && (team ? ws->ci[j] < ws->ci[lane] : j < (unsigned)lane))) before = sat_add(before, ws->cg[j]);
     }
     const uint64_t left = r2 > before ? r2 - before : 0;
     extra = __umul64hi(value(ki), gi < left ? gi : left);
@@ -571,7 +694,10 @@ __device__ __noinline__ uint64_t missed_column(const typename RowsOf<gmem>::type
   const unsigned tm = __ballot_sync(kFull, thr >= 0);
   const int32_t found = tm ? __shfl_sync(kFull, thr, __ffs(tm) - 1) : -1;
   *hint_out = found >= 0 ? -2 - found : -1;
-  __syncwarp();
+  if (team)
+    T.sync();
+  else
+    __syncwarp();
   return acc + warp_sum_u64(extra);
 }
 
@@ -596,19 +722,19 @@ __device__ __forceinline__ void settle_column(const Problem& P, const Columns& C
   if constexpr (shared) {
     const XRows rows{D.rows + c.a * 4u};
     if (f32 && i < n32)
-      q = missed_column<true, 3, kUnitTrips>(rows, Bounds<true, 3>{D.pairs + c.a * 8u, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk,
-                                 c.acc, c.flt, c.geq, scratch, none, lane, &ho);
+      q = missed_column<true, 3, kUnitTrips, false>(rows, Bounds<true, 3>{D.pairs + c.a * 8u, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk,
+                                 c.acc, c.flt, c.geq, Team{1, 0, 0, scratch}, none, lane, &ho);
     else
-      q = missed_column<false, 3, kUnitTrips>(rows, Bounds<false, 3>{(f32 ? D.exact : D.pairs) + c.a * 16u, 0}, c.k, c.rem, V, pess,
-                                  neighbor, vk, c.acc, c.flt, c.geq, scratch, none, lane, &ho);
+      q = missed_column<false, 3, kUnitTrips, false>(rows, Bounds<false, 3>{(f32 ? D.exact : D.pairs) + c.a * 16u, 0}, c.k, c.rem, V, pess,
+                                  neighbor, vk, c.acc, c.flt, c.geq, Team{1, 0, 0, scratch}, none, lane, &ho);
   } else {
     const GRows rows{P.rowval + c.a};
     if (f32 && i < n32)
-      q = missed_column<true, 1, kUnitTrips>(rows, Bounds<true, 1>{P.lg32 + c.a, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk, c.acc,
-                                 c.flt, c.geq, scratch, none, lane, &ho);
+      q = missed_column<true, 1, kUnitTrips, false>(rows, Bounds<true, 1>{P.lg32 + c.a, 32 - c.x}, c.k, c.rem, V, pess, neighbor, vk, c.acc,
+                                 c.flt, c.geq, Team{1, 0, 0, scratch}, none, lane, &ho);
     else
-      q = missed_column<false, 1, kUnitTrips>(rows, Bounds<false, 1>{f32 ? P.lgx + c.x : P.lg + c.a, 0}, c.k, c.rem, V, pess,
-                                  neighbor, vk, c.acc, c.flt, c.geq, scratch, none, lane, &ho);
+      q = missed_column<false, 1, kUnitTrips, false>(rows, Bounds<false, 1>{f32 ? P.lgx + c.x : P.lg + c.a, 0}, c.k, c.rem, V, pess,
+                                  neighbor, vk, c.acc, c.flt, c.geq, Team{1, 0, 0, scratch}, none, lane, &ho);
   }
   if (lane == 0) {
     const uint32_t lc = c.lc & ~kMoving;

@@ -138,6 +138,9 @@ GRID = {
     "scattered": lambda: _lengths(3001, (60, 61, 190, 256, 257, 31), 13),
     "wide": lambda: _lengths(2100, (1279, 1280, 1281, 40, 1900), 14),
     "loose": lambda: _lengths(2500, (90, 200, 33), 15, wide=True),
+    # few columns to a CTA: its misses are settled by teams of warps
+    "few_long": lambda: _lengths(900, (500, 700, 333, 899), 16),
+    "few_loose": lambda: _lengths(700, (640, 321), 17, wide=True),
 }
 
 
