@@ -301,8 +301,8 @@ struct ResidentPlan {
 constexpr int kGridMaxChunks = 16;  // per CTA
 // Models of this many transitions or more keep the per-iteration direct kernel:
 // there the transitions have left L2 when a missed column is settled (pimdp_2,
-// 48 M: grid kernel 53.1 ms and 42.8 ms on 32-bit storage, direct 54.8 and 40.3;
-// 29 M in two actions: 24.8 against 29.6).
+// 48 M: grid kernel 53.1 ms and 41.4 ms on 32-bit storage, direct 54.8 and 40.3;
+// 29 M, columns of 716: 24.8 against 29.6).
 constexpr int64_t kGridMostEntries = 32000000;
 struct GridWindow {
   int32_t w0, len;  // states [w0, w0 + len)

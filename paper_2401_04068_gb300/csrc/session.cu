@@ -504,8 +504,16 @@ imdp_status Session::plan_grid(cudaStream_t st) {
   whole = GridPlan{};
   const DevModel* m = models[0];
   GridCut cut;
-  if (L.tiny_ok || resident.n_units > 0 || count != 1 || !plan_grid_unit(m, fixed_h.data(), grid, cut)) return IMDP_OK;
   const bool f32 = m->lg32 != nullptr;
+  if (L.tiny_ok || resident.n_units > 0 || count != 1) return IMDP_OK;
+  // Many long columns stay on the direct kernel: it settles a missed column while
+  // its entries are still in L1 and L2 (100 iterations, direct and grid kernel, ms:
+  // 48,000 columns of 500 entries 21.0 / 19.1, 56,000 of 376 16.7 / 16.5, 84,000 of
+  // 376 20.2 / 20.8; on 32-bit storage 42,000 of 376 8.2 / 7.0, 48,000 of 500 15.7 /
+  // 15.9, 90,000 of 300 14.5 / 16.4). Against the ring kernel, which short columns
+  // take otherwise, it gains at any number (126,000 of 230 20.5 / 17.5).
+  if (m->nnz >= (int64_t)kRuleLongColumn * m->n_cols && m->n_cols > (f32 ? 45000 : 56000)) return IMDP_OK;
+  if (!plan_grid_unit(m, fixed_h.data(), grid, cut)) return IMDP_OK;
   const size_t need = grid_bytes(cut, f32), all = need + 64 + 20 * (size_t)cut.entries;
   whole.smem = (uint32_t)((all <= kResidentSmem ? all : need) + 15) & ~15u;
   whole.grid = whole.steal_ctas = grid;
