@@ -354,9 +354,10 @@ def run_ours(args, rank, world, local_rank):
     launch_ms = kernel_ms / max(1, launches)  # per launched iteration (includes any past convergence)
     n_tiles, n_wide, wide_entries = g.imdp_session_plan(sess)
     wide_share = wide_entries / max(1, m.nnz)
-    kernel = "bellman_wide_kernel" if wide_share > 0.5 else KERNEL_NAMES.get(launch["kernel"], "bellman_step_kernel")
+    by_rule = launch["chosen_by"] == "rule"
+    kernel = "bellman_wide_kernel" if wide_share > 0.5 and not by_rule else kernel_name(launch)
     achieved = alg_bytes / (launch_ms / 1e3) / 1e9
-    traffic = recorded_traffic(args.workload + ("" if args.dtype == "f64" else ":f32"))
+    traffic = None if by_rule else recorded_traffic(args.workload + ("" if args.dtype == "f64" else ":f32"))
     cfg = workload_config(args.workload, m, args.horizon)
     metric = METRIC
     if args.infinite:
@@ -391,10 +392,11 @@ def run_ours(args, rank, world, local_rank):
                      "algorithmic_bytes_per_launch": alg_bytes, "avg_launch_ms": launch_ms,
                      "plan": {"tiles": n_tiles, "wide_states": n_wide, "wide_entry_share": wide_share,
                               "launch": launch},
-                     "timing": "CUDA events around each step's launches (both step kernels) / launches"},
+                     "timing": "CUDA events around each step's launches (both step kernels) / iterations"},
         "clocks": clk,
-        # step kernels (two per iteration when the model has wide states) + one value-reset kernel per step
-        "gpu_launches": int(launches * (2 if n_wide > 0 else 1) + args.steps),
+        # step kernels (per iteration, two when the model has wide states; by rule at least one a step) + one
+        # value-reset kernel per step
+        "gpu_launches": counted_launches(launch, int(launches), args.steps, 2 if n_wide > 0 else 1) + args.steps,
         "e2e": e2e,
     }
     if world == 1 and not args.no_cpu_baseline:
@@ -429,15 +431,16 @@ def parse_launch(text: str) -> dict:
     return out
 
 
-def apply_launch(g, sess, args, stream, tune_iters: int) -> dict:
+def apply_launch(g, sess, args, stream, tune_iters: int, default: str = "off") -> dict:
     """Launch configuration of the timed session: explicit (--launch), the
     autotuner's cached or freshly timed choice (--tune), or the rule."""
+    tune = args.tune or default
     if args.launch:
         g.imdp_session_set_launch(sess, stream=stream, **parse_launch(args.launch))
         how = "explicit"
-    elif args.tune != "off":
+    elif tune != "off":
         cache = args.tune_cache or TUNE_CACHE
-        if args.tune == "fresh":
+        if tune == "fresh":
             cache = None
         _, ms = g.imdp_session_autotune(sess, tune_iters, cache, stream=stream)
         how = "autotuner (cached choice)" if ms == 0.0 else f"autotuner (timed now: {ms:.4f} ms per iteration)"
@@ -445,7 +448,22 @@ def apply_launch(g, sess, args, stream, tune_iters: int) -> dict:
         how = "rule"
     out = g.imdp_session_get_launch(sess)
     out["chosen_by"] = how
+    if how == "rule":
+        out["note"] = ("step calls of 4 or more iterations are one launch of the resident or grid kernel where the "
+                       "rule plans one; the fields are those of the per-iteration kernel otherwise")
     return out
+
+
+def kernel_name(launch) -> str:
+    if launch["chosen_by"] == "rule" and launch["kernel"] != 3:
+        return "bellman_cluster_kernel or bellman_grid_kernel, by rule"
+    return KERNEL_NAMES.get(launch["kernel"], "bellman_step_kernel")
+
+
+def counted_launches(launch, iterations: int, calls: int, per_iteration: int) -> int:
+    """Step-kernel launches: by rule at least one per step call (iterations share
+    launches), else every iteration's."""
+    return calls if launch["chosen_by"] == "rule" else iterations * per_iteration
 
 
 def _gpu_setup(rank, world, local_rank):
@@ -478,7 +496,7 @@ def run_polished(args, rank, world, local_rank):
     launches = []
     for mdl in (m32, m64):  # the autotuner's configuration of each storage
         s_ = g.imdp_session_create([mdl], [spec], stream=stream)
-        launches.append(apply_launch(g, s_, args, stream, 64))
+        launches.append(apply_launch(g, s_, args, stream, 64, "cache"))
         s_.close()
     Vd = torch.empty(m.n_states, dtype=torch.float64, device=dev)
     res = torch.empty(m.n_states, dtype=torch.float64, device=dev)
@@ -610,9 +628,9 @@ def run_uneven(args, rank, world, local_rank):
                    "generation_s": round(gen_s, 1), "parallelism": "replicas", "launch": launch},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "traffic": None, "peak_kind": peak_kind,
-                     "kernel": KERNEL_NAMES.get(launch["kernel"], "bellman_step_kernel"),
+                     "kernel": kernel_name(launch),
                      "note": "algorithmic bytes of every running problem summed over the step's launches"},
-        "clocks": clk, "gpu_launches": int(launches + args.steps), "e2e": None,
+        "clocks": clk, "gpu_launches": counted_launches(launch, int(launches), args.steps, 1) + args.steps, "e2e": None,
     }
     print(json.dumps(out), flush=True)
 
@@ -867,7 +885,7 @@ def run_state_sharded(args, rank, world, local_rank):
     lengths = np.diff(bounds)
     runner = SliceRunner(m, bounds, rank, dict(horizon=args.horizon, reach=m.goal), dtype)
     # each slice's session takes the autotuner's configuration for its own shape
-    launch = apply_launch(g, runner.session, args, None, min(args.horizon, 200))
+    launch = apply_launch(g, runner.session, args, None, min(args.horizon, 200), "cache")
 
     def one_step():
         runner.reset()
@@ -930,8 +948,9 @@ def main():
     ap.add_argument("--f32-budget", type=float, default=0.0,
                     help="32-bit storage: per-iteration error budget of the correction stage (0: library default)")
     ap.add_argument("--launch", default="", help="explicit launch configuration, e.g. ring:24, direct:4:1024 or slice:4")
-    ap.add_argument("--tune", default="cache", choices=["cache", "fresh", "off"],
-                    help="autotuner: cached choice (timing only shapes missing from the cache), time now, or rule")
+    ap.add_argument("--tune", default="", choices=["", "cache", "fresh", "off"],
+                    help="off: by rule (the default, but for polished and state-sharded queries); autotuner of the per-iteration kernels: cached choice (timing only shapes "
+                         "missing from the cache), or time now")
     ap.add_argument("--tune-cache", default="", help="autotuner cache file (default: the package's GB300 table)")
     ap.add_argument("--requests", type=int, default=2000, help="served workload: number of requests")
     ap.add_argument("--rate", type=float, default=2000.0, help="served workload: Poisson arrival rate per second")
