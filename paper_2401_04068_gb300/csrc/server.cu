@@ -87,10 +87,14 @@ class Arena {
 // Per-iteration launches of the direct kernel take what the launch and its last
 // wave take, 500 times over, while a few large requests hold most of the work
 // (64 requests of 50 to 4000 states, 100 to 500 iterations: 49.3 ms,
-// 30.2 with shared launches; 19 requests 20.6 and 10.1). Bound by the misses of the
-// first iterations (a launch of 2 ms of steady iterations takes 6) and by 4 ms of
-// admission and results on the host.
+// 26.5 with shared launches; 1000 requests/s: p50 34 ms and 11 to 16). Bound by the
+// misses of the first iterations and by 4 ms of admission and results on the host.
 constexpr int32_t kGuessedIterations = 200;
+// Thresholds still move in a request's first iterations and most columns miss: a
+// launch planned for 2 ms without this took 5.9 with new requests in it, and the
+// CTAs of the others waited (the burst of 64 above: 30.2 ms, 26.5 with it).
+constexpr int32_t kEarlyIterations = 30;
+constexpr double kEarlyCost = 3.0;
 // Transitions (and 40 for a column) an SM takes per second: the grid kernel's
 // rate on models of 100 and more transitions a column.
 constexpr double kEntriesPerSecond = 2.4e9;
@@ -124,6 +128,18 @@ struct Request {
     const int32_t cap = spec.infinite_time ? (spec.horizon > 0 ? spec.horizon : 1000000) : spec.horizon;
     const int32_t n = std::max(cap - k, 1);
     return spec.infinite_time ? std::min(n, kGuessedIterations) : n;
+  }
+  // `n` iterations from `k` on, the first ones of a request counted several times
+  static double weighted(int32_t k, double n) {
+    const double early = std::max(0.0, std::min(n, (double)(kEarlyIterations - k)));
+    return n + (kEarlyCost - 1.0) * early;
+  }
+  double work_left() const { return weighted(k, left()); }
+  // how many iterations make a weighted number of them (at least)
+  int32_t iterations(double w) const {
+    const double early = std::max(0, kEarlyIterations - k);
+    const double n = w <= early * kEarlyCost ? w / kEarlyCost : early + (w - early * kEarlyCost);
+    return (int32_t)std::min<double>(left(), std::max(1.0, std::ceil(n - 1e-9)));
   }
   double seconds(int ctas) const {
     const double work = (double)model->nnz + 40.0 * model->n_cols;
@@ -392,7 +408,7 @@ struct Server {
     std::vector<double> load;
     int used = 0;
     for (Request* r : rs) {  // longest first
-      const double n = r->left(), one = n * r->seconds(1);
+      const double n = r->work_left(), one = n * r->seconds(1);
       if (r->least == 1 && one <= T) {
         size_t b = 0;
         while (b < load.size() && load[b] + one > T) ++b;
@@ -432,15 +448,18 @@ struct Server {
     const bool f32 = !rs.empty() && rs[0]->model->lg32;
     for (const Request* r : rs)
       if ((r->model->lg32 != nullptr) != f32 || r->model->nnz >= kGridMostEntries) return false;
-    if (rs.empty()) return false;
+    // more requests than that would mostly follow one another on single CTAs, where
+    // every CTA waits for the one with the most new requests (2000 requests/s, 360
+    // running: 0.88e11 transition-updates/s shared, 0.89 to 0.96e11 per iteration)
+    if (rs.empty() || (int)rs.size() > grid / 2) return false;
     std::stable_sort(rs.begin(), rs.end(), [](const Request* a, const Request* b) {
-      return a->left() * a->seconds(1) > b->left() * b->seconds(1);
+      return a->work_left() * a->seconds(1) > b->work_left() * b->seconds(1);
     });
     Share best, now;
     std::vector<GridCut> cuts;
     for (int attempt = 0;; ++attempt) {
       double hi = 0.0, lo = 0.0;
-      for (const Request* r : rs) hi += r->left() * r->seconds(1);
+      for (const Request* r : rs) hi += r->work_left() * r->seconds(1);
       if (!share(rs, hi, grid, best)) return false;  // the least that the requests need is too much
       for (int i = 0; i < 20; ++i) {
         const double mid = 0.5 * (lo + hi);
@@ -464,7 +483,7 @@ struct Server {
       for (auto& b : best.bins) {
         // the one that ends first runs first
         std::stable_sort(b.begin(), b.end(), [](const Request* x, const Request* y) {
-          return x->left() * x->seconds(1) < y->left() * y->seconds(1);
+          return x->work_left() * x->seconds(1) < y->work_left() * y->seconds(1);
         });
         for (Request* r : b) cut(r, 1);
       }
@@ -582,7 +601,7 @@ struct Server {
     auto per = [&](int u) { return g_reqs[u]->seconds(g_units[u].ctas); };
     for (size_t c = 0; c < g_work.size(); ++c) {
       for (int u = g_work[c].x; u < g_work[c].y; ++u)
-        if (g_reqs[u]) left[c] += g_reqs[u]->left() * per(u);
+        if (g_reqs[u]) left[c] += g_reqs[u]->work_left() * per(u);
       longest = std::max(longest, left[c]);
     }
     const double f = longest > kQuantumSeconds ? kQuantumSeconds / longest : 1.0;
@@ -593,9 +612,9 @@ struct Server {
       for (int u = g_work[c].x; u < g_work[c].y && (w.y == 0 || budget > 1e-7); ++u) {
         Request* r = g_reqs[u];
         if (!r) continue;
-        const int32_t n = (int32_t)std::min<double>(r->left(), std::ceil(budget / per(u) - 1e-9));
-        g_units[u].iters = std::max(n, 1);
-        budget -= n * per(u);
+        const int32_t n = r->iterations(budget / per(u));
+        g_units[u].iters = n;
+        budget -= Request::weighted(r->k, n) * per(u);
         if (w.y == 0) w.x = u;
         w.y = u + 1;
       }
