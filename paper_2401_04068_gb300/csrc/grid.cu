@@ -22,8 +22,8 @@
 // The warm start streams at 0.8 of the copy bandwidth (pimdp_2, 300,000 cycles
 // an iteration); a missed column takes 15,000 to 45,000 cycles of a warp, which
 // is what bounds the first iterations of every model. Measured, K = 200 or to
-// convergence: 20,000 states of 24 scattered transitions 3.6 -> 1.75 ms,
-// cartpole_960 4.9 -> 2.5, harrier 43.7 -> 36.2, cartpole_3840 13.7 -> 13.0.
+// convergence: 20,000 states of 24 scattered transitions 3.6 -> 1.27 ms,
+// cartpole_960 4.8 -> 2.1, harrier 44.1 -> 34.5, cartpole_3840 13.7 -> 11.4.
 #include <cuda_runtime.h>
 
 #include <algorithm>

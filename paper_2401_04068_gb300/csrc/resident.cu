@@ -16,8 +16,8 @@
 // storage: 55 % issue slots busy, 7 TB/s from L2, DRAM 3 %); a transition costs
 // 32 warp instructions per 32 lanes, a warp's four columns 290 more. Measured
 // against the per-iteration kernels, K = 200: those 4096 parts 115 -> 66 ms
-// (32-bit storage 117 -> 68), 256 problems of up to 961 states and horizons from
-// 100 to 500 137 -> 82 ms, one problem of 241 states 2.8 -> 1.0 ms per query.
+// (32-bit storage 117 -> 66), 256 problems of up to 961 states and horizons from
+// 100 to 500 126 -> 70 ms, one problem of 241 states 2.6 -> 0.95 ms per query.
 //
 // Within a CTA an iteration has three phases: the warm start of the CTA's
 // columns by groups of lanes (longest columns first, so the columns that share
