@@ -395,6 +395,8 @@ __global__ void __launch_bounds__(NT, MINB) bellman_cluster_kernel(StepLaunch L,
   A.rank = rank;
   A.single = R.single;
 
+  // shared memory of another CTA may be written only once that CTA has started
+  cluster_sync(size);
   for (int j = 0;; ++j) {
     // the next part, taken by rank 0 for the whole cluster
     if (rank == 0 && tid == 0) {
