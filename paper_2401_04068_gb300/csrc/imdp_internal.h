@@ -21,6 +21,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/imdp.h"
+#include "buffers.h"
 
 namespace imdp {
 
@@ -475,14 +476,14 @@ struct Session {
   bool graph_stalled = false;  // captured while the failure-detection test hook was on
   int64_t launches = 0;
   int64_t launched_since_reset = 0;
-  std::vector<void*> allocs;
-  // small buffers lie behind one another in slabs (among `allocs`): most of a
-  // small query's creation and destruction was a driver call per buffer
-  unsigned char* slab = nullptr;
-  size_t slab_left = 0;
+  Buffers mem{get_memory, put_memory};
+  // the buffers of the installed launch plan
+  Buffers::Plan tiles_mem, wide_mem, items_mem, item_end_mem, win_mem;
 
+  static void* get_memory(size_t bytes);
+  static void put_memory(void* p);
   ~Session();
-  template <class T> T* alloc(size_t n);
+  template <class T> T* alloc(size_t n) { return (T*)mem.alloc(n * sizeof(T)); }
   static imdp_status create(const std::vector<DevModel*>& ms, const std::vector<const imdp_spec*>& specs,
                             const int32_t* want_policy, cudaStream_t st, Session** out);
   imdp_status reset(cudaStream_t st);

@@ -52,9 +52,6 @@ uint64_t eps_to_fixed(double eps) {
 
 constexpr int kGraphChunk = 16;
 
-// Device buffers of up to kSlabMost bytes share allocations of kSlab bytes.
-constexpr size_t kSlab = 256 * 1024, kSlabMost = 32 * 1024;
-
 // One problem's values in read_all: its words, and where they go.
 struct ExportItem {
   const uint64_t* V;
@@ -128,29 +125,16 @@ imdp_status check_spec(const DevModel* m, const imdp_spec* sp) {
 Session::~Session() {
   if (graph) cudaGraphExecDestroy(graph);
   side.destroy();
-  for (void* p : allocs) cudaFree(p);
 }
 
-template <class T>
-T* Session::alloc(size_t n) {
-  const size_t bytes = (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~size_t(255);
-  const bool small = bytes <= kSlabMost;
-  if (!small || bytes > slab_left) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, small ? kSlab : bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    allocs.push_back(p);
-    if (!small) return (T*)p;
-    slab = (unsigned char*)p;
-    slab_left = kSlab;
-  }
-  T* t = (T*)slab;
-  slab += bytes;
-  slab_left -= bytes;
-  return t;
+void* Session::get_memory(size_t bytes) {
+  void* p = nullptr;
+  if (cudaMalloc(&p, bytes) == cudaSuccess) return p;
+  cudaGetLastError();
+  return nullptr;
 }
+
+void Session::put_memory(void* p) { cudaFree(p); }
 
 imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<const imdp_spec*>& specs,
                             const int32_t* want_policy, cudaStream_t st, Session** out) {
@@ -561,24 +545,16 @@ imdp_status Session::plan_grid(cudaStream_t st) {
 
 imdp_status Session::install_plan(const std::vector<Tile>& tl, const std::vector<int2>& wl, cudaStream_t st,
                                   bool slice) {
-  auto release = [&](void* p) {
-    const auto it = std::find(allocs.begin(), allocs.end(), p);
-    if (!p || it == allocs.end()) return;  // (part of a slab: freed with the session)
-    allocs.erase(it);
-    cudaFree(p);
-  };
   cudaError_t e = cudaStreamSynchronize(st);  // launches in flight may still read the old plan
   if (e != cudaSuccess) return cuda_status(e, "session plan");
-  release(tiles);
-  release(wide);
-  release(items);
-  release(tile_item_end);
-  release(win_cnt);
+  mem.drop(items_mem);
+  mem.drop(item_end_mem);
+  mem.drop(win_mem);
   items = nullptr;
   tile_item_end = nullptr;
   win_cnt = nullptr;
-  tiles = alloc<Tile>(tl.size());
-  wide = alloc<int2>(wl.size());
+  tiles = (Tile*)mem.refit(tiles_mem, sizeof(Tile) * tl.size());
+  wide = (int2*)mem.refit(wide_mem, sizeof(int2) * wl.size());
   if (!tiles || !wide) { set_error("device allocation failed (tile plan)"); return IMDP_ENOMEM; }
   // slice kernel: one work item per slice of every window (tile), in tile order
   std::vector<int2> it;
@@ -589,9 +565,9 @@ imdp_status Session::install_plan(const std::vector<Tile>& tl, const std::vector
       for (int32_t g = tl[t].x0; g < tl[t].x1; ++g) it.push_back(make_int2((int32_t)t, g));
       tend[t] = (int32_t)it.size();
     }
-    items = alloc<int2>(it.size());
-    tile_item_end = alloc<int32_t>(tend.size());
-    win_cnt = alloc<unsigned int>(tl.size());
+    items = (int2*)mem.refit(items_mem, sizeof(int2) * it.size());
+    tile_item_end = (int32_t*)mem.refit(item_end_mem, sizeof(int32_t) * tend.size());
+    win_cnt = (unsigned int*)mem.refit(win_mem, sizeof(unsigned int) * tl.size());
     if (!items || !tile_item_end || !win_cnt) { set_error("device allocation failed (slice plan)"); return IMDP_ENOMEM; }
     if (!it.empty()) e = cudaMemcpyAsync(items, it.data(), sizeof(int2) * it.size(), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess && !tend.empty())
