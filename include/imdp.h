@@ -357,6 +357,25 @@ IMDP_API imdp_status imdp_session_set_launch(imdp_session* s, const imdp_launch_
 /* The configuration the session's launches use, with every field resolved by
  * the rule where the set configuration left it open. */
 IMDP_API imdp_status imdp_session_get_launch(const imdp_session* s, imdp_launch_config* cfg);
+/* What a step call of `n_iters` iterations runs (host-only query; no counterpart
+ * in the paper):
+ *   kernel     1 ring, 2 direct, 3 single CTA, 4 slice (imdp_launch_config), or by
+ *              rule 5 resident, 6 grid
+ *   launches   launches of Bellman kernels in the call
+ *   and for the resident and the grid kernel (0 for the others):
+ *   units      problems, or parts of one problem, that CTAs share
+ *   cluster    CTAs that work on one unit together
+ *   ctas       CTAs of a launch
+ *   threads    threads of a CTA
+ *   group      lanes that share a column's warm start
+ *   copied     1: the transitions stay in shared memory
+ * IMDP_EINVAL for NULL or n_iters < 1. */
+typedef struct {
+  int32_t kernel;
+  int64_t launches;
+  int32_t units, cluster, ctas, threads, group, copied;
+} imdp_step_route;
+IMDP_API imdp_status imdp_session_step_route(const imdp_session* s, int32_t n_iters, imdp_step_route* route);
 /* The session's current tile plan (it follows the launch configuration's
  * tile_entries and wide_col): tiles streamed by the tiled kernels (windows of
  * the slice layout for the slice kernel), wide states and their transitions.
@@ -506,6 +525,10 @@ IMDP_API imdp_status imdp_server_set_launch(imdp_server* s, const imdp_launch_co
  * output may be NULL. Thread-safe. */
 IMDP_API imdp_status imdp_server_stats(imdp_server* s, double* device_ms, double* wall_ms, int64_t* chunks,
                                        double* mean_requests);
+/* Bellman launches since the server's creation: `shared` launches of the grid
+ * kernel (by rule, all running requests in each) and `per_iteration` ones. Any
+ * output may be NULL. Thread-safe. */
+IMDP_API imdp_status imdp_server_launches(imdp_server* s, int64_t* shared, int64_t* per_iteration);
 /* Queue a request; returns at once with a ticket. IMDP_ENOMEM if the request
  * alone exceeds the budget, IMDP_EBUSY if the queue is full. */
 IMDP_API imdp_status imdp_server_submit(imdp_server* s, imdp_model* m, const imdp_spec* spec, uint64_t* ticket);

@@ -35,7 +35,8 @@ EXPORTED = [
     "imdp_session_checkpoint", "imdp_session_restore",
     "imdp_session_set_launch", "imdp_session_get_launch", "imdp_session_autotune", "imdp_session_plan",
     "imdp_create_csc_f32", "imdp_model_exact_columns", "imdp_session_residual", "imdp_session_stop_threshold",
-    "imdp_server_set_launch", "imdp_server_stats", "imdp_value_iteration_polished",
+    "imdp_server_set_launch", "imdp_server_stats", "imdp_value_iteration_polished", "imdp_session_step_route",
+    "imdp_server_launches",
 ]
 
 
@@ -52,7 +53,16 @@ class imdp_launch_config(C.Structure):
         return {f: int(getattr(self, f)) for f, _ in self._fields_}
 
 
+class imdp_step_route(C.Structure):
+    _fields_ = [("kernel", C.c_int32), ("launches", C.c_int64)] + [
+        (f, C.c_int32) for f in ("units", "cluster", "ctas", "threads", "group", "copied")]
+
+    def as_dict(self):
+        return {f: int(getattr(self, f)) for f, _ in self._fields_}
+
+
 KERNEL_RULE, KERNEL_RING, KERNEL_DIRECT, KERNEL_TINY, KERNEL_SLICE = 0, 1, 2, 3, 4
+KERNEL_RESIDENT, KERNEL_GRID = 5, 6  # by rule only (imdp_step_route)
 
 
 class ImdpError(RuntimeError):
@@ -136,6 +146,8 @@ def load(path: Optional[str] = None):
     lib.imdp_session_get_launch.argtypes = [vp, C.POINTER(imdp_launch_config)]
     lib.imdp_session_plan.argtypes = [vp, C.POINTER(C.c_int32), C.POINTER(C.c_int32), C.POINTER(C.c_int64)]
     lib.imdp_server_set_launch.argtypes = [vp, C.POINTER(imdp_launch_config)]
+    lib.imdp_session_step_route.argtypes = [vp, C.c_int32, C.POINTER(imdp_step_route)]
+    lib.imdp_server_launches.argtypes = [vp, C.POINTER(C.c_int64), C.POINTER(C.c_int64)]
     lib.imdp_server_stats.argtypes = [vp, C.POINTER(C.c_double), C.POINTER(C.c_double), C.POINTER(C.c_int64),
                                       C.POINTER(C.c_double)]
     lib.imdp_session_residual.argtypes = [vp, C.c_int32, C.c_int32, C.c_int32, C.c_int32, vp, vp]
@@ -461,6 +473,13 @@ def imdp_session_get_launch(s: Session) -> dict:
     return cfg.as_dict()
 
 
+def imdp_session_step_route(s: Session, n_iters: int) -> dict:
+    """The kernel, launches and shape that a step call of ``n_iters`` iterations takes."""
+    r = imdp_step_route()
+    _check(load().imdp_session_step_route(C.c_void_p(s.handle), int(n_iters), C.byref(r)), "imdp_session_step_route")
+    return r.as_dict()
+
+
 def imdp_session_residual(s: Session, index: int, k: int, s0: int, s1: int, dst, stream=None):
     """max |V_k - V_{k-1}| over states [s0, s1) (raw word) into one device word ``dst``."""
     _check(load().imdp_session_residual(C.c_void_p(s.handle), int(index), int(k), int(s0), int(s1), _ptr(dst),
@@ -544,6 +563,13 @@ def imdp_server_stats(server: Server) -> dict:
     _check(load().imdp_server_stats(C.c_void_p(server.handle), C.byref(d), C.byref(w), C.byref(c), C.byref(r)),
            "imdp_server_stats")
     return dict(device_ms=d.value, wall_ms=w.value, chunks=c.value, mean_requests=r.value)
+
+
+def imdp_server_launches(server: Server) -> dict:
+    """Launches of the grid kernel (requests share them) and per-iteration ones."""
+    a, b = C.c_int64(0), C.c_int64(0)
+    _check(load().imdp_server_launches(C.c_void_p(server.handle), C.byref(a), C.byref(b)), "imdp_server_launches")
+    return dict(shared=a.value, per_iteration=b.value)
 
 
 def imdp_server_submit(server: Server, model: Model, spec) -> int:

@@ -196,6 +196,42 @@ IMDP_API imdp_status imdp_session_get_launch(const imdp_session* s, imdp_launch_
   return IMDP_OK;
 }
 
+IMDP_API imdp_status imdp_session_step_route(const imdp_session* s, int32_t n_iters, imdp_step_route* route) {
+  set_error("");
+  if (!s || !s->s || !route) { set_error("NULL session or route"); return IMDP_EINVAL; }
+  if (n_iters < 1) { set_error("n_iters must be >= 1"); return IMDP_EINVAL; }
+  const Session* S = s->s;
+  std::memset(route, 0, sizeof(*route));
+  route->kernel = S->step_kernel(n_iters);
+  const ResidentPlan& R = S->resident;
+  const int32_t most = S->launch_iterations();
+  switch (route->kernel) {
+    case kKernelTiny:
+      route->launches = 1;
+      break;
+    case kKernelResident:
+      route->launches = (n_iters + (int64_t)most - 1) / most;
+      route->units = R.n_units;
+      route->cluster = R.cluster;
+      route->ctas = R.clusters * R.cluster;
+      route->threads = R.threads;
+      route->group = R.group;
+      route->copied = S->copied ? 1 : 0;
+      break;
+    case kKernelGrid:
+      route->launches = (n_iters + (int64_t)most - 1) / most;
+      route->units = 1;
+      route->cluster = route->ctas = S->whole.grid;
+      route->threads = kGridThreads;
+      route->group = S->whole.group;
+      route->copied = S->copied ? 1 : 0;
+      break;
+    default:  // a tiled kernel, and the wide states' beside it
+      route->launches = (int64_t)n_iters * (S->n_wide > 0 ? 2 : 1);
+  }
+  return IMDP_OK;
+}
+
 IMDP_API imdp_status imdp_session_plan(const imdp_session* s, int32_t* n_tiles, int32_t* n_wide,
                                       int64_t* wide_entries) {
   set_error("");

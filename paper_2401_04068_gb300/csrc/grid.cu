@@ -35,7 +35,6 @@ namespace imdp {
 
 namespace {
 
-constexpr int kGridThreads = 768;
 constexpr int kGridWarps = kGridThreads / 32;
 // Misses that a CTA settles by itself, two rounds of its warps; more are listed
 // for all CTAs, which costs two more barriers.

@@ -188,7 +188,8 @@ struct StepControl {
 
 // Launch configuration of the Bellman step (per session; chosen by rule or by
 // the autotuner). Zero fields mean "by rule".
-enum : int32_t { kKernelRule = 0, kKernelRing = 1, kKernelDirect = 2, kKernelTiny = 3, kKernelSlice = 4 };
+enum : int32_t { kKernelRule = 0, kKernelRing = 1, kKernelDirect = 2, kKernelTiny = 3, kKernelSlice = 4,
+                 kKernelResident = 5, kKernelGrid = 6 };  // the last two by rule only
 // A session of one problem this small runs all its iterations in one launch of
 // one CTA, with the model and values in shared memory (bellman_tiny_kernel).
 constexpr int32_t kTinyMaxStates = 1024, kTinyMaxCols = 1024, kTinyMaxEntries = 4096;
@@ -388,6 +389,7 @@ size_t grid_bytes(const GridCut& c, bool f32);
 bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut& out);
 cudaError_t grid_prepare(const GridPlan& R);
 cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t n_iters, cudaStream_t st);
+constexpr int kGridThreads = 768;  // of a CTA
 // CTAs of the persistent tiled kernel: one per SM.
 int bellman_grid();
 // The configuration a launch of `L` with `cfg` (nullable) actually uses: kernel,
@@ -468,6 +470,10 @@ struct Session {
   imdp_status plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st);
   GridPlan whole{};  // the grid kernel's (n_units 0: not taken)
   imdp_status plan_grid(cudaStream_t st);
+  bool copied = false;  // the plan above keeps the transitions in shared memory
+  // The kernel that a step call of n iterations takes, and how many of them one launch runs.
+  int32_t step_kernel(int32_t n) const;
+  int32_t launch_iterations() const;
   SideStream side;  // created when the session has both tiles and wide states
   LaunchConfig cfg;  // launch configuration (rule, set_launch or the autotuner)
   StepLaunch L{};

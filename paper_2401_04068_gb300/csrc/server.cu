@@ -193,7 +193,7 @@ struct Server {
   // events around each chunk's launches), wall time of the loop while requests
   // were running, chunks, and requests in the launches summed over chunks
   double st_device_ms = 0.0, st_wall_ms = 0.0, st_slots = 0.0;
-  int64_t st_chunks = 0;
+  int64_t st_chunks = 0, st_shared = 0;  // all launches (of chunks), and those of the grid kernel
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 
   explicit Server(size_t budget) : arena(budget) {}
@@ -803,6 +803,7 @@ struct Server {
         std::lock_guard<std::mutex> lk(mu);
         st_device_ms += dev_ms;
         st_chunks += 1;
+        st_shared += grid_kernel ? 1 : 0;
         st_slots += active;
         // wall time from this chunk's launches to the end of its retirements;
         // admission and table uploads before the next chunk are added there
@@ -842,6 +843,16 @@ imdp_status imdp_server_stats(imdp_server* srv, double* device_ms, double* wall_
   if (wall_ms) *wall_ms = S->st_wall_ms;
   if (chunks) *chunks = S->st_chunks;
   if (mean_requests) *mean_requests = S->st_chunks ? S->st_slots / (double)S->st_chunks : 0.0;
+  return IMDP_OK;
+}
+
+imdp_status imdp_server_launches(imdp_server* srv, int64_t* shared, int64_t* per_iteration) {
+  set_error("");
+  if (!srv || !srv->s) { set_error("NULL server"); return IMDP_EINVAL; }
+  Server* S = srv->s;
+  std::lock_guard<std::mutex> lk(S->mu);
+  if (shared) *shared = S->st_shared;
+  if (per_iteration) *per_iteration = (S->st_chunks - S->st_shared) * S->chunk;
   return IMDP_OK;
 }
 

@@ -447,7 +447,8 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
       // latency in its iterations; pendulum_240 alone 1.03 ms against 1.11). With
       // many units the wider clusters that takes cost more than it saves.
       const size_t all = need + 64 + (size_t)rank_entries * 20;
-      resident.smem = (uint32_t)(n_units == 1 && all <= kResidentSmem ? all : need);
+      copied = n_units == 1 && all <= kResidentSmem;
+      resident.smem = (uint32_t)(copied ? all : need);
       break;
     }
   }
@@ -499,7 +500,8 @@ imdp_status Session::plan_grid(cudaStream_t st) {
   if (m->nnz >= (int64_t)kRuleLongColumn * m->n_cols && m->n_cols > (f32 ? 45000 : 56000)) return IMDP_OK;
   if (!plan_grid_unit(m, fixed_h.data(), grid, cut)) return IMDP_OK;
   const size_t need = grid_bytes(cut, f32), all = need + 64 + 20 * (size_t)cut.entries;
-  whole.smem = (uint32_t)((all <= kResidentSmem ? all : need) + 15) & ~15u;
+  copied = all <= kResidentSmem;
+  whole.smem = (uint32_t)((copied ? all : need) + 15) & ~15u;
   whole.grid = whole.steal_ctas = grid;
   whole.group = m->nnz >= 256 * (int64_t)m->n_cols || m->n_cols < 48 * (int64_t)grid ? 32 : 8;
   whole.f32 = f32 ? 1 : 0;
@@ -735,12 +737,28 @@ imdp_status Session::reset(cudaStream_t st) {
   return IMDP_OK;
 }
 
+int32_t Session::step_kernel(int32_t n) const {
+  if (cfg.kernel == kKernelRule && n >= kResidentSteps) {
+    if (resident.n_units > 0) return kKernelResident;
+    if (whole.n_units > 0) return kKernelGrid;
+  }
+  return resolve_launch(L, &cfg).kernel;
+}
+
+int32_t Session::launch_iterations() const {
+  // launches of about half a second, so that a long call does not hold the SMs
+  // that another stream's grid kernel waits for
+  int64_t entries = 0;
+  for (const DevModel* m : models) entries += m->nnz;
+  return (int32_t)std::min<int64_t>(50000, 64 + 100000000000ll / std::max<int64_t>(entries, 1));
+}
+
 imdp_status Session::step(int32_t n, cudaStream_t st) {
   if (n <= 0) return IMDP_OK;
   TraceRange trace("imdp session step");
   cudaError_t e = cudaSuccess;
-  const bool long_step = cfg.kernel == kKernelRule && n >= kResidentSteps && (resident.n_units > 0 || whole.n_units > 0);
-  if (!long_step && resolve_launch(L, &cfg).kernel == kKernelTiny) {
+  const int32_t kernel = step_kernel(n);
+  if (kernel == kKernelTiny) {
     // one small problem, few iterations: all of them in one launch of one CTA
     e = launch_bellman_tiny(L, n, models[0]->lg32 != nullptr, st);
     if (e != cudaSuccess) return cuda_status(e, "bellman step");
@@ -748,16 +766,13 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
     launched_since_reset += n;
     return IMDP_OK;
   }
-  if (long_step) {
-    // by rule: all n iterations in one launch of the resident or the grid kernel,
-    // or in several of about half a second, so that a long call does not hold the
-    // SMs that another stream's grid kernel waits for
-    int64_t entries = 0;
-    for (const DevModel* m : models) entries += m->nnz;
-    const int32_t most = (int32_t)std::min<int64_t>(50000, 64 + 100000000000ll / std::max<int64_t>(entries, 1));
+  if (kernel == kKernelResident || kernel == kKernelGrid) {
+    // by rule: all n iterations in one launch, or in a few
+    const int32_t most = launch_iterations();
     for (int32_t done = 0; done < n && e == cudaSuccess;) {
       const int32_t some = std::min(most, n - done);
-      e = resident.n_units > 0 ? launch_bellman_resident(L, resident, some, st) : launch_bellman_grid(L, whole, some, st);
+      e = kernel == kKernelResident ? launch_bellman_resident(L, resident, some, st)
+                                    : launch_bellman_grid(L, whole, some, st);
       done += some;
     }
     if (e != cudaSuccess) return cuda_status(e, "bellman step");

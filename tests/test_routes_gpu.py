@@ -1,0 +1,113 @@
+"""Which kernel a step call takes: the shapes by which the resident and the grid
+kernel are tested do run on them, so a rule or a plan that sends one elsewhere
+shows up here."""
+import time
+
+import numpy as np
+import pytest
+
+import paper_2401_04068_gb300 as g
+from test_resident_gpu import GRID, _lengths, _run, _same
+from workloads import banded_batch, banded_imdp, random_imdp
+from workloads.imdp_synth import concat_block_diagonal
+
+pytestmark = pytest.mark.gpu
+
+
+def _route(models, specs, n, **launch):
+    sess = g.imdp_session_create(models, specs)
+    if launch:
+        g.imdp_session_set_launch(sess, **launch)
+    r = g.imdp_session_step_route(sess, n)
+    sess.close()
+    return r
+
+
+def _alone(m, n=20, dtype=g.IMDP_F64, **kw):
+    model = g.create_model(m, dtype=dtype)
+    r = _route([model], [g.make_spec(horizon=20, reach=m.goal, **kw)], n)
+    model.close()
+    return r
+
+
+@pytest.mark.parametrize("dtype", [g.IMDP_F64, g.IMDP_F32])
+def test_kernels_of_one_problem(dtype):
+    for lens, kernel in (((1, 2, 7, 8, 9), g.KERNEL_RESIDENT), ((31, 32, 33, 63, 64, 65), g.KERNEL_RESIDENT),
+                         ((255, 256, 257, 300), g.KERNEL_GRID), ((5,), g.KERNEL_RESIDENT)):
+        r = _alone(_lengths(1100, lens, 5), dtype=dtype)
+        assert (r["kernel"], r["launches"], r["copied"]) == (kernel, 1, 1), lens
+    for name in GRID:
+        r = _alone(GRID[name](), dtype=dtype)
+        assert (r["kernel"], r["launches"], r["threads"]) == (g.KERNEL_GRID, 1, 768), name
+        assert r["group"] == (8 if name == "sink" else 32) and r["copied"] == (name not in ("long_sink", "wide")), name
+    for n, a, k in ((1, 1, 1), (5, 1, 5), (7, 3, 4), (64, 1, 12), (330, 3, 4), (1000, 1, 3)):
+        r = _alone(banded_imdp(n, a, n * a * (min(k, n) + 1) + 1, eps=0.1, seed=n), dtype=dtype)
+        assert r["kernel"] == g.KERNEL_RESIDENT and r["units"] == 1 and r["copied"] == 1, n
+        assert (r["cluster"] == 1) == (n in (1, 5)), n
+    for a, threads in ((1, 384), (3, 768)):
+        r = _alone(banded_imdp(610, a, 610 * a * 21 + 610 * a + 1, eps=0.1, seed=31), dtype=dtype)
+        assert (r["kernel"], r["cluster"], r["threads"]) == (g.KERNEL_RESIDENT, 16, threads)
+
+
+def test_kernels_of_many_problems():
+    ms = [banded_imdp(20 + 7 * (i % 60), 1 + i % 3, (20 + 7 * (i % 60)) * (1 + i % 3) * (3 + i % 17) + 1, seed=100 + i)
+          for i in range(200)]
+    models = [g.create_model(x) for x in ms]
+    specs = [g.make_spec(horizon=30, reach=x.goal) for x in ms]
+    r = _route(models, specs, 30)
+    assert r["kernel"] == g.KERNEL_RESIDENT and r["units"] == 200 and r["threads"] == 384 and r["ctas"] > 152
+    # short calls and explicit configurations run one launch an iteration
+    assert _route(models, specs, 3)["launches"] == 3
+    assert _route(models, specs, 30, kernel=g.KERNEL_RING) == dict(kernel=g.KERNEL_RING, launches=30, units=0,
+                                                                  cluster=0, ctas=0, threads=0, group=0, copied=0)
+    m = concat_block_diagonal([banded_batch(40, 60, 1, 60 * 12 + 60 + 1, seed=3), random_imdp(1, seed=4),
+                               banded_imdp(330, 1, 330 * 70 + 330 + 1, seed=5),
+                               random_imdp(37, max_actions=1, seed=6)])
+    model = g.create_model(m)
+    finite, infinite = g.make_spec(horizon=30, reach=m.goal), g.make_spec(infinite_time=True, horizon=50, reach=m.goal)
+    r = _route([model], [finite], 30)
+    assert r["kernel"] == g.KERNEL_RESIDENT and r["units"] > 40 and r["cluster"] > 1
+    assert _route([model], [infinite], 30)["units"] == 1
+
+
+# more parts than two CTAs on every SM hold, in CTAs of half the threads; rounds of them, the last one not full
+@pytest.mark.parametrize("storage", [g.IMDP_F64, g.IMDP_F32])
+@pytest.mark.parametrize("blocks", [304, 1001])
+def test_parts_on_half_size_ctas(storage, blocks):
+    m = banded_batch(blocks, 40, 2, 40 * 2 * 11 + 40 * 2 + 1, eps=0.1, seed=blocks)
+    model = g.create_model(m, dtype=storage)
+    specs = [g.make_spec(horizon=25, reach=m.goal)]
+    r = _route([model], specs, 25)
+    assert (r["kernel"], r["units"], r["cluster"], r["threads"], r["ctas"]) == (g.KERNEL_RESIDENT, blocks, 1, 384, 304)
+    _same(_run([model], [m], specs, g.KERNEL_RING, policy=True), _run([model], [m], specs, g.KERNEL_RULE, policy=True))
+    model.close()
+
+
+def test_bad_route_queries():
+    m = random_imdp(5, seed=1)
+    model = g.create_model(m)
+    sess = g.imdp_session_create([model], [g.make_spec(horizon=3, reach=m.goal)])
+    with pytest.raises(g.ImdpError):
+        g.imdp_session_step_route(sess, 0)
+    sess.close()
+    model.close()
+
+
+@pytest.mark.parametrize("storage", [g.IMDP_F64, g.IMDP_F32])
+def test_requests_share_launches(storage):
+    ms = [banded_imdp(2000, 2, 2000 * 2 * 150 + 2001, eps=0.1, seed=70), banded_imdp(6000, 3, 6000 * 3 * 3 + 1, seed=71),
+          banded_imdp(70, 2, 70 * 2 * 9 + 1, seed=75)]
+    models = [g.create_model(m, dtype=storage) for m in ms]
+    for launch in ({}, dict(kernel=g.KERNEL_RING)):
+        server = g.imdp_server_create(256 << 20)
+        if launch:
+            g.imdp_server_set_launch(server, **launch)
+        tickets = [g.imdp_server_submit(server, models[i % 3], g.make_spec(horizon=60 + i, reach=ms[i % 3].goal))
+                   for i in range(12)]
+        for i, t in enumerate(tickets):
+            assert g.imdp_server_wait(server, t, 60000.0, np.zeros(ms[i % 3].n_states)) == g.IMDP_OK
+        time.sleep(0.2)  # the worker counts a launch after its requests have retired
+        n = g.imdp_server_launches(server)
+        assert (n["shared"] > 0, n["per_iteration"] > 0) == ((False, True) if launch else (True, False)), n
+        assert n["shared"] + n["per_iteration"] // 8 == g.imdp_server_stats(server)["chunks"]
+        server.close()
