@@ -312,7 +312,9 @@ IMDP_API void imdp_session_destroy(imdp_session* s);
  *                 model already has its slice layout (see 4 below: building it
  *                 costs about as many iterations' time as a few hundred save),
  *                 otherwise ring (the server's rule is the grid kernel, several
- *                 requests in one launch, or ring);
+ *                 requests in one launch, or ring). With kernel 0 and any field
+ *                 below given, every step runs these per-iteration kernels, in the
+ *                 shape asked for;
  *                 1 ring: a producer warp bulk-copies tiles of
  *                 consecutive states into a three-stage shared-memory ring for
  *                 consumer warps; 2 direct: every warp takes the next tile and

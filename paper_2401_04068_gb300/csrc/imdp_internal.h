@@ -210,6 +210,10 @@ struct LaunchConfig {
   int32_t ctas_per_sm = 0;       // direct and slice: 3 or 4 CTAs per SM
   int32_t tile_entries = 0;      // tile plan: entries per tile (<= kTileEntries)
   int32_t wide_col = 0;          // columns this long make their state wide
+  // nothing asked for: step calls may take the resident or the grid kernel, which have no such fields
+  bool by_rule() const {
+    return kernel == kKernelRule && !cta_warps && !ctas_per_sm && !tile_entries && !wide_col;
+  }
 };
 
 // Second stream on which the wide-state kernel runs beside the tiled one.

@@ -709,7 +709,7 @@ struct Server {
       {
         std::lock_guard<std::mutex> lk(mu);
         lc = cfg;
-        if (lc.kernel == kKernelRule && fits) {
+        if (lc.by_rule() && fits) {
           // planned again when a quarter of the CTAs have run out of work
           grid_kernel = gplan.n_units > 0 && !changed && plan_quantum(work) * 4 > gplan.grid * 3;
           if (!grid_kernel) {

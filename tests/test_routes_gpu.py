@@ -111,3 +111,35 @@ def test_requests_share_launches(storage):
         assert (n["shared"] > 0, n["per_iteration"] > 0) == ((False, True) if launch else (True, False)), n
         assert n["shared"] + n["per_iteration"] // 8 == g.imdp_server_stats(server)["chunks"]
         server.close()
+
+
+@pytest.mark.parametrize("field", ["cta_warps", "ctas_per_sm", "tile_entries", "wide_col"])
+def test_a_partial_configuration_shapes_the_steps(field):
+    # kernel 0 with a field given: the per-iteration kernels run in that shape, as
+    # imdp_session_get_launch reports; all zero goes back to the rule
+    value = dict(cta_warps=24, ctas_per_sm=3, tile_entries=600, wide_col=200)[field]
+    m = banded_imdp(2000, 1, 2000 * 40 + 2000 + 1, eps=0.05, seed=82)
+    model = g.create_model(m)
+    spec = g.make_spec(horizon=30, reach=m.goal)
+    sess = g.imdp_session_create([model], [spec])
+    assert g.imdp_session_step_route(sess, 30)["kernel"] in (g.KERNEL_RESIDENT, g.KERNEL_GRID)
+    g.imdp_session_set_launch(sess, **{field: value})
+    r, got = g.imdp_session_step_route(sess, 30), g.imdp_session_get_launch(sess)
+    assert r["kernel"] == got["kernel"] == g.KERNEL_RING and r["launches"] == 30
+    assert field == "ctas_per_sm" or got[field] == value
+    g.imdp_session_step(sess, 30)
+    raw, _ = g.imdp_session_checkpoint(sess, 0)
+    g.imdp_session_set_launch(sess)
+    assert g.imdp_session_step_route(sess, 30)["kernel"] in (g.KERNEL_RESIDENT, g.KERNEL_GRID)
+    g.imdp_session_reset(sess)
+    g.imdp_session_step(sess, 30)
+    np.testing.assert_array_equal(raw, g.imdp_session_checkpoint(sess, 0)[0])
+    sess.close()
+    server = g.imdp_server_create(64 << 20)
+    g.imdp_server_set_launch(server, **{field: value})
+    t = g.imdp_server_submit(server, model, spec)
+    assert g.imdp_server_wait(server, t, 60000.0, np.zeros(m.n_states)) == g.IMDP_OK
+    time.sleep(0.2)
+    assert g.imdp_server_launches(server)["shared"] == 0
+    server.close()
+    model.close()
