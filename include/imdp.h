@@ -391,9 +391,13 @@ IMDP_API imdp_status imdp_session_plan(const imdp_session* s, int32_t* n_tiles, 
  * JSON file `cache_path` (nullable: no cache) under a key describing the
  * session's shape (storage, mean transitions per column, columns per state,
  * states, whether it has wide states); a later call with the same key applies
- * the cached configuration without timing. The session is reset afterwards.
- * `chosen` (nullable) receives the configuration in use; `ms_per_iter`
- * (nullable) its measured time per iteration (0 when taken from the cache).
+ * the cached configuration without timing (an entry of a file from before the
+ * resident and grid kernels is timed against them once). The session is reset
+ * afterwards. Steps of 4 and more iterations go on by rule (resident or grid
+ * kernel) where that was faster than every configuration; imdp_session_step_route
+ * tells. `chosen` (nullable) receives the configuration in use (of the other
+ * steps, in that case); `ms_per_iter` (nullable) the measured time per iteration
+ * of the fastest (0 when taken from the cache).
  */
 IMDP_API imdp_status imdp_session_autotune(imdp_session* s, int32_t iters, const char* cache_path, void* stream,
                                            imdp_launch_config* chosen, double* ms_per_iter);

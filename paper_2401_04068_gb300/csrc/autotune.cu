@@ -79,6 +79,9 @@ std::string shape_key(const Session* S) {
 }
 
 // The cache file: {"key": {"kernel": 2, "cta_warps": 8, ...}, ...} as written below.
+// "long_by_rule": 1 when steps of kResidentSteps iterations and more were faster
+// by rule (resident or grid kernel); no such field when that was not timed (a
+// session that plans neither, a file from before those kernels).
 std::map<std::string, std::string> read_cache(const char* path) {
   std::map<std::string, std::string> out;
   if (!path) return out;
@@ -111,8 +114,9 @@ bool field(const std::string& body, const char* name, double* v) {
   return std::sscanf(body.c_str() + at + pat.size(), "%lf", v) == 1;
 }
 
-bool parse_entry(const std::string& body, LaunchConfig* c) {
-  double k, w, p, t, wc;
+// `knows_rule`: the entry was chosen with the rule's own kernels among the candidates.
+bool parse_entry(const std::string& body, LaunchConfig* c, bool* knows_rule) {
+  double k, w, p, t, wc, rule = 0.0;
   if (!field(body, "kernel", &k) || !field(body, "cta_warps", &w) || !field(body, "ctas_per_sm", &p) ||
       !field(body, "tile_entries", &t) || !field(body, "wide_col", &wc))
     return false;
@@ -121,6 +125,8 @@ bool parse_entry(const std::string& body, LaunchConfig* c) {
   c->ctas_per_sm = (int32_t)p;
   c->tile_entries = (int32_t)t;
   c->wide_col = (int32_t)wc;
+  *knows_rule = field(body, "long_by_rule", &rule);
+  c->long_by_rule = rule != 0.0;
   return true;
 }
 
@@ -138,12 +144,13 @@ bool write_cache(const char* path, const std::map<std::string, std::string>& ent
   return ok && std::rename(tmp.c_str(), path) == 0;
 }
 
-std::string entry_body(const LaunchConfig& c, double ms) {
+std::string entry_body(const LaunchConfig& c, bool rule_timed, double ms) {
   char buf[256];
   std::snprintf(buf, sizeof(buf),
                 "{\"kernel\": %d, \"cta_warps\": %d, \"ctas_per_sm\": %d, \"tile_entries\": %d, \"wide_col\": %d, "
-                "\"ms_per_iter\": %.6f}",
-                c.kernel, c.cta_warps, c.ctas_per_sm, c.tile_entries, c.wide_col, ms);
+                "%s\"ms_per_iter\": %.6f}",
+                c.kernel, c.cta_warps, c.ctas_per_sm, c.tile_entries, c.wide_col,
+                !rule_timed ? "" : (c.long_by_rule ? "\"long_by_rule\": 1, " : "\"long_by_rule\": 0, "), ms);
   return buf;
 }
 
@@ -256,7 +263,12 @@ IMDP_API imdp_status imdp_session_autotune(imdp_session* s, int32_t iters, const
   double best_ms = 0.0;
   imdp_status r = IMDP_OK;
   auto it = cache.find(key);
-  if (it != cache.end() && parse_entry(it->second, &best)) {
+  bool knows_rule = false;
+  const bool cached = it != cache.end() && parse_entry(it->second, &best, &knows_rule);
+  // (an entry from before the rule's own kernels is timed against them)
+  const bool time_rule = S->plans_long_steps() && !(cached && knows_rule);
+  if (cached && !time_rule) {
+    best.long_by_rule = best.long_by_rule && S->plans_long_steps();
     r = S->set_launch(best, st);
   } else {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -293,6 +305,7 @@ IMDP_API imdp_status imdp_session_autotune(imdp_session* s, int32_t iters, const
     add(kKernelSlice, kSliceWarps, 4, kTileEntries, kWideCol);
     add(kKernelSlice, kSliceWarps, 3, kTileEntries, kWideCol);
     bool have = false;
+    if (cached) cands.assign(1, best);
     for (const LaunchConfig& c : cands) {
       double ms = 0.0;
       if ((r = time_config(S, c, iters, st, e0, e1, &ms)) != IMDP_OK) break;
@@ -303,7 +316,7 @@ IMDP_API imdp_status imdp_session_autotune(imdp_session* s, int32_t iters, const
       }
     }
     // stage 2: the wide-state threshold, for models with long columns
-    if (r == IMDP_OK && max_col >= 640 && best.kernel != kKernelTiny && best.kernel != kKernelSlice) {
+    if (r == IMDP_OK && !cached && max_col >= 640 && best.kernel != kKernelTiny && best.kernel != kKernelSlice) {
       for (int32_t wc : {640, 2560, 1 << 30}) {
         LaunchConfig c = best;
         c.wide_col = wc;
@@ -316,12 +329,21 @@ IMDP_API imdp_status imdp_session_autotune(imdp_session* s, int32_t iters, const
         }
       }
     }
+    // stage 3: the kernels that long steps take by rule (at least as many iterations as those take)
+    if (r == IMDP_OK && time_rule) {
+      double ms = 0.0;
+      r = time_config(S, LaunchConfig{}, std::max(iters, kResidentSteps), st, e0, e1, &ms);
+      if (r == IMDP_OK && ms < best_ms) {
+        best.long_by_rule = true;
+        best_ms = ms;
+      }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (r == IMDP_OK) r = S->set_launch(best, st);
     if (r == IMDP_OK && cache_path) {
-      cache[key] = entry_body(best, best_ms);
-      if (!write_cache(cache_path, cache)) {
+      cache[key] = entry_body(best, time_rule, best_ms);
+      if (!write_cache(cache_path, cache) && !cached) {
         set_error(std::string("autotune: cannot write the cache file ") + cache_path);
         r = IMDP_EIO;
       }

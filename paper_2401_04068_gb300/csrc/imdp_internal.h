@@ -210,6 +210,8 @@ struct LaunchConfig {
   int32_t ctas_per_sm = 0;       // direct and slice: 3 or 4 CTAs per SM
   int32_t tile_entries = 0;      // tile plan: entries per tile (<= kTileEntries)
   int32_t wide_col = 0;          // columns this long make their state wide
+  // the autotuner's: the fields are those of short step calls, long ones go by rule
+  bool long_by_rule = false;
   // nothing asked for: step calls may take the resident or the grid kernel, which have no such fields
   bool by_rule() const {
     return kernel == kKernelRule && !cta_warps && !ctas_per_sm && !tile_entries && !wide_col;
@@ -475,6 +477,7 @@ struct Session {
   GridPlan whole{};  // the grid kernel's (n_units 0: not taken)
   imdp_status plan_grid(cudaStream_t st);
   bool copied = false;  // the plan above keeps the transitions in shared memory
+  bool plans_long_steps() const { return resident.n_units > 0 || whole.n_units > 0; }
   // The kernel that a step call of n iterations takes, and how many of them one launch runs.
   int32_t step_kernel(int32_t n) const;
   int32_t launch_iterations() const;

@@ -738,7 +738,7 @@ imdp_status Session::reset(cudaStream_t st) {
 }
 
 int32_t Session::step_kernel(int32_t n) const {
-  if (cfg.by_rule() && n >= kResidentSteps) {
+  if ((cfg.by_rule() || cfg.long_by_rule) && n >= kResidentSteps) {
     if (resident.n_units > 0) return kKernelResident;
     if (whole.n_units > 0) return kKernelGrid;
   }

@@ -1,6 +1,7 @@
 """Which kernel a step call takes: the shapes by which the resident and the grid
 kernel are tested do run on them, so a rule or a plan that sends one elsewhere
 shows up here."""
+import json
 import time
 
 import numpy as np
@@ -142,4 +143,51 @@ def test_a_partial_configuration_shapes_the_steps(field):
     time.sleep(0.2)
     assert g.imdp_server_launches(server)["shared"] == 0
     server.close()
+    model.close()
+
+
+def test_autotuned_sessions_keep_the_faster_rule(tmp_path):
+    # The rule's own kernels are among the candidates: a tuned session is no slower
+    # than an untuned one. 64 parts of 120 states take the resident kernel by rule.
+    m = banded_batch(64, 120, 1, 120 * 30 + 120 + 1, eps=0.05, seed=7)
+    model = g.create_model(m)
+    spec = g.make_spec(horizon=60, reach=m.goal)
+    cache = tmp_path / "tuned.json"
+
+    def tuned(iters=60):
+        sess = g.imdp_session_create([model], [spec])
+        cfg, ms = g.imdp_session_autotune(sess, iters, str(cache))
+        return sess, cfg, ms
+
+    sess, cfg, ms = tuned()
+    # (this query per iteration takes about 10 us an iteration at best, by rule about 3)
+    assert g.imdp_session_step_route(sess, 60)["kernel"] == g.KERNEL_RESIDENT
+    assert cfg["kernel"] in (g.KERNEL_RING, g.KERNEL_DIRECT, g.KERNEL_SLICE) and ms > 0
+    assert cfg["kernel"] == g.imdp_session_get_launch(sess)["kernel"] == g.imdp_session_step_route(sess, 1)["kernel"]
+    g.imdp_session_run(sess)
+    raw, k = g.imdp_session_checkpoint(sess, 0)
+    sess.close()
+    assert k == 60
+    plain = g.imdp_session_create([model], [spec])
+    g.imdp_session_run(plain)
+    np.testing.assert_array_equal(raw, g.imdp_session_checkpoint(plain, 0)[0])
+    plain.close()
+    # the cached choice: the same, without timing
+    sess, cfg2, ms = tuned()
+    assert ms == 0.0 and cfg2 == cfg and g.imdp_session_step_route(sess, 60)["kernel"] == g.KERNEL_RESIDENT
+    sess.close()
+    # an entry that knows nothing of the rule's kernels is timed against them once
+    data = json.loads(cache.read_text())
+    entry = next(iter(data.values()))
+    assert entry.pop("long_by_rule") == 1
+    cache.write_text(json.dumps(data).replace("}, ", "},\n"))
+    sess, cfg3, ms = tuned()
+    assert ms > 0 and cfg3 == cfg and g.imdp_session_step_route(sess, 60)["kernel"] == g.KERNEL_RESIDENT
+    sess.close()
+    assert next(iter(json.loads(cache.read_text()).values()))["long_by_rule"] == 1
+    # tuned on single iterations: the same
+    cache.unlink()
+    sess, _, _ = tuned(1)
+    assert g.imdp_session_step_route(sess, 60)["kernel"] == g.KERNEL_RESIDENT
+    sess.close()
     model.close()
