@@ -280,6 +280,7 @@ struct StepLaunch {
 constexpr int kMaxCluster = 16;
 constexpr int32_t kResidentThreads = 768;  // threads of an SM (80 registers each), as one CTA or two
 constexpr size_t kResidentSmem = 232448;  // dynamic shared memory one CTA can have
+constexpr size_t kResidentHalfSmem = 115712;  // what each of two CTAs of an SM can have (228 KB less 1 KB a CTA)
 constexpr int32_t kResidentSteps = 4;  // step calls of fewer iterations launch one by one
 struct ResidentUnit {
   int32_t p;       // problem

@@ -393,7 +393,8 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
   while (c > 1 && cols < 7 * (int64_t)c * n_units) c /= 2;
   const bool alone = count == 1 && n_units == 1;
   // Two CTAs of an SM overlap each other's barriers while both their units stay
-  // in L2 (4096 parts of 0.3 MB on 32-bit storage: 68 ms against 74 with one).
+  // in L2 (4096 parts of 0.3 MB on 32-bit storage: 68 ms against 74 with one) and
+  // have room beside each other (below).
   const bool two = n_units * (int64_t)c >= 2 * grid && unit_bytes * (2 * grid / c) <= 100e6;
   // Half the warps also where they hold a CTA's few short columns: their barriers
   // are cheaper (5 columns 238 us against 251, 600 columns 607 against 799).
@@ -441,7 +442,13 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
         prev = s;
       }
     }
-    const size_t need = resident_bytes(states, resident.cap_cols, resident.cap_own, f32, resident.threads);
+    size_t need = resident_bytes(states, resident.cap_cols, resident.cap_own, f32, resident.threads);
+    if (two && !few && need > kResidentHalfSmem) {
+      // alone on its SM, a CTA of half the threads leaves half of it idle (1,000 parts
+      // of 1,500 states and 5 entries a column: 33.6 ms, 23.2 with all threads)
+      resident.threads = kResidentThreads;
+      need = resident_bytes(states, resident.cap_cols, resident.cap_own, f32, resident.threads);
+    }
     if (need <= kResidentSmem && resident.cap_cols <= 65535) {
       // one unit: its entries go to shared memory as well where they fit (no L2
       // latency in its iterations; pendulum_240 alone 1.03 ms against 1.11). With

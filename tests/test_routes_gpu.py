@@ -191,3 +191,16 @@ def test_autotuned_sessions_keep_the_faster_rule(tmp_path):
     assert g.imdp_session_step_route(sess, 60)["kernel"] == g.KERNEL_RESIDENT
     sess.close()
     model.close()
+
+
+# parts on either side of the shared memory that each of two CTAs of an SM can have
+@pytest.mark.parametrize("storage", [g.IMDP_F64, g.IMDP_F32])
+@pytest.mark.parametrize("states,threads,ctas", [(1000, 384, 304), (1300, 768, 152)])
+def test_half_size_ctas_only_where_two_fit_an_sm(storage, states, threads, ctas):
+    m = banded_batch(310, states, 1, states * 4 + 1, eps=0.1, seed=states)
+    model = g.create_model(m, dtype=storage)
+    specs = [g.make_spec(horizon=12, reach=m.goal)]
+    r = _route([model], specs, 12)
+    assert (r["kernel"], r["units"], r["cluster"], r["threads"], r["ctas"]) == (g.KERNEL_RESIDENT, 310, 1, threads, ctas)
+    _same(_run([model], [m], specs, g.KERNEL_RING), _run([model], [m], specs, g.KERNEL_RULE))
+    model.close()
