@@ -474,7 +474,9 @@ struct Session {
   imdp_status prepare_slices(cudaStream_t st);
   // Step calls by rule: the resident kernel's plan (n_units 0: not taken).
   ResidentPlan resident{};
-  imdp_status plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st);
+  // `beside_grid`: not where the grid kernel is the faster one by the cost model.
+  imdp_status plan_resident(const std::vector<const imdp_spec*>& specs, bool beside_grid, cudaStream_t st);
+  bool grid_possible() const;  // by the model's size and columns
   GridPlan whole{};  // the grid kernel's (n_units 0: not taken)
   imdp_status plan_grid(cudaStream_t st);
   bool copied = false;  // the plan above keeps the transitions in shared memory

@@ -306,8 +306,10 @@ imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<
     S->L.shape_f32 = all32 ? 1 : 0;
   }
   S->grid = bellman_grid();
-  imdp_status r = S->plan_resident(specs, st);
+  imdp_status r = S->plan_resident(specs, true, st);
   if (r == IMDP_OK) r = S->plan_grid(st);
+  // (left to the grid kernel, whose shares do not fit)
+  if (r == IMDP_OK && !S->plans_long_steps() && S->grid_possible()) r = S->plan_resident(specs, false, st);
   if (r != IMDP_OK) { delete S; return r; }
   const bool slice = resolve_launch(S->L, &S->cfg).kernel == kKernelSlice;
   r = slice ? S->prepare_slices(st) : IMDP_OK;
@@ -323,7 +325,19 @@ imdp_status Session::create(const std::vector<DevModel*>& ms, const std::vector<
   return IMDP_OK;
 }
 
-imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, cudaStream_t st) {
+bool Session::grid_possible() const {
+  const DevModel* m = models[0];
+  if (L.tiny_ok || count != 1 || is_slice(m) || m->nnz >= kGridMostEntries) return false;
+  // Many long columns stay on the direct kernel: it settles a missed column while
+  // its entries are still in L1 and L2 (100 iterations, direct and grid kernel, ms:
+  // 48,000 columns of 500 entries 21.0 / 19.1, 56,000 of 376 16.7 / 16.5, 84,000 of
+  // 376 20.2 / 20.8; on 32-bit storage 42,000 of 376 8.2 / 7.0, 48,000 of 500 15.7 /
+  // 15.9, 90,000 of 300 14.5 / 16.4). Against the ring kernel, which short columns
+  // take otherwise, it gains at any number (126,000 of 230 20.5 / 17.5).
+  return m->nnz < (int64_t)kRuleLongColumn * m->n_cols || m->n_cols <= (m->lg32 ? 45000 : 56000);
+}
+
+imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, bool beside_grid, cudaStream_t st) {
   resident = ResidentPlan{};
   bool any32 = false, any64 = false;
   for (const DevModel* m : models) {
@@ -361,9 +375,10 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
       us.push_back(Work{ResidentUnit{p, 0, models[p]->n_states}, e, e * std::max<int64_t>(K, 1)});
     }
   }
-  int64_t entries = 0, work = 0, most = 0, cols = 0;
+  int64_t entries = 0, work = 0, most = 0, cols = 0, longest = 1;  // iterations of the longest (parts: 1)
   int32_t states = 0, max_col = 0;
   for (const Work& w : us) {
+    longest = std::max(longest, w.work / std::max<int64_t>(w.entries, 1));
     entries += w.entries;
     work += w.work;
     most = std::max(most, w.work);
@@ -395,26 +410,31 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
   // Two CTAs of an SM overlap each other's barriers while both their units stay
   // in L2 (4096 parts of 0.3 MB on 32-bit storage: 68 ms against 74 with one) and
   // have room beside each other (below).
-  const bool two = n_units * (int64_t)c >= 2 * grid && unit_bytes * (2 * grid / c) <= 100e6;
+  const auto two_of = [&](int c) { return n_units * (int64_t)c >= 2 * grid && unit_bytes * (2 * grid / c) <= 100e6; };
   // Half the warps also where they hold a CTA's few short columns: their barriers
   // are cheaper (5 columns 238 us against 251, 600 columns 607 against 799).
   const bool few = alone && cols <= 48 * c && entries <= 32 * cols;
-  resident.threads = two || few ? kResidentThreads / 2 : kResidentThreads;
-  // Seconds an iteration takes: per-iteration launches about 10 us and 0.64
-  // transitions a cycle and SM, this kernel about 3 us and 1.17 on the SMs it
+  // Seconds for all iterations: per-iteration launches take about 10 us each and
+  // 0.64 transitions a cycle and SM, this kernel about 3 us and 1.17 on the SMs it
   // covers, the grid kernel (one problem only) about 6.5 us and 1 on all.
-  const double sms = std::min<double>(grid, (double)n_units * c), hz = 1.9e9, e = (double)entries;
-  double other = 10e-6 + e / (0.64 * grid * hz);
-  if (alone) other = std::min(other, 6.5e-6 + e / (1.0 * grid * hz));
-  if (3e-6 + e / (1.17 * sms * hz) > other) return IMDP_OK;
-  // ranks of a unit: contiguous states of about equal work
+  const double hz = 1.9e9, iters = (double)longest, all_work = (double)work;
+  double other = iters * 10e-6 + all_work / (0.64 * grid * hz);
+  const double by_grid = iters * 6.5e-6 + all_work / (1.0 * grid * hz);
+  if (beside_grid && grid_possible()) other = std::min(other, by_grid);
+  const auto spread = [&](int c) {
+    return iters * 3e-6 + all_work / (1.17 * std::min<double>(grid, (double)n_units * c) * hz);
+  };
+  if (spread(c) > other) return IMDP_OK;
+  // Ranks of a unit: contiguous states of about equal work. False when a rank's
+  // share does not fit a CTA.
   std::vector<int32_t> bounds;
-  int64_t rank_entries = 0;
-  for (;; c *= 2) {
-    if (c > kMaxCluster || resident_bytes(states, 1, 1, f32, resident.threads) > kResidentSmem) return IMDP_OK;
+  const auto shape = [&](int c) -> bool {
+    int64_t rank_entries = 0;
+    const bool two = two_of(c);
+    resident.threads = two || few ? kResidentThreads / 2 : kResidentThreads;
+    if (resident_bytes(states, 1, 1, f32, resident.threads) > kResidentSmem) return false;
     resident.cap_cols = 32;
     resident.cap_own = 0;
-    rank_entries = 0;
     bounds.clear();
     bounds.reserve((size_t)n_units * (c + 1));
     for (const Work& w : us) {
@@ -449,31 +469,68 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
       resident.threads = kResidentThreads;
       need = resident_bytes(states, resident.cap_cols, resident.cap_own, f32, resident.threads);
     }
-    if (need <= kResidentSmem && resident.cap_cols <= 65535) {
-      // one unit: its entries go to shared memory as well where they fit (no L2
-      // latency in its iterations; pendulum_240 alone 1.03 ms against 1.11). With
-      // many units the wider clusters that takes cost more than it saves.
-      const size_t all = need + 64 + (size_t)rank_entries * 20;
-      copied = n_units == 1 && all <= kResidentSmem;
-      resident.smem = (uint32_t)(copied ? all : need);
-      break;
-    }
-  }
-  const double k = (double)entries / std::max<int64_t>(cols, 1);
-  // lanes to a column: whole warps when the columns are long or too few for groups
-  resident.group = k >= 256 || (double)cols / n_units / c < 4.0 * resident.threads / 32 / 2 ? 32 : 8;
-  resident.cluster = c;
+    if (need > kResidentSmem || resident.cap_cols > 65535) return false;
+    // one unit: its entries go to shared memory as well where they fit (no L2
+    // latency in its iterations; pendulum_240 alone 1.03 ms against 1.11). With
+    // many units the wider clusters that takes cost more than it saves.
+    const size_t all = need + 64 + (size_t)rank_entries * 20;
+    copied = n_units == 1 && all <= kResidentSmem;
+    resident.smem = (uint32_t)(copied ? all : need);
+    // lanes to a column: whole warps when the columns are long or too few for groups
+    const double k = (double)entries / std::max<int64_t>(cols, 1);
+    resident.group = k >= 256 || (double)cols / n_units / c < 4.0 * resident.threads / 32 / 2 ? 32 : 8;
+    resident.cluster = c;
+    return resident_prepare(resident) == cudaSuccess;  // (wide clusters may not fit the device)
+  };
   resident.parts = parts ? 1 : 0;
   resident.f32 = f32 ? 1 : 0;
   resident.cap_states = states;
   resident.max_col = max_col;
   resident.n_units = n_units;
-  cudaError_t err = resident_prepare(resident);
-  if (err != cudaSuccess) {  // clusters this wide do not fit the device: the per-iteration kernels run
+  const auto none = [&]() {
     cudaGetLastError();
     resident.n_units = 0;
     return IMDP_OK;
+  };
+  while (!shape(c))
+    if ((c *= 2) > kMaxCluster) return none();
+  // A unit has its cluster's SMs only, and where there are a few units more than
+  // clusters (of 16 CTAs 7 fit the GPU, of 8 15) some wait for another one. A cluster
+  // takes 1.25 to 1.46 transitions a cycle and SM. 200 iterations: 5 million
+  // transitions with small units beside them 26.8 ms, on the grid kernel 5.2, per
+  // iteration 10.4. Beside 40 units of 80,000 and 20 iterations: 1 million, 500
+  // iterations 12.8, per iteration 8.4; 300,000, 200 iterations 3.0 and 3.7.
+  const auto uneven = [&](int c) {
+    const size_t m = resident.clusters;
+    const auto seconds = [&](size_t i, double rate) {
+      const double its = (double)(us[i].work / std::max<int64_t>(us[i].entries, 1));
+      return its * 3e-6 + us[i].work / (rate * c * hz);
+    };
+    // two CTAs of an SM share its rate while there are units for both
+    const double shared = resident.clusters * c > grid ? 1.35 / 2 : 1.35;
+    double rest = 0.0;
+    for (size_t i = 1; i < us.size(); ++i) rest += seconds(i, shared) / m;
+    double first = seconds(0, shared);
+    if (first > rest) first = rest + (1.0 - rest / first) * seconds(0, 1.35);
+    return c > 1 && us.size() > m ? std::max(first, seconds(m - 1, shared) + seconds(m, shared)) : first;
+  };
+  // a few units too many for the clusters: more, smaller clusters where that is faster
+  // (8 units of 80,000 transitions: 2.05 ms with 7 clusters of 16, 1.40 with 8 of 8;
+  // 64 of 6,000: 1.07 with 36 of 4, 0.62 with 64 of 2)
+  while (c > 1 && n_units > resident.clusters && n_units <= 2 * resident.clusters &&
+         unit_bytes * (2 * grid / c) <= 200e6) {
+    const ResidentPlan wide = resident;
+    const std::vector<int32_t> wide_bounds = bounds;
+    const double before = std::max(uneven(c), spread(c));
+    if (shape(c / 2) && std::max(uneven(c / 2), spread(c / 2)) < before) {
+      c /= 2;
+      continue;
+    }
+    resident = wide;
+    bounds = wide_bounds;
+    break;
   }
+  if (std::max(uneven(c), spread(c)) > other) return none();
   std::vector<ResidentUnit> uh(n_units);
   for (int32_t i = 0; i < n_units; ++i) uh[i] = us[i].u;
   ResidentUnit* du = alloc<ResidentUnit>(uh.size());
@@ -483,7 +540,7 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, c
     set_error("device allocation failed (session)");
     return IMDP_ENOMEM;
   }
-  err = cudaMemcpyAsync(du, uh.data(), sizeof(ResidentUnit) * uh.size(), cudaMemcpyHostToDevice, st);
+  cudaError_t err = cudaMemcpyAsync(du, uh.data(), sizeof(ResidentUnit) * uh.size(), cudaMemcpyHostToDevice, st);
   if (err == cudaSuccess) err = cudaMemcpyAsync(db, bounds.data(), sizeof(int32_t) * bounds.size(), cudaMemcpyHostToDevice, st);
   if (err == cudaSuccess) err = cudaStreamSynchronize(st);  // the host vectors go out of scope
   if (err != cudaSuccess) return cuda_status(err, "session plan");
@@ -497,14 +554,7 @@ imdp_status Session::plan_grid(cudaStream_t st) {
   const DevModel* m = models[0];
   GridCut cut;
   const bool f32 = m->lg32 != nullptr;
-  if (L.tiny_ok || resident.n_units > 0 || count != 1) return IMDP_OK;
-  // Many long columns stay on the direct kernel: it settles a missed column while
-  // its entries are still in L1 and L2 (100 iterations, direct and grid kernel, ms:
-  // 48,000 columns of 500 entries 21.0 / 19.1, 56,000 of 376 16.7 / 16.5, 84,000 of
-  // 376 20.2 / 20.8; on 32-bit storage 42,000 of 376 8.2 / 7.0, 48,000 of 500 15.7 /
-  // 15.9, 90,000 of 300 14.5 / 16.4). Against the ring kernel, which short columns
-  // take otherwise, it gains at any number (126,000 of 230 20.5 / 17.5).
-  if (m->nnz >= (int64_t)kRuleLongColumn * m->n_cols && m->n_cols > (f32 ? 45000 : 56000)) return IMDP_OK;
+  if (resident.n_units > 0 || !grid_possible()) return IMDP_OK;
   if (!plan_grid_unit(m, fixed_h.data(), grid, cut)) return IMDP_OK;
   const size_t need = grid_bytes(cut, f32), all = need + 64 + 20 * (size_t)cut.entries;
   copied = all <= kResidentSmem;

@@ -204,3 +204,46 @@ def test_half_size_ctas_only_where_two_fit_an_sm(storage, states, threads, ctas)
     assert (r["kernel"], r["units"], r["cluster"], r["threads"], r["ctas"]) == (g.KERNEL_RESIDENT, 310, 1, threads, ctas)
     _same(_run([model], [m], specs, g.KERNEL_RING), _run([model], [m], specs, g.KERNEL_RULE))
     model.close()
+
+
+# one large unit beside small ones: its cluster alone would take longer than the whole GPU does
+@pytest.mark.parametrize("as_parts", [True, False])
+def test_a_dominant_unit_takes_the_whole_gpu(as_parts):
+    ms = [banded_imdp(2000, 2, 2000 * 2 * 1251 + 1, eps=0.1, seed=1)]
+    ms += [banded_imdp(200, 1, 200 * 21 + 1, eps=0.1, seed=2 + i) for i in range(12)]
+    if as_parts:
+        ms = [concat_block_diagonal(ms)]
+    models = [g.create_model(m) for m in ms]
+    specs = [g.make_spec(horizon=12, reach=m.goal) for m in ms]
+    kernel = _route(models, specs, 12)["kernel"]
+    assert kernel == g.KERNEL_GRID if as_parts else kernel not in (g.KERNEL_GRID, g.KERNEL_RESIDENT)
+    _same(_run(models, ms, specs, g.KERNEL_RING), _run(models, ms, specs, g.KERNEL_RULE))
+    for m in models:
+        m.close()
+
+
+def test_a_long_horizon_counts_in_the_choice():
+    # one problem with a long horizon beside 40 small ones with a short one: most of the
+    # time its cluster would run alone, which pays for 300,000 transitions only
+    small = banded_imdp(400, 1, 400 * 201 + 1, eps=0.1, seed=2)
+    for n, k, K, resident in ((700, 450, 200, True), (1000, 990, 500, False)):
+        ms = [banded_imdp(n, 1, n * (k + 1) + 1, eps=0.1, seed=1)] + [small] * 40
+        models = [g.create_model(m) for m in ms]
+        specs = [g.make_spec(horizon=20 if i else K, reach=m.goal) for i, m in enumerate(ms)]
+        assert (_route(models, specs, K)["kernel"] == g.KERNEL_RESIDENT) == resident, n
+        for m in models:
+            m.close()
+
+
+# units a few more than clusters of 16 (7 fit the GPU) or 8 CTAs (15): smaller clusters, all at once
+@pytest.mark.parametrize("n,cluster", [(4, 16), (8, 8), (20, 4)])
+@pytest.mark.parametrize("storage", [g.IMDP_F64, g.IMDP_F32])
+def test_every_unit_has_a_cluster(n, cluster, storage):
+    one = banded_imdp(400, 1, 400 * 201 + 1, eps=0.1, seed=5)
+    m = concat_block_diagonal([one] * n)
+    model = g.create_model(m, dtype=storage)
+    specs = [g.make_spec(horizon=12, reach=m.goal)]
+    r = _route([model], specs, 12)
+    assert (r["kernel"], r["units"], r["cluster"], r["ctas"]) == (g.KERNEL_RESIDENT, n, cluster, n * cluster)
+    _same(_run([model], [m], specs, g.KERNEL_RING), _run([model], [m], specs, g.KERNEL_RULE))
+    model.close()
