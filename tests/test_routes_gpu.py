@@ -247,3 +247,20 @@ def test_every_unit_has_a_cluster(n, cluster, storage):
     assert (r["kernel"], r["units"], r["cluster"], r["ctas"]) == (g.KERNEL_RESIDENT, n, cluster, n * cluster)
     _same(_run([model], [m], specs, g.KERNEL_RING), _run([model], [m], specs, g.KERNEL_RULE))
     model.close()
+
+
+# a state or a few that nothing connects to the model, before, behind and between: they count as part of it
+@pytest.mark.parametrize("where", ["behind", "before", "both", "several"])
+@pytest.mark.parametrize("shape", [(5, 5), (240, 108), (960, 559)])
+def test_detached_states_are_no_unit_of_their_own(shape, where):
+    n, k = shape
+    body = banded_imdp(n, 1, n * (k + 1) + 1, eps=0.1, seed=1)
+    dot = random_imdp(1, 1, 1, seed=2)
+    m = concat_block_diagonal({"behind": [body, dot], "before": [dot, body], "both": [dot, body, dot],
+                               "several": [dot, dot, body, dot, dot, dot]}[where])
+    model, alone = g.create_model(m), _alone(body)
+    specs = [g.make_spec(horizon=20, reach=m.goal)]
+    r = _route([model], specs, 20)
+    assert (r["kernel"], r["units"], r["copied"]) == (alone["kernel"], 1, 1)
+    _same(_run([model], [m], specs, g.KERNEL_RING, policy=True), _run([model], [m], specs, g.KERNEL_RULE, policy=True))
+    model.close()
