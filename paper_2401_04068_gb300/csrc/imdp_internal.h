@@ -481,6 +481,7 @@ struct Session {
   imdp_status plan_grid(cudaStream_t st);
   bool copied = false;  // the plan above keeps the transitions in shared memory
   bool plans_long_steps() const { return resident.n_units > 0 || whole.n_units > 0; }
+  double long_seconds = 0.0;  // an iteration of it, by the cost model
   // The kernel that a step call of n iterations takes, and how many of them one launch runs.
   int32_t step_kernel(int32_t n) const;
   int32_t launch_iterations() const;

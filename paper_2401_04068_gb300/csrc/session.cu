@@ -542,7 +542,9 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, b
     bounds = wide_bounds;
     break;
   }
-  if (std::max(uneven(c), spread(c)) > other) return none();
+  const double mine = std::max(uneven(c), spread(c));
+  if (mine > other) return none();
+  long_seconds = mine / iters;
   std::vector<ResidentUnit> uh(n_units);
   for (int32_t i = 0; i < n_units; ++i) uh[i] = us[i].u;
   ResidentUnit* du = alloc<ResidentUnit>(uh.size());
@@ -608,6 +610,7 @@ imdp_status Session::plan_grid(cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(work, all_of_one.data(), sizeof(int2) * grid, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host vectors go out of scope
   if (e != cudaSuccess) return cuda_status(e, "session plan");
+  long_seconds = 6.5e-6 + m->nnz / (1.0 * grid * 1.9e9);
   whole.units = du;
   whole.work = work;
   whole.n_units = 1;
@@ -814,12 +817,16 @@ int32_t Session::step_kernel(int32_t n) const {
   return resolve_launch(L, &cfg).kernel;
 }
 
+// Iterations of one launch of a long step call. Another stream's grid kernel waits
+// for all SMs together, so a launch takes about 10 ms, which costs nothing that can
+// be measured (cartpole_3840 11.48 ms in one launch and 11.49 so). A launch whose
+// units follow one another on the clusters reads their transitions from memory
+// again and has a last round of its own: about 100 ms (4096 pendulum parts, 65.3 ms
+// in one launch: 67.0 in launches of 30 ms, 69.0 of 10; on 32-bit storage 65.8,
+// 70.9, 74.2; 256 uneven problems 71.4, 74.2, 76.8).
 int32_t Session::launch_iterations() const {
-  // launches of about half a second, so that a long call does not hold the SMs
-  // that another stream's grid kernel waits for
-  int64_t entries = 0;
-  for (const DevModel* m : models) entries += m->nnz;
-  return (int32_t)std::min<int64_t>(50000, 64 + 100000000000ll / std::max<int64_t>(entries, 1));
+  const double most = resident.n_units > resident.clusters ? 0.1 : 0.01;
+  return (int32_t)std::min(50000.0, std::max(16.0, most / std::max(long_seconds, 1e-9)));
 }
 
 imdp_status Session::step(int32_t n, cudaStream_t st) {

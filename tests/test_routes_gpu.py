@@ -6,6 +6,7 @@ import time
 
 import numpy as np
 import pytest
+import torch
 
 import paper_2401_04068_gb300 as g
 from test_resident_gpu import GRID, _lengths, _run, _same
@@ -263,4 +264,26 @@ def test_detached_states_are_no_unit_of_their_own(shape, where):
     r = _route([model], specs, 20)
     assert (r["kernel"], r["units"], r["copied"]) == (alone["kernel"], 1, 1)
     _same(_run([model], [m], specs, g.KERNEL_RING, policy=True), _run([model], [m], specs, g.KERNEL_RULE, policy=True))
+    model.close()
+
+
+# how long one launch of a long step call holds the GPU: about 10 ms, about 100 where the
+# units do not all run at once (four times that, as the estimate is one of a cost model)
+@pytest.mark.parametrize("shape,n,bound", [("small", 40000, 0.04), ("large", 12000, 0.04), ("rounds", 2000, 0.4)])
+def test_launches_are_bounded(shape, n, bound):
+    m = {"small": lambda: banded_imdp(240, 1, 240 * 109 + 1, eps=0.1, seed=1),
+         "large": lambda: banded_imdp(960, 1, 960 * 560 + 1, eps=0.1, seed=1),
+         "rounds": lambda: banded_batch(1000, 200, 1, 200 * 101 + 1, eps=0.1, seed=1)}[shape]()
+    model = g.create_model(m)
+    sess = g.imdp_session_create([model], [g.make_spec(horizon=n, reach=m.goal)])
+    r = g.imdp_session_step_route(sess, n)
+    assert r["kernel"] == (g.KERNEL_GRID if shape == "large" else g.KERNEL_RESIDENT)
+    g.imdp_session_step(sess, 4)
+    torch.cuda.synchronize()
+    t = time.perf_counter()
+    g.imdp_session_step(sess, n - 4)
+    torch.cuda.synchronize()
+    seconds = (time.perf_counter() - t) / g.imdp_session_step_route(sess, n - 4)["launches"]
+    assert seconds <= bound, (seconds, r)
+    sess.close()
     model.close()
