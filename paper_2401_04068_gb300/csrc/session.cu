@@ -549,10 +549,10 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, b
   for (int32_t i = 0; i < n_units; ++i) uh[i] = us[i].u;
   ResidentUnit* du = alloc<ResidentUnit>(uh.size());
   int32_t* db = alloc<int32_t>(bounds.size());
-  if (!du || !db) {
-    resident.n_units = 0;
-    set_error("device allocation failed (session)");
-    return IMDP_ENOMEM;
+  if (!du || !db) {  // no room for the plan: the per-iteration kernels need none
+    mem.release(du);
+    mem.release(db);
+    return none();
   }
   cudaError_t err = cudaMemcpyAsync(du, uh.data(), sizeof(ResidentUnit) * uh.size(), cudaMemcpyHostToDevice, st);
   if (err == cudaSuccess) err = cudaMemcpyAsync(db, bounds.data(), sizeof(int32_t) * bounds.size(), cudaMemcpyHostToDevice, st);
@@ -587,9 +587,10 @@ imdp_status Session::plan_grid(cudaStream_t st) {
   GridUnit u{};
   u.misses = alloc<GridMiss>((size_t)grid * cut.most_cols);
   u.steal = whole.steal = alloc<uint32_t>(4 * (size_t)grid);
-  if (!dc || !dw || !du || !work || !u.misses || !u.steal) {
-    set_error("device allocation failed (session)");
-    return IMDP_ENOMEM;
+  if (!dc || !dw || !du || !work || !u.misses || !u.steal) {  // as above
+    for (void* p : {(void*)dc, (void*)dw, (void*)du, (void*)work, (void*)u.misses, (void*)u.steal}) mem.release(p);
+    whole = GridPlan{};
+    return IMDP_OK;
   }
   u.chunk = dc;
   u.win = dw;
