@@ -197,6 +197,12 @@ IMDP_API imdp_status imdp_model_plan(const imdp_model* m, int32_t* n_tiles, int3
  * that is reset after a timeout runs normally. */
 IMDP_API void imdp_debug_stall_producer(int32_t on);
 
+/* TEST-ONLY hook (no counterpart in the paper): while `on` is nonzero, launches of
+ * the grid kernel report on the host that its CTAs do not fit the GPU together, as
+ * where fewer SMs are given to the process than it was planned for. Sessions and
+ * servers then go on per iteration. Process-wide. */
+IMDP_API void imdp_debug_refuse_cooperative(int32_t on);
+
 /*
  * value_iteration / control_synthesis (Sec. 3.2) on one model.
  *   V_out         double[n_states] (host or device): V_k after the last iteration

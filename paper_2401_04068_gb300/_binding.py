@@ -36,7 +36,7 @@ EXPORTED = [
     "imdp_session_set_launch", "imdp_session_get_launch", "imdp_session_autotune", "imdp_session_plan",
     "imdp_create_csc_f32", "imdp_model_exact_columns", "imdp_session_residual", "imdp_session_stop_threshold",
     "imdp_server_set_launch", "imdp_server_stats", "imdp_value_iteration_polished", "imdp_session_step_route",
-    "imdp_server_launches",
+    "imdp_server_launches", "imdp_debug_refuse_cooperative",
 ]
 
 
@@ -717,6 +717,11 @@ def imdp_model_plan(model: Model):
 def imdp_debug_stall_producer(on: bool):
     """Test hook: step launches leave every consumer wait unsatisfied (see include/imdp.h)."""
     load().imdp_debug_stall_producer(1 if on else 0)
+
+
+def imdp_debug_refuse_cooperative(on: bool):
+    """Test-only: launches of the grid kernel report that they do not fit the GPU."""
+    load().imdp_debug_refuse_cooperative(1 if on else 0)
 
 
 # ---------------------------------------------------------------- model files (Sec. 3.1)

@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 
 #include "resident.cuh"
@@ -906,17 +907,20 @@ bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut&
   return grid_bytes(out, f32) <= kResidentSmem;
 }
 
+std::atomic<int> g_refuse_cooperative{0};
+
 cudaError_t grid_prepare(const GridPlan& R) {
   cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(grid_kernel(R)),
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentSmem);
   int n = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, grid_kernel(R), kGridThreads, R.smem);
-  return e == cudaSuccess && n < 1 ? cudaErrorInvalidConfiguration : e;
+  return e == cudaSuccess && n * bellman_grid() < R.grid ? cudaErrorCooperativeLaunchTooLarge : e;
 }
 
 // `n_iters` 0: each unit's own number of iterations.
 cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t n_iters, cudaStream_t st) {
   if (n_iters < 0) return cudaSuccess;
+  if (g_refuse_cooperative.load(std::memory_order_relaxed)) return cudaErrorCooperativeLaunchTooLarge;
   cudaError_t e = cudaMemsetAsync(R.steal, 0, sizeof(uint32_t) * 4 * (size_t)R.steal_ctas, st);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t c;

@@ -373,6 +373,8 @@ struct TraceRange {
 // Test hook (imdp_debug_stall_producer): launches made while set leave the
 // consumers' waits unsatisfied, to exercise the bounded-wait error path.
 extern std::atomic<int> g_stall_producer;
+// Test hook (imdp_debug_refuse_cooperative): the grid kernel's launches report that they do not fit.
+extern std::atomic<int> g_refuse_cooperative;
 // One Bellman iteration: the wide-state kernel (on `side`, beside the tiled one,
 // when given) and the tiled kernel; the last CTA of the two advances the
 // iteration state.
@@ -395,6 +397,8 @@ cudaError_t launch_bellman_resident(const StepLaunch& L, const ResidentPlan& R, 
 size_t grid_bytes(const GridCut& c, bool f32);
 bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut& out);
 cudaError_t grid_prepare(const GridPlan& R);
+// cudaErrorCooperativeLaunchTooLarge when the CTAs do not fit the device together
+// (fewer SMs are given to the process than it was planned for).
 cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t n_iters, cudaStream_t st);
 constexpr int kGridThreads = 768;  // of a CTA
 // CTAs of the persistent tiled kernel: one per SM.

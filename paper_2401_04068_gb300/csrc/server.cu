@@ -659,6 +659,7 @@ struct Server {
     std::vector<int2> work;
     int32_t count = 0;  // slots [0, count) are in the launch
     bool stale = true;  // the per-iteration launches' tables are older than the slots
+    bool refused = false;  // a shared launch did not fit the device
     bool fits = true;   // the running requests fit the grid kernel together, as far as known
     while (true) {
       bool changed = false;
@@ -709,7 +710,7 @@ struct Server {
       {
         std::lock_guard<std::mutex> lk(mu);
         lc = cfg;
-        if (lc.by_rule() && fits) {
+        if (lc.by_rule() && fits && !refused) {
           // planned again when a quarter of the CTAs have run out of work
           grid_kernel = gplan.n_units > 0 && !changed && plan_quantum(work) * 4 > gplan.grid * 3;
           if (!grid_kernel) {
@@ -763,6 +764,11 @@ struct Server {
       if (e == cudaSuccess) e = cudaEventRecord(ev0, stream);
       if (grid_kernel) {
         if (e == cudaSuccess) e = launch_bellman_grid(L, gplan, 0, stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {  // nothing was launched: per iteration from here on
+          cudaGetLastError();
+          refused = true;
+          continue;
+        }
       } else {
         for (int i = 0; i < chunk && e == cudaSuccess; ++i) e = launch_bellman_step(L, grid, stream, &side, &lc);
       }

@@ -835,6 +835,7 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
   TraceRange trace("imdp session step");
   cudaError_t e = cudaSuccess;
   const int32_t kernel = step_kernel(n);
+  int32_t done = 0;
   if (kernel == kKernelTiny) {
     // one small problem, few iterations: all of them in one launch of one CTA
     e = launch_bellman_tiny(L, n, models[0]->lg32 != nullptr, st);
@@ -846,19 +847,19 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
   if (kernel == kKernelResident || kernel == kKernelGrid) {
     // by rule: all n iterations in one launch, or in a few
     const int32_t most = launch_iterations();
-    for (int32_t done = 0; done < n && e == cudaSuccess;) {
+    while (done < n && e == cudaSuccess) {
       const int32_t some = std::min(most, n - done);
       e = kernel == kKernelResident ? launch_bellman_resident(L, resident, some, st)
                                     : launch_bellman_grid(L, whole, some, st);
-      done += some;
+      if (e == cudaSuccess) done += some;
     }
-    if (e != cudaSuccess) return cuda_status(e, "bellman step");
-    launches += n;
-    launched_since_reset += n;
-    return IMDP_OK;
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // nothing was launched: per iteration from here on
+      cudaGetLastError();
+      whole.n_units = 0;
+      e = cudaSuccess;
+    }
   }
-  int32_t done = 0;
-  if (st != nullptr && n >= kGraphChunk) {
+  if (e == cudaSuccess && st != nullptr && n - done >= kGraphChunk) {
     if (!graph) {
       cudaGraph_t g = nullptr;
       graph_stalled = g_stall_producer.load() != 0;
