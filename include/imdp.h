@@ -188,9 +188,9 @@ IMDP_API imdp_status imdp_model_plan(const imdp_model* m, int32_t* n_tiles, int3
 
 /* TEST-ONLY hook for failure detection (no counterpart in the paper; never
  * call it in production code). While `on` is nonzero, step launches of the
- * ring kernel (launch configuration kernel 1) issue no tile copies: every
- * consumer wait runs into its bound
- * (about 2 s), the kernel records the error and returns, and the next read of
+ * ring kernel (launch configuration kernel 1) issue no tile copies, and the first
+ * CTA of a problem on the grid kernel never arrives at its barriers: every wait
+ * for them runs into its bound (about 2 s), the kernel records the error and returns, and the next read of
  * the session reports IMDP_ETIMEOUT; the CUDA context stays usable. The switch
  * is process-wide; imdp_session_reset turns it off again (and drops the
  * session's captured graph, which may hold stalled launches), so a session

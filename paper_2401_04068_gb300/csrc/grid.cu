@@ -70,6 +70,7 @@ struct GridShared {
   int32_t n32, n_cols, n_own, n_win;
   uint32_t n_free, n_lc;
   int32_t copied;
+  int32_t stall;  // test hook: the unit's first CTA never arrives at its barriers
   EntryCopy copy;
   int32_t ok;
   uint32_t states, v;                  // the unit's layout
@@ -714,7 +715,7 @@ __device__ __forceinline__ int32_t grid_iterate(const Problem& P, const GridTabl
       }
       if (list) atomicAdd(&ctl->misses[k & 3], list);
       steal[me] = list;
-      grid_arrive(ctl);
+      if (!(S.stall && me == 0)) grid_arrive(ctl);
     }
     if (!settle_misses<f32, copied>(P, T, D, Vg, scratch, k, barrier * (uint32_t)S.unit.ctas, list, lane, warp, S)) return -1;
     if (S.total != 0) {
@@ -774,8 +775,9 @@ __global__ void __launch_bounds__(kGridThreads, 1) bellman_grid_kernel(StepLaunc
           cells += w.len;
         }
         S.chunk_own[n_chunks] = own;
-      S.states = lay.states;
-      S.v = lay.v;
+        S.states = lay.states;
+        S.v = lay.v;
+        S.stall = L.stall;
         S.n_win = U.one_window ? min(1, n_chunks) : n_chunks;
       }
       __syncthreads();
@@ -934,7 +936,9 @@ cudaError_t launch_bellman_grid(const StepLaunch& L, const GridPlan& R, int32_t 
   attr.val.cooperative = 1;
   c.attrs = &attr;
   c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, grid_kernel(R), L, R, n_iters);
+  StepLaunch l = L;
+  l.stall = g_stall_producer.load(std::memory_order_relaxed);
+  return cudaLaunchKernelEx(&c, grid_kernel(R), l, R, n_iters);
 }
 
 }  // namespace imdp

@@ -270,7 +270,7 @@ struct StepLaunch {
   unsigned int* win_cnt;
   int32_t n_items;
   int32_t grid_total;  // CTAs of both step kernels in this launch (set by the launcher)
-  int32_t stall;       // test hook: the producer issues nothing, so every wait runs out
+  int32_t stall;       // test hook: a producer issues nothing, a CTA does not arrive, so every wait runs out
 };
 
 // The resident kernel (resident.cu): all iterations of a step call in one

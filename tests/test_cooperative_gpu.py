@@ -69,3 +69,31 @@ def test_servers_go_on_per_iteration():
         g.imdp_debug_refuse_cooperative(False)
     server.close()
     model.close()
+
+
+def test_bounded_grid_barrier_reports_timeout_and_context_survives():
+    m, model = _case()
+    spec = g.make_spec(horizon=40, reach=m.goal)
+    ref, _ = _ring(model, spec)
+    sess = g.imdp_session_create([model], [spec])
+    assert g.imdp_session_step_route(sess, 20)["kernel"] == g.KERNEL_GRID
+    V = np.zeros(m.n_states)
+    g.imdp_debug_stall_producer(True)
+    try:
+        t = time.time()
+        g.imdp_session_step(sess, 20)
+        st = g.imdp_session_read(sess, 0, V, check=False)
+        elapsed = time.time() - t
+    finally:
+        g.imdp_debug_stall_producer(False)
+    assert st == g.IMDP_ETIMEOUT
+    assert elapsed < 30.0  # bounded: the waits gave up on their own
+    assert not V.any()  # no output of a failed run
+    # the same session, reset, runs normally afterwards
+    g.imdp_session_reset(sess)
+    g.imdp_session_step(sess, 40)
+    raw, k = g.imdp_session_checkpoint(sess, 0)
+    assert k == 40
+    np.testing.assert_array_equal(raw, ref)
+    sess.close()
+    model.close()
