@@ -999,7 +999,19 @@ imdp_status Session::read_all(double* const* V_out, int32_t* k_out, cudaStream_t
   std::sort(spans.begin(), spans.end());
   bool apart = count <= 65535;  // (the launch's limit)
   for (int p = 1; p < count; ++p) apart = apart && spans[p].first >= spans[p - 1].second;
-  if (!apart) {  // outputs that overlap are written one problem after the other
+  ExportItem* d_items = nullptr;
+  double* stage = nullptr;
+  cudaError_t e = cudaSuccess;
+  if (apart) {
+    e = cudaMalloc(&d_items, sizeof(ExportItem) * count);
+    if (e == cudaSuccess && host > 0) e = cudaMalloc(&stage, sizeof(double) * host);
+    apart = e == cudaSuccess;
+  }
+  // outputs that overlap are written one problem after the other, and so are
+  // those that find no room together
+  if (!apart) {
+    cudaGetLastError();
+    cudaFree(d_items);
     imdp_status worst = IMDP_OK;
     for (int p = 0; p < count; ++p) {
       int32_t k = 0;
@@ -1011,10 +1023,6 @@ imdp_status Session::read_all(double* const* V_out, int32_t* k_out, cudaStream_t
     return worst;
   }
   std::vector<ExportItem> items(count);
-  ExportItem* d_items = nullptr;
-  double* stage = nullptr;
-  cudaError_t e = cudaMalloc(&d_items, sizeof(ExportItem) * count);
-  if (e == cudaSuccess && host > 0) e = cudaMalloc(&stage, sizeof(double) * host);
   for (int p = 0; p < count; ++p) {
     const Problem& P = probs_h[p];
     const int32_t k = s[p].done ? s[p].k_final : s[p].iter;

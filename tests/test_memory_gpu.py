@@ -66,3 +66,32 @@ def test_a_session_without_room_for_its_plan():
     assert route not in (g.KERNEL_GRID, g.KERNEL_RESIDENT) and k == 12
     np.testing.assert_array_equal(raw, ref)
     model.close()
+
+
+def test_batch_results_without_room_for_all_of_them():
+    # 32 models of a million absorbing states: their results are 256 MB together, 8 MB each
+    n = 1000000
+    ptr = np.arange(n + 1, dtype=np.int32)
+    one = np.ones(n)
+    model = g.imdp_create_csc(n, n, n, ptr, ptr, ptr[:n], one, one)
+    count = 32
+    specs = [g.make_spec(horizon=2 + i % 3, reach=np.arange(i, n, 7, dtype=np.int32)) for i in range(count)]
+    outs = [np.full(n, -1.0) for _ in range(count)]
+    g.imdp_value_iteration_batch([model] * count, specs, outs, [0] * count)
+    want = [o.copy() for o in outs]
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    sess = g.imdp_session_create([model] * count, specs)
+    need = free - torch.cuda.mem_get_info()[0]
+    sess.close()
+    for o in outs:
+        o[:] = -1.0
+    ks = [0] * count
+    with Leave(need + 24 * MB):
+        assert torch.cuda.mem_get_info()[0] < need + 36 * MB
+        assert g.imdp_value_iteration_batch([model] * count, specs, outs, ks) == g.IMDP_OK
+    assert ks == [2 + i % 3 for i in range(count)]
+    for i, (o, w) in enumerate(zip(outs, want)):
+        np.testing.assert_array_equal(o, w)
+        np.testing.assert_array_equal(o, (np.arange(n) % 7 == i % 7) & (np.arange(n) >= i))
+    model.close()
