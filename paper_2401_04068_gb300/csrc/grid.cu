@@ -40,6 +40,7 @@ constexpr int kGridWarps = kGridThreads / 32;
 // Misses that a CTA settles by itself, two rounds of its warps; more are listed
 // for all CTAs, which costs two more barriers.
 constexpr uint32_t kGridFewMisses = 2 * kGridWarps;
+constexpr int32_t kGridMostCols = 5000;  // of one CTA
 constexpr int kSettleTrips = 4;  // trips in flight while a missed column is settled
 constexpr int kGridBuckets = 256;  // length classes of the column order, as in the resident kernel
 constexpr long long kGridWaitCycles = 4000000000ll;  // ~2 s at 2 GHz: bound of the grid barrier's wait
@@ -843,6 +844,20 @@ size_t grid_bytes(const GridCut& c, bool f32) {
   return (size_t)l.data + l.q;
 }
 
+// Fewer CTAs than this cannot hold the model's free columns and states, however it
+// is cut (the windows are left out).
+int32_t grid_least_ctas(const DevModel* m, const uint8_t* fx) {
+  int64_t cols = 0, own = 0;
+  for (int32_t s = 0; s < m->n_states; ++s)
+    if (!fx[s]) {
+      cols += m->h_stateptr[s + 1] - m->h_stateptr[s];
+      own += 1;
+    }
+  const int64_t bytes = cols * (int64_t)(sizeof(GridCol) + sizeof(uint64_t)) + own * (int64_t)sizeof(GridState);
+  const int64_t room = (int64_t)kResidentSmem - (int64_t)kGridColumnsAt;
+  return (int32_t)std::max<int64_t>({1, (bytes + room - 1) / room, (cols + kGridMostCols - 1) / kGridMostCols});
+}
+
 // Cuts the states of a model (`fx`: those the property fixes) into chunks for
 // `ctas` CTAs. False when no CTA's share fits.
 bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut& out) {
@@ -901,7 +916,7 @@ bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut&
   most_cells = std::min<int64_t>(most_cells, n);
   const int64_t most_cols = *std::max_element(cols.begin(), cols.end());
   const int64_t most_own = *std::max_element(own.begin(), own.end());
-  if (most_cells > 60000 || most_cols > 5000 || most_own > 60000) return false;
+  if (most_cells > 60000 || most_cols > kGridMostCols || most_own > 60000) return false;
   out.most_cells = (int32_t)most_cells;
   out.most_cols = (int32_t)most_cols;
   out.most_own = (int32_t)most_own;

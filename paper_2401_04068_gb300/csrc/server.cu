@@ -121,7 +121,10 @@ struct Request {
   bool planned = false;        // the two below are set (on the first per-iteration launch)
   std::vector<Tile> tiles;     // tile plan under that configuration (fixed states left out)
   std::vector<int32_t> wide;   // wide states
-  int32_t least = 1;           // CTAs the grid kernel needs for it, as far as known
+  // CTAs the grid kernel needs for it, as far as known (0: not looked at). Kept, so
+  // that a mix that does not fit is seen at once the next time (12 requests of 300,000
+  // columns: 9 cuts of each took 15 ms, again after every arrival and retirement)
+  int32_t least = 0;
   // iterations left (an infinite horizon: a guess, it ends by itself), and what
   // one of them costs the grid kernel on one SM
   int32_t left() const {
@@ -432,8 +435,9 @@ struct Server {
     return true;
   }
 
-  // Plans the running requests for the grid kernel (called with mu held: the
-  // arena). False when they do not fit it together.
+  // Plans the running requests for the grid kernel. False when they do not fit it
+  // together. (Not under the mutex: slots and arena are the worker's own, and cutting
+  // the models takes milliseconds.)
   bool plan_grid(int32_t count) {
     drop_grid();
     std::vector<Request*> rs;
@@ -452,6 +456,8 @@ struct Server {
     // every CTA waits for the one with the most new requests (2000 requests/s, 360
     // running: 0.88e11 transition-updates/s shared, 0.89 to 0.96e11 per iteration)
     if (rs.empty() || (int)rs.size() > grid / 2) return false;
+    for (Request* r : rs)
+      if (r->least == 0) r->least = grid_least_ctas(r->model, r->fixed.data());
     std::stable_sort(rs.begin(), rs.end(), [](const Request* a, const Request* b) {
       return a->work_left() * a->seconds(1) > b->work_left() * b->seconds(1);
     });
@@ -710,16 +716,16 @@ struct Server {
       {
         std::lock_guard<std::mutex> lk(mu);
         lc = cfg;
-        if (lc.by_rule() && fits && !refused) {
-          // planned again when a quarter of the CTAs have run out of work
-          grid_kernel = gplan.n_units > 0 && !changed && plan_quantum(work) * 4 > gplan.grid * 3;
-          if (!grid_kernel) {
-            grid_kernel = fits = plan_grid(count);
-            if (grid_kernel) plan_quantum(work);
-          }
-        }
-        if (!grid_kernel) drop_grid();
       }
+      if (lc.by_rule() && fits && !refused) {
+        // planned again when a quarter of the CTAs have run out of work
+        grid_kernel = gplan.n_units > 0 && !changed && plan_quantum(work) * 4 > gplan.grid * 3;
+        if (!grid_kernel) {
+          grid_kernel = fits = plan_grid(count);
+          if (grid_kernel) plan_quantum(work);
+        }
+      }
+      if (!grid_kernel) drop_grid();
       if (!grid_kernel && stale && e == cudaSuccess) {
         const imdp_status st = upload_tables(count);
         if (st != IMDP_OK) {
