@@ -747,6 +747,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) bellman_grid_kernel(StepLaunc
       reinterpret_cast<uint32_t*>(&S.unit)[tid] = reinterpret_cast<const uint32_t*>(R.units + u)[tid];
     __syncthreads();
     const GridUnit& U = S.unit;
+    if (n_iters == 0 && U.iters == 0) continue;  // not in this launch
     const GridLayout lay = grid_layout(U.most_cols, U.most_own, U.most_cells, cell);
     const uint32_t end = R.smem & ~15u;
     const GridTable T{end};

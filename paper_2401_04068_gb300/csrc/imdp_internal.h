@@ -340,7 +340,7 @@ struct GridUnit {
   int32_t single;          // every state has one action
   int32_t most_cols, most_own, most_cells;  // of one CTA
   int32_t max_col;
-  int32_t iters;           // iterations in this launch, when the launch does not say
+  int32_t iters;           // iterations in this launch (0: none), when the launch does not say
   int32_t pad;
 };
 struct GridPlan {
