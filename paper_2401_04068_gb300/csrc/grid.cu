@@ -846,14 +846,15 @@ size_t grid_bytes(const GridCut& c, bool f32) {
 }
 
 // Fewer CTAs than this cannot hold the model's free columns and states, however it
-// is cut (the windows are left out).
-int32_t grid_least_ctas(const DevModel* m, const uint8_t* fx) {
+// is cut (the windows are left out). `columns`: the free ones.
+int32_t grid_least_ctas(const DevModel* m, const uint8_t* fx, int64_t* columns) {
   int64_t cols = 0, own = 0;
   for (int32_t s = 0; s < m->n_states; ++s)
     if (!fx[s]) {
       cols += m->h_stateptr[s + 1] - m->h_stateptr[s];
       own += 1;
     }
+  *columns = cols;
   const int64_t bytes = cols * (int64_t)(sizeof(GridCol) + sizeof(uint64_t)) + own * (int64_t)sizeof(GridState);
   const int64_t room = (int64_t)kResidentSmem - (int64_t)kGridColumnsAt;
   return (int32_t)std::max<int64_t>({1, (bytes + room - 1) / room, (cols + kGridMostCols - 1) / kGridMostCols});

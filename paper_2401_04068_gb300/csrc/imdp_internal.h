@@ -395,7 +395,7 @@ cudaError_t launch_bellman_resident(const StepLaunch& L, const ResidentPlan& R, 
 // grid.cu
 // Shared memory of one CTA.
 size_t grid_bytes(const GridCut& c, bool f32);
-int32_t grid_least_ctas(const DevModel* m, const uint8_t* fx);
+int32_t grid_least_ctas(const DevModel* m, const uint8_t* fx, int64_t* columns);
 bool plan_grid_unit(const DevModel* m, const uint8_t* fx, int32_t ctas, GridCut& out);
 cudaError_t grid_prepare(const GridPlan& R);
 // cudaErrorCooperativeLaunchTooLarge when the CTAs do not fit the device together

@@ -75,6 +75,11 @@ class Arena {
     }
   }
   size_t size() const { return size_; }
+  size_t largest() const {
+    size_t most = 0;
+    for (const auto& f : free_) most = std::max(most, f.second);
+    return most;
+  }
 
  private:
   size_t size_;
@@ -125,6 +130,7 @@ struct Request {
   // that a mix that does not fit is seen at once the next time (12 requests of 300,000
   // columns: 9 cuts of each took 15 ms, again after every arrival and retirement)
   int32_t least = 0;
+  int64_t columns = 0;  // free ones, looked at with it
   // iterations left (an infinite horizon: a guess, it ends by itself), and what
   // one of them costs the grid kernel on one SM
   int32_t left() const {
@@ -477,8 +483,14 @@ struct Server {
     // every CTA waits for the one with the most new requests (2000 requests/s, 360
     // running: 0.88e11 transition-updates/s shared, 0.89 to 0.96e11 per iteration)
     if (rs.empty() || (int)rs.size() > grid / 2) return false;
-    for (Request* r : rs)
-      if (r->least == 0) r->least = grid_least_ctas(r->model, r->fixed.data());
+    size_t lists = 0;
+    for (Request* r : rs) {
+      if (r->least == 0) r->least = grid_least_ctas(r->model, r->fixed.data(), &r->columns);
+      lists += r->columns * sizeof(GridMiss);
+    }
+    // no room for the lists of missed columns (most of the block below): the models
+    // need not be cut to see it
+    if (lists > arena.largest()) return false;
     std::stable_sort(rs.begin(), rs.end(), [](const Request* a, const Request* b) {
       return a->work_left() * a->seconds(1) > b->work_left() * b->seconds(1);
     });

@@ -61,3 +61,26 @@ def test_callers_do_not_wait_for_a_plan():
         for o in outs[i::3]:
             np.testing.assert_array_equal(o, V)
         models[i].close()
+
+
+def test_no_cuts_for_a_plan_that_has_no_room():
+    # the budget holds the requests and little more; the lists of missed columns (64 B
+    # a column) find no room, which the worker sees without cutting the models
+    n, count = 45000, 10
+    ms = [banded_imdp(n, 1, n * 7 + 1, eps=0.1, seed=200 + i) for i in range(count)]
+    models = [g.create_model(m) for m in ms]
+    host_ms = 1e9
+    for _ in range(3):
+        server = g.imdp_server_create(count * (37 * (n + 1)) + (1 << 20))
+        tickets = [g.imdp_server_submit(server, x, g.make_spec(horizon=40 + 16 * i, reach=m.goal))
+                   for i, (x, m) in enumerate(zip(models, ms))]
+        for t in tickets:
+            assert g.imdp_server_wait(server, t, 120000.0, np.zeros(n + 1)) == g.IMDP_OK
+        time.sleep(0.1)
+        s, launches = g.imdp_server_stats(server), g.imdp_server_launches(server)
+        host_ms = min(host_ms, s["wall_ms"] - s["device_ms"])
+        server.close()
+    assert launches["per_iteration"] > 0
+    assert host_ms < 5.5, host_ms  # 8.0 when it cuts them
+    for x in models:
+        x.close()
