@@ -500,6 +500,7 @@ struct Session {
   int64_t launched_since_reset = 0;
   Buffers mem{get_memory, put_memory};
   // the buffers of the installed launch plan
+  bool plan_lost = false;  // a plan change failed halfway
   Buffers::Plan tiles_mem, wide_mem, items_mem, item_end_mem, win_mem;
 
   static void* get_memory(size_t bytes);

@@ -622,6 +622,7 @@ imdp_status Session::install_plan(const std::vector<Tile>& tl, const std::vector
                                   bool slice) {
   cudaError_t e = cudaStreamSynchronize(st);  // launches in flight may still read the old plan
   if (e != cudaSuccess) return cuda_status(e, "session plan");
+  plan_lost = true;  // until the new one is complete: a step must not read the old one's memory
   mem.drop(items_mem);
   mem.drop(item_end_mem);
   mem.drop(win_mem);
@@ -690,6 +691,7 @@ imdp_status Session::install_plan(const std::vector<Tile>& tl, const std::vector
     cudaGraphExecDestroy(graph);
     graph = nullptr;
   }
+  plan_lost = false;
   return IMDP_OK;
 }
 
@@ -758,7 +760,7 @@ void Session::build_plan(const LaunchConfig& c, std::vector<Tile>& tl, std::vect
 imdp_status Session::set_launch(const LaunchConfig& c, cudaStream_t st) {
   const LaunchConfig old = resolve_launch(L, &cfg), now = resolve_launch(L, &c);
   const bool slice = now.kernel == kKernelSlice;
-  if (now.tile_entries != old.tile_entries || now.wide_col != old.wide_col || slice != (old.kernel == kKernelSlice)) {
+  if (plan_lost || now.tile_entries != old.tile_entries || now.wide_col != old.wide_col || slice != (old.kernel == kKernelSlice)) {
     if (slice) {
       imdp_status r = prepare_slices(st);
       if (r != IMDP_OK) return r;
@@ -858,6 +860,10 @@ imdp_status Session::step(int32_t n, cudaStream_t st) {
       whole.n_units = 0;
       e = cudaSuccess;
     }
+  }
+  if (done < n && plan_lost) {
+    set_error("the session has no launch plan (a change of its configuration found no memory); set one");
+    return IMDP_ENOMEM;
   }
   if (e == cudaSuccess && st != nullptr && n - done >= kGraphChunk) {
     if (!graph) {

@@ -1,6 +1,11 @@
 """Little device memory left: what the per-iteration kernels and one-by-one reads
 can do in it is done. The GPU's memory is taken by tensors; every kernel has run
-before, so nothing is loaded meanwhile."""
+before, so nothing is loaded meanwhile. Each case has a process of its own, since the
+memory that a process's pool keeps is given back when an allocation needs it."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -37,7 +42,7 @@ class Leave:
         torch.cuda.empty_cache()
 
 
-def test_a_session_without_room_for_its_plan():
+def session_without_room_for_its_plan():
     # the grid kernel's lists of missed columns (64 B a column) do not fit
     m = banded_imdp(200000, 2, 200000 * 2 * 6 + 1, eps=0.1, seed=1)
     model = g.create_model(m)
@@ -68,7 +73,7 @@ def test_a_session_without_room_for_its_plan():
     model.close()
 
 
-def test_batch_results_without_room_for_all_of_them():
+def batch_results_without_room_for_all_of_them():
     # 32 models of a million absorbing states: their results are 256 MB together, 8 MB each
     n = 1000000
     ptr = np.arange(n + 1, dtype=np.int32)
@@ -95,3 +100,40 @@ def test_batch_results_without_room_for_all_of_them():
         np.testing.assert_array_equal(o, w)
         np.testing.assert_array_equal(o, (np.arange(n) % 7 == i % 7) & (np.arange(n) >= i))
     model.close()
+
+
+def plan_change_without_room():
+    # one tile a state: a table of 36 MB, which does not fit; steps then report that
+    # there is no plan (the old one's memory is gone) until one is set
+    n = 1000000
+    ptr = np.arange(n + 1, dtype=np.int32)
+    one = np.ones(n)
+    model = g.imdp_create_csc(n, n, n, ptr, ptr, ptr[:n], one, one)
+    spec = g.make_spec(horizon=9, reach=np.arange(0, n, 3, dtype=np.int32))
+    sess = g.imdp_session_create([model], [spec])
+    g.imdp_session_set_launch(sess, kernel=g.KERNEL_RING)
+    g.imdp_session_step(sess, 3)
+    with Leave(12 * MB):
+        with pytest.raises(g.ImdpError) as e:
+            g.imdp_session_set_launch(sess, kernel=g.KERNEL_RING, tile_entries=1)
+        assert e.value.status == g.IMDP_ENOMEM
+        with pytest.raises(g.ImdpError) as e:
+            g.imdp_session_step(sess, 1)
+        assert e.value.status == g.IMDP_ENOMEM
+    g.imdp_session_set_launch(sess, kernel=g.KERNEL_RING)
+    g.imdp_session_run(sess)
+    V, k = np.zeros(n), [0]
+    assert g.imdp_session_read(sess, 0, V, k) == g.IMDP_OK and k[0] == 9
+    np.testing.assert_array_equal(V, np.arange(n) % 3 == 0)
+    sess.close()
+    model.close()
+
+
+@pytest.mark.parametrize("case", ["session_without_room_for_its_plan", "batch_results_without_room_for_all_of_them",
+                                  "plan_change_without_room"])
+def test_little_memory(case):
+    here = os.path.dirname(os.path.abspath(__file__))
+    torch.cuda.empty_cache()
+    code = f"import sys; sys.path[:0] = [{os.path.dirname(here)!r}, {here!r}]; import test_memory_gpu as t; t.{case}()"
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stdout + out.stderr
