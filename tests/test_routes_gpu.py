@@ -287,3 +287,35 @@ def test_launches_are_bounded(shape, n, bound):
     assert seconds <= bound, (seconds, r)
     sess.close()
     model.close()
+
+
+# few, very long columns on 32-bit storage whose bounds are mostly kept exact: the
+# per-iteration kernels are the faster ones there
+@pytest.mark.parametrize("n,k,grid", [(3840, 2227, False), (3000, 1500, True)])
+def test_long_exact_columns_stay_per_iteration(n, k, grid):
+    m = banded_imdp(n, 1, n * (k + 1) + 1, eps=0.1, seed=1)
+    model = g.create_model(m, dtype=g.IMDP_F32)
+    exact = g.imdp_model_exact_columns(model)[1] / m.nnz
+    spec = g.make_spec(horizon=100, reach=m.goal)
+    kernel = _route([model], [spec], 100)["kernel"]
+    assert (kernel == g.KERNEL_GRID) == grid and exact > (0.6 if grid else 0.8), exact
+    assert _alone(m, 100)["kernel"] == g.KERNEL_GRID  # on 64-bit storage
+
+    def seconds(**launch):
+        sess = g.imdp_session_create([model], [spec])
+        if launch:
+            g.imdp_session_set_launch(sess, **launch)
+        best = 1.0
+        for _ in range(4):
+            g.imdp_session_reset(sess)
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            g.imdp_session_step(sess, 100)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t)
+        sess.close()
+        return best
+
+    # the rule's choice is no slower than the kernel it took before there was a grid kernel
+    assert seconds() <= 1.05 * seconds(kernel=g.KERNEL_DIRECT, ctas_per_sm=3, tile_entries=1024)
+    model.close()
