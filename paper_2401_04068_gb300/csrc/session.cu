@@ -832,9 +832,16 @@ int32_t Session::step_kernel(int32_t n) const {
 // units follow one another on the clusters reads their transitions from memory
 // again and has a last round of its own: about 100 ms (4096 pendulum parts, 65.3 ms
 // in one launch: 67.0 in launches of 30 ms, 69.0 of 10; on 32-bit storage 65.8,
-// 70.9, 74.2; 256 uneven problems 71.4, 74.2, 76.8).
+// 70.9, 74.2; 256 uneven problems 71.4, 74.2, 76.8), and 100 times as long as that
+// reading takes (10,000 uneven problems, 32 GB: 2.30 s in launches of half a second,
+// 2.39 of a tenth).
 int32_t Session::launch_iterations() const {
-  const double most = resident.n_units > resident.clusters ? 0.1 : 0.01;
+  double most = 0.01;
+  if (resident.n_units > resident.clusters) {
+    double bytes = 0.0;
+    for (const DevModel* m : models) bytes += m->nnz * (m->lg32 ? 12.0 : 20.0);
+    most = std::max(0.1, 100.0 * bytes / 6.8e12);
+  }
   return (int32_t)std::min(50000.0, std::max(16.0, most / std::max(long_seconds, 1e-9)));
 }
 
