@@ -269,14 +269,15 @@ def run_ours(args, rank, world, local_rank):
     sess = g.imdp_session_create([model], [spec], want_policy=[1] if args.policy else None, stream=stream)
     # tuned on the query's own iterations: early iterations (many threshold
     # searches) and late ones (warm starts) favour different kernels
-    launch = apply_launch(g, sess, args, stream, min(args.horizon, 200) if not args.infinite else 64)
+    call = 32 if args.infinite else args.horizon  # iterations of a step call
+    launch = apply_launch(g, sess, args, stream, min(args.horizon, 200) if not args.infinite else 64, call)
 
     def one_step(ev=None):
         g.imdp_session_reset(sess, stream)
         if ev is not None:
             ev[0].record(stream)
         if args.infinite:
-            g.imdp_session_run(sess, 32, stream)  # to convergence (max |V_k - V_k-1| < eps)
+            g.imdp_session_run(sess, call, stream)  # to convergence (max |V_k - V_k-1| < eps)
         else:
             g.imdp_session_step(sess, args.horizon, stream)
         if ev is not None:
@@ -354,10 +355,10 @@ def run_ours(args, rank, world, local_rank):
     launch_ms = kernel_ms / max(1, launches)  # per launched iteration (includes any past convergence)
     n_tiles, n_wide, wide_entries = g.imdp_session_plan(sess)
     wide_share = wide_entries / max(1, m.nnz)
-    by_rule = launch["chosen_by"] == "rule"
-    kernel = "bellman_wide_kernel" if wide_share > 0.5 and not by_rule else kernel_name(launch)
-    achieved = alg_bytes / (launch_ms / 1e3) / 1e9
-    traffic = None if by_rule else recorded_traffic(args.workload + ("" if args.dtype == "f64" else ":f32"))
+    per_iteration = launch["route"]["kernel"] in KERNEL_NAMES
+    kernel = "bellman_wide_kernel" if wide_share > 0.5 and per_iteration else kernel_name(launch)
+    traffic = recorded_traffic(args.workload + ("" if args.dtype == "f64" else ":f32")) if per_iteration else None
+    calls = -(-iters // call)  # step calls of a step
     cfg = workload_config(args.workload, m, args.horizon)
     metric = METRIC
     if args.infinite:
@@ -387,16 +388,16 @@ def run_ours(args, rank, world, local_rank):
         if (args.workload == "pimdp2" and args.horizon == 200 and not args.infinite and not args.policy) else None,
         "dtype": "u32" if args.dtype == "f32" else "u64", "data": "synthetic (seeded banded IMDPs shaped like the paper's benchmark table)",
         "config": cfg,
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": traffic, "peak_kind": peak_kind, "kernel": kernel,
-                     "algorithmic_bytes_per_launch": alg_bytes, "avg_launch_ms": launch_ms,
-                     "plan": {"tiles": n_tiles, "wide_states": n_wide, "wide_entry_share": wide_share,
-                              "launch": launch},
-                     "timing": "CUDA events around each step's launches (both step kernels) / iterations"},
+        "roofline": dict(roofline(launch, alg_bytes * launches, alg_bytes * args.steps * calls * launch["route"]["launches"],
+                                  alg_bytes, kernel_ms / 1e3, peak),
+                         traffic=traffic, peak_kind=peak_kind, kernel=kernel,
+                         algorithmic_bytes_per_iteration=alg_bytes, avg_iteration_ms=launch_ms,
+                         plan={"tiles": n_tiles, "wide_states": n_wide, "wide_entry_share": wide_share,
+                               "launch": launch},
+                         timing="CUDA events around each step's launches / iterations"),
         "clocks": clk,
-        # step kernels (per iteration, two when the model has wide states; by rule at least one a step) + one
-        # value-reset kernel per step
-        "gpu_launches": counted_launches(launch, int(launches), args.steps, 2 if n_wide > 0 else 1) + args.steps,
+        # launches of Bellman kernels in the step calls, and one value-reset kernel per step
+        "gpu_launches": args.steps * (calls * launch["route"]["launches"] + 1),
         "e2e": e2e,
     }
     if world == 1 and not args.no_cpu_baseline:
@@ -416,6 +417,9 @@ KERNEL_NAMES = {1: "bellman_step_kernel", 2: "bellman_direct_kernel", 3: "bellma
                 4: "bellman_slice_kernel"}
 
 
+RULE_KERNELS = {5: "bellman_cluster_kernel", 6: "bellman_grid_kernel"}  # several iterations in a launch
+
+
 def parse_launch(text: str) -> dict:
     """'ring[:warps]', 'direct[:ctas_per_sm[:tile_entries[:wide_col]]]' or
     'slice[:ctas_per_sm]' -> launch fields."""
@@ -431,9 +435,10 @@ def parse_launch(text: str) -> dict:
     return out
 
 
-def apply_launch(g, sess, args, stream, tune_iters: int, default: str = "off") -> dict:
+def apply_launch(g, sess, args, stream, tune_iters: int, call: int, default: str = "off") -> dict:
     """Launch configuration of the timed session: explicit (--launch), the
-    autotuner's cached or freshly timed choice (--tune), or the rule."""
+    autotuner's cached or freshly timed choice (--tune), or the rule. `route`: the
+    kernel and launches of a step call of `call` iterations."""
     tune = args.tune or default
     if args.launch:
         g.imdp_session_set_launch(sess, stream=stream, **parse_launch(args.launch))
@@ -448,22 +453,31 @@ def apply_launch(g, sess, args, stream, tune_iters: int, default: str = "off") -
         how = "rule"
     out = g.imdp_session_get_launch(sess)
     out["chosen_by"] = how
-    if how == "rule":
-        out["note"] = ("step calls of 4 or more iterations are one launch of the resident or grid kernel where the "
-                       "rule plans one; the fields are those of the per-iteration kernel otherwise")
+    out["route"] = g.imdp_session_step_route(sess, call)
     return out
 
 
 def kernel_name(launch) -> str:
-    if launch["chosen_by"] == "rule" and launch["kernel"] != 3:
-        return "bellman_cluster_kernel or bellman_grid_kernel, by rule"
-    return KERNEL_NAMES.get(launch["kernel"], "bellman_step_kernel")
+    return {**KERNEL_NAMES, **RULE_KERNELS}[launch["route"]["kernel"]]
 
 
-def counted_launches(launch, iterations: int, calls: int, per_iteration: int) -> int:
-    """Step-kernel launches: by rule at least one per step call (iterations share
-    launches), else every iteration's."""
-    return calls if launch["chosen_by"] == "rule" else iterations * per_iteration
+L2_BYTES = 129e6
+
+
+def roofline(launch, streamed: float, once: float, model_bytes: float, seconds: float, peak: float) -> dict:
+    """What the Bellman launches of `seconds` moved: `streamed` bytes are what every
+    iteration reads and writes by the algorithm, `once` what has to come from memory
+    when a launch keeps it on chip. Per-iteration kernels, and the grid kernel on a
+    model larger than L2, stream from HBM; the others read L2 or shared memory, and
+    their share of the HBM peak is that of `once`."""
+    route = launch["route"]
+    rate, hbm = streamed / seconds / 1e9, once / seconds / 1e9
+    larger = route["kernel"] == 6 and not route["copied"] and model_bytes > L2_BYTES
+    if route["kernel"] in (1, 2, 4) or larger:
+        return {"bound": "hbm", "achieved": rate, "peak": peak, "unit": "GB/s", "frac": rate / peak}
+    source = "shared memory" if route["copied"] or route["kernel"] == 3 else "L2"
+    return {"bound": f"instruction issue and latency (transitions from {source})", "achieved": hbm, "peak": peak,
+            "unit": "GB/s", "frac": hbm / peak, "on_chip_gbs": rate}
 
 
 def _gpu_setup(rank, world, local_rank):
@@ -496,15 +510,18 @@ def run_polished(args, rank, world, local_rank):
     launches = []
     for mdl in (m32, m64):  # the autotuner's configuration of each storage
         s_ = g.imdp_session_create([mdl], [spec], stream=stream)
-        launches.append(apply_launch(g, s_, args, stream, 64, "cache"))
+        launches.append(apply_launch(g, s_, args, stream, 64, 32, "cache"))
         s_.close()
+    # (a session left to the rule has no configuration to pass on)
+    explicit = {k: {f: v for f, v in l.items() if f not in ("chosen_by", "route")}
+                for k, l in zip(("launch32", "launch64"), launches) if l["route"]["kernel"] in KERNEL_NAMES}
     Vd = torch.empty(m.n_states, dtype=torch.float64, device=dev)
     res = torch.empty(m.n_states, dtype=torch.float64, device=dev)
 
     def one_step():
         k = [0]
         st, k32 = g.imdp_value_iteration_polished(m32, m64, spec, Vd, k, res, stream=stream,
-                                                  launch32=launches[0], launch64=launches[1])
+                                                  **explicit)
         assert st == g.IMDP_OK
         return k32, k[0]
 
@@ -570,7 +587,7 @@ def run_uneven(args, rank, world, local_rank):
     kmax = int(Ks.max())
     # tuned on 200 iterations: the batch runs to horizons of 50..500, and its
     # first iterations (threshold searches) favour other kernels than the rest
-    launch = apply_launch(g, sess, args, stream, 200)
+    launch = apply_launch(g, sess, args, stream, 200, kmax)
 
     def one_step(ev=None):
         g.imdp_session_reset(sess, stream)
@@ -613,9 +630,8 @@ def run_uneven(args, rank, world, local_rank):
     if rank != 0:
         return
     peak, peak_kind = measured_peak_hbm()
-    alg = sum(algorithmic_bytes_per_iteration(m, args.dtype, g.imdp_model_exact_columns(x)[1], fixed=m.goal)
-              * int(K) for m, x, K in zip(ms, models, Ks))
-    achieved = alg * args.steps / (kernel_ms / 1e3) / 1e9
+    alg = [algorithmic_bytes_per_iteration(m, args.dtype, g.imdp_model_exact_columns(x)[1], fixed=m.goal)
+           for m, x in zip(ms, models)]
     out = {
         "metric": METRIC.replace("K=200", "K per problem"), "value": total_units / (elapsed_ms / 1e3), "unit": UNIT,
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": elapsed_ms / args.steps,
@@ -626,11 +642,11 @@ def run_uneven(args, rank, world, local_rank):
                    "max_horizon": kmax, "shapes": "states U{6..961}, actions U{1..4}, window U{2..min(400,n)}",
                    "l2": "inputs larger than L2 (%.1f GB resident)" % (nnz.sum() * 20 / 1e9),
                    "generation_s": round(gen_s, 1), "parallelism": "replicas", "launch": launch},
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                     "traffic": None, "peak_kind": peak_kind,
-                     "kernel": kernel_name(launch),
-                     "note": "algorithmic bytes of every running problem summed over the step's launches"},
-        "clocks": clk, "gpu_launches": counted_launches(launch, int(launches), args.steps, 1) + args.steps, "e2e": None,
+        "roofline": dict(roofline(launch, sum(b * int(K) for b, K in zip(alg, Ks)) * args.steps,
+                                  sum(alg) * args.steps * launch["route"]["launches"], sum(alg), kernel_ms / 1e3, peak),
+                         traffic=None, peak_kind=peak_kind, kernel=kernel_name(launch),
+                         note="algorithmic bytes of every running problem summed over the step's iterations"),
+        "clocks": clk, "gpu_launches": args.steps * (launch["route"]["launches"] + 1), "e2e": None,
     }
     print(json.dumps(out), flush=True)
 
@@ -729,7 +745,7 @@ def run_latency(args, rank, world, local_rank):
                                   "us_per_iteration": pct(dev_ms, 50) * 1e3 / K},
         },
         "transition_updates_per_s": nnz * K / (pct(e2e, 50) / 1e3),
-        "clocks": clk, "gpu_launches": int(K * n), "roofline": None,
+        "clocks": clk, "gpu_launches": n * (g.imdp_session_step_route(sess, K)["launches"] + 1), "roofline": None,
         "e2e": {"value": pct(e2e, 50), "unit": "ms per query", "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": int(m.n_states * 8)},
     }
@@ -837,7 +853,7 @@ def run_served(args, rank, world, local_rank):
     ok = all(d[0] == g.IMDP_OK and d[1] == r[1] for d, r in zip(done, reqs))
     span = max(d[2] for d in done) - t0
     units = float(sum(models_h[r[0]].nnz * r[1] for r in reqs))
-    stats = g.imdp_server_stats(server)
+    stats = dict(g.imdp_server_stats(server), **g.imdp_server_launches(server))
     server.close()
     if rank != 0:
         return
@@ -885,7 +901,7 @@ def run_state_sharded(args, rank, world, local_rank):
     lengths = np.diff(bounds)
     runner = SliceRunner(m, bounds, rank, dict(horizon=args.horizon, reach=m.goal), dtype)
     # each slice's session takes the autotuner's configuration for its own shape
-    launch = apply_launch(g, runner.session, args, None, min(args.horizon, 200), "cache")
+    launch = apply_launch(g, runner.session, args, None, min(args.horizon, 200), 1, "cache")
 
     def one_step():
         runner.reset()
@@ -949,8 +965,8 @@ def main():
                     help="32-bit storage: per-iteration error budget of the correction stage (0: library default)")
     ap.add_argument("--launch", default="", help="explicit launch configuration, e.g. ring:24, direct:4:1024 or slice:4")
     ap.add_argument("--tune", default="", choices=["", "cache", "fresh", "off"],
-                    help="off: by rule (the default, but for polished and state-sharded queries); autotuner of the per-iteration kernels: cached choice (timing only shapes "
-                         "missing from the cache), or time now")
+                    help="off: by rule (the default, but for polished and state-sharded queries); autotuner: cached "
+                         "choice (timing only shapes missing from the cache), or time now")
     ap.add_argument("--tune-cache", default="", help="autotuner cache file (default: the package's GB300 table)")
     ap.add_argument("--requests", type=int, default=2000, help="served workload: number of requests")
     ap.add_argument("--rate", type=float, default=2000.0, help="served workload: Poisson arrival rate per second")
