@@ -272,9 +272,9 @@ IMDP_API imdp_status imdp_session_create(imdp_model* const* models, const imdp_s
 /* Reset every problem to V_0 and iteration 0 (asynchronous on `stream`). */
 IMDP_API imdp_status imdp_session_reset(imdp_session* s, void* stream);
 
-/* Launch `n_iters` Bellman iterations (one kernel each, or all in one where the
- * launch rule says so; problems that are done or past their horizon are skipped
- * on the device). Asynchronous on `stream`;
+/* Launch `n_iters` Bellman iterations (one kernel each, or many in each launch
+ * where the launch rule says so; problems that are done or past their horizon are
+ * skipped on the device). Asynchronous on `stream`;
  * chunks of iterations are replayed from a captured CUDA graph when `stream`
  * is not the legacy default stream. */
 IMDP_API imdp_status imdp_session_step(imdp_session* s, int32_t n_iters, void* stream);
@@ -300,7 +300,9 @@ IMDP_API void imdp_session_destroy(imdp_session* s);
  * paper, whose GPU kernels have one fixed shape). Every configuration computes
  * the same words; they differ in speed only. Zero fields mean "by rule".
  *   kernel        0 by rule: step calls of 4 or more iterations run them in one
- *                 launch of the resident kernel where its values fit shared memory
+ *                 launch (of about 10 ms, or 100 ms and more where problems follow
+ *                 one another on the SMs; else in several) of the resident kernel
+ *                 where its values fit shared memory
  *                 and its cost model says it pays (no state slices, one storage
  *                 format): every problem, or every part of one finite-horizon
  *                 problem that no transition leaves, belongs to a thread-block

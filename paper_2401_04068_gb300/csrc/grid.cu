@@ -12,16 +12,17 @@
 // first, for the warm start. Columns it does not decide are settled by the CTA's
 // warps when they are few; otherwise they are listed in global memory, and CTAs
 // that have finished take them from any list (a few regions hold most of them:
-// with each CTA settling its own, pimdp_2 spends 27 % of its time waiting). One
+// with each CTA settling its own, 178,000 of 612,000 cycles of a late iteration of
+// pimdp_2, run here without the limit on transitions, were spent waiting). One
 // barrier of the grid ends an iteration, three when misses were listed.
 //
 // A per-iteration launch of the direct kernel has a chain of dependent loads in
 // front of every tile (tile counter, tile, descriptor, column words, hint entry,
 // its value) and gathers V through L1 and L2; here nothing but the entries
 // themselves is loaded in the loop, and entries that fit stay in shared memory.
-// The warm start streams at 0.8 of the copy bandwidth (pimdp_2, 300,000 cycles
-// an iteration); a missed column takes 15,000 to 45,000 cycles of a warp, which
-// is what bounds the first iterations of every model. Measured, K = 200 or to
+// The warm start streams at 0.8 of the copy bandwidth (harrier, 109,000 of the
+// 230,000 cycles of a late iteration; the rest are misses, 20,000 to 76,000 cycles
+// each), and misses bound the first iterations of every model. Measured, K = 200 or to
 // convergence: 20,000 states of 24 scattered transitions 3.6 -> 1.27 ms,
 // cartpole_960 4.8 -> 2.1, harrier 44.1 -> 34.5, cartpole_3840 13.7 -> 11.4.
 #include <cuda_runtime.h>

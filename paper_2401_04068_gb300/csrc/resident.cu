@@ -12,8 +12,8 @@
 // chosen so that the parts in progress together fit L2, so HBM is read about
 // once per part instead of once per iteration.
 //
-// Bound by instruction issue and L2 latency (4096 parts of 240 states, 64-bit
-// storage: 55 % issue slots busy, 7 TB/s from L2, DRAM 3 %); a transition costs
+// Bound by instruction issue and L2 latency (parts of 240 states, 64-bit storage:
+// 50 % issue slots busy, 6.6 TB/s from L2, DRAM 3 % with 1,024 of them under ncu); a transition costs
 // 32 warp instructions per 32 lanes, a warp's four columns 290 more. Measured
 // against the per-iteration kernels, K = 200: those 4096 parts 115 -> 66 ms
 // (32-bit storage 117 -> 66), 256 problems of up to 961 states and horizons from
