@@ -550,7 +550,9 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, b
   }
   const double mine = std::max(uneven(c), spread(c));
   if (mine > other) return none();
-  long_seconds = mine / iters;
+  // (at first all units run, with short horizons beside a long one much more than on average)
+  const double all = 3e-6 + (double)entries / (1.17 * std::min<double>(grid, (double)n_units * c) * hz);
+  long_seconds = std::max(mine / iters, 0.5 * all);
   std::vector<ResidentUnit> uh(n_units);
   for (int32_t i = 0; i < n_units; ++i) uh[i] = us[i].u;
   ResidentUnit* du = alloc<ResidentUnit>(uh.size());

@@ -319,3 +319,19 @@ def test_long_exact_columns_stay_per_iteration(n, k, grid):
     # the rule's choice is no slower than the kernel it took before there was a grid kernel
     assert seconds() <= 1.05 * seconds(kernel=g.KERNEL_DIRECT, ctas_per_sm=3, tile_entries=1024)
     model.close()
+
+
+def test_launches_are_bounded_beside_a_long_horizon():
+    # 2,000 problems of 300 iterations and one of 20,000: the launch that runs them all
+    # is no longer than others, although an average iteration takes next to nothing
+    small = banded_imdp(200, 1, 200 * 101 + 1, eps=0.1, seed=3)
+    model = g.create_model(small)
+    n = 2001
+    specs = [g.make_spec(horizon=20000 if i == 0 else 300, reach=small.goal) for i in range(n)]
+    sess = g.imdp_session_create([model] * n, specs)
+    r = g.imdp_session_step_route(sess, 20000)
+    assert r["kernel"] == g.KERNEL_RESIDENT
+    # (40 million transitions take 0.12 ms an iteration at the resident kernel's rate; twice the usual 0.1 s)
+    assert 20000 / r["launches"] <= 2 * 0.1 / 0.12e-3, r
+    sess.close()
+    model.close()
