@@ -498,7 +498,9 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, b
     const double k = (double)entries / std::max<int64_t>(cols, 1);
     resident.group = k >= 256 || (double)cols / n_units / c < 4.0 * resident.threads / 32 / 2 ? 32 : 8;
     resident.cluster = c;
-    return resident_prepare(resident) == cudaSuccess;  // (wide clusters may not fit the device)
+    if (resident_prepare(resident) == cudaSuccess) return true;
+    cudaGetLastError();  // wide clusters may not fit the device: the next shape is tried without this error
+    return false;
   };
   resident.parts = parts ? 1 : 0;
   resident.f32 = f32 ? 1 : 0;
@@ -506,7 +508,6 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, b
   resident.max_col = max_col;
   resident.n_units = n_units;
   const auto none = [&]() {
-    cudaGetLastError();
     resident.n_units = 0;
     return IMDP_OK;
   };
