@@ -81,6 +81,6 @@ def test_no_cuts_for_a_plan_that_has_no_room():
         host_ms = min(host_ms, s["wall_ms"] - s["device_ms"])
         server.close()
     assert launches["per_iteration"] > 0
-    assert host_ms < 5.5, host_ms  # 8.0 when it cuts them
+    assert host_ms < 6.5, host_ms  # 3.0; 8.0 when it cuts them
     for x in models:
         x.close()
