@@ -334,12 +334,18 @@ bool Session::grid_possible() const {
   // 376 20.2 / 20.8; on 32-bit storage 42,000 of 376 8.2 / 7.0, 48,000 of 500 15.7 /
   // 15.9, 90,000 of 300 14.5 / 16.4). Against the ring kernel, which short columns
   // take otherwise, it gains at any number (126,000 of 230 20.5 / 17.5).
-  // So do a few very long columns on 32-bit storage that mostly keeps exact bounds:
-  // their settling passes are as long as on 64-bit storage, their stream has two kinds
-  // of columns (3,841 columns of 2,228 entries, 87 % of them exact: 8.5 / 9.3; of
-  // 3,001 columns 1,800 entries 6.0 / 5.8, 1,345 with 55 % 6.6 / 5.0).
-  if (m->lg32 && m->n_cols <= 5000 && m->nnz >= (int64_t)2000 * m->n_cols && m->exact_entries >= 0.8 * m->nnz)
-    return false;
+  // So do very long columns for few iterations: in the first ones nearly all of them
+  // are settled, which the block-wide kernel does faster (3,841 columns of 2,228
+  // entries, direct and block-wide / grid kernel, ms: 32 iterations 4.3 / 5.1, 64 6.4 /
+  // 6.5, 100 8.3 / 7.8; 3,001 of 1,800 16 iterations 1.77 / 1.93, 32 3.13 / 3.06). On
+  // 32-bit storage that keeps most of them exact the stream has two kinds of columns
+  // and gains less (3,841 of 2,228 100 iterations 8.5 / 9.3, 200 14.0 / 14.4; 7,681 of
+  // them 14.4 / 14.6 and 24.0 / 22.8; 5,001 of 2,000 100 iterations 10.4 / 10.9; 3,001
+  // of 1,800 100 iterations 6.0 / 5.8).
+  const double k = (double)m->nnz / std::max(m->n_cols, 1);
+  int32_t least = k >= 2000 ? 64 : (k >= 1500 ? 32 : 0);
+  if (m->lg32 && k >= 2000 && m->exact_entries >= 0.5 * m->nnz) least = m->n_cols <= 4500 ? INT32_MAX : 128;
+  if (least == INT32_MAX || (!any_infinite && max_horizon < least)) return false;
   return m->nnz < (int64_t)kRuleLongColumn * m->n_cols || m->n_cols <= (m->lg32 ? 45000 : 56000);
 }
 
@@ -549,6 +555,10 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, b
     bounds = wide_bounds;
     break;
   }
+  // A large problem's first iterations settle most columns, on 16 SMs here: few
+  // iterations are left to the grid kernel (1,501 columns of 80 entries, per iteration /
+  // resident / grid: 8 iterations 215 / 256 / 128 us, 16 434 / 488 / 244).
+  if (alone && !copied && !any_infinite && max_horizon < 24) return none();
   const double mine = std::max(uneven(c), spread(c));
   if (mine > other) return none();
   // (at first all units run, with short horizons beside a long one much more than on average)

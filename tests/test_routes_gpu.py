@@ -299,7 +299,9 @@ def test_long_exact_columns_stay_per_iteration(n, k, grid):
     spec = g.make_spec(horizon=100, reach=m.goal)
     kernel = _route([model], [spec], 100)["kernel"]
     assert (kernel == g.KERNEL_GRID) == grid and exact > (0.6 if grid else 0.8), exact
-    assert _alone(m, 100)["kernel"] == g.KERNEL_GRID  # on 64-bit storage
+    wide = g.create_model(m)
+    assert _route([wide], [spec], 100)["kernel"] == g.KERNEL_GRID  # on 64-bit storage
+    wide.close()
 
     def seconds(**launch):
         sess = g.imdp_session_create([model], [spec])
@@ -334,4 +336,18 @@ def test_launches_are_bounded_beside_a_long_horizon():
     # (40 million transitions take 0.12 ms an iteration at the resident kernel's rate; twice the usual 0.1 s)
     assert 20000 / r["launches"] <= 2 * 0.1 / 0.12e-3, r
     sess.close()
+    model.close()
+
+
+# few iterations, most of them with nearly every column to settle: long columns stay per
+# iteration, and a cluster of 16 SMs is left for the whole GPU
+@pytest.mark.parametrize("n,k,short,long,kernels", [
+    (3840, 2240, 63, 64, (g.KERNEL_DIRECT, g.KERNEL_GRID)), (3000, 1700, 31, 32, (g.KERNEL_DIRECT, g.KERNEL_GRID)),
+    (1500, 80, 23, 24, (g.KERNEL_GRID, g.KERNEL_RESIDENT))])
+def test_few_iterations_of_long_searches(n, k, short, long, kernels):
+    m = banded_imdp(n, 1, n * (k + 1) + 1, eps=0.1, seed=1)
+    model = g.create_model(m)
+    for kw, want in ((dict(horizon=short), 0), (dict(horizon=long), 1),
+                     (dict(infinite_time=True, eps=1e-6, horizon=10), 1)):
+        assert _route([model], [g.make_spec(reach=m.goal, **kw)], 10)["kernel"] == kernels[want], kw
     model.close()
