@@ -414,6 +414,11 @@ imdp_status Session::plan_resident(const std::vector<const imdp_spec*>& specs, b
     cols += m->n_cols;
     resident.single = resident.single && m->n_cols == m->n_states;
   }
+  // The very smallest stay on the single-CTA kernel, which has less to set up: up to 5
+  // states of one action (200 iterations of 5: 212 us, 232 here; of 9 columns 325 and
+  // 238), and with the residual of an infinite horizon up to 5 states of 16 columns
+  // (64 iterations of 3 states and 3 columns 127 and 165 us, 72 of 5 and 15 232 and 277).
+  if (L.tiny_ok && states <= 5 && cols <= (any_infinite ? 16 : (resident.single ? 5 : 0))) return IMDP_OK;
   const int32_t n_units = (int32_t)us.size();
   std::stable_sort(us.begin(), us.end(), [](const Work& a, const Work& b) { return a.work > b.work; });
   // Cluster size. More CTAs to a unit cost synchronisation; fewer leave the GPU

@@ -42,10 +42,15 @@ def test_kernels_of_one_problem(dtype):
         r = _alone(GRID[name](), dtype=dtype)
         assert (r["kernel"], r["launches"], r["threads"]) == (g.KERNEL_GRID, 1, 768), name
         assert r["group"] == (8 if name == "sink" else 32) and r["copied"] == (name not in ("long_sink", "wide")), name
-    for n, a, k in ((1, 1, 1), (5, 1, 5), (7, 3, 4), (64, 1, 12), (330, 3, 4), (1000, 1, 3)):
+    for n, a, k in ((5, 1, 5), (7, 3, 4), (64, 1, 12), (330, 3, 4), (1000, 1, 3)):
         r = _alone(banded_imdp(n, a, n * a * (min(k, n) + 1) + 1, eps=0.1, seed=n), dtype=dtype)
         assert r["kernel"] == g.KERNEL_RESIDENT and r["units"] == 1 and r["copied"] == 1, n
-        assert (r["cluster"] == 1) == (n in (1, 5)), n
+        assert (r["cluster"] == 1) == (n == 5), n
+    # (the sink is a state more)
+    for n, a, finite, infinite in ((1, 1, 3, 3), (4, 1, 3, 3), (4, 2, 5, 3), (5, 1, 5, 5), (4, 5, 5, 5)):
+        m = banded_imdp(n, a, n * a * (min(2, n) + 1) + 1, eps=0.1, seed=n)
+        assert _alone(m, dtype=dtype)["kernel"] == finite, (n, a)
+        assert _alone(m, dtype=dtype, infinite_time=True, eps=1e-6)["kernel"] == infinite, (n, a)
     for a, threads in ((1, 384), (3, 768)):
         r = _alone(banded_imdp(610, a, 610 * a * 21 + 610 * a + 1, eps=0.1, seed=31), dtype=dtype)
         assert (r["kernel"], r["cluster"], r["threads"]) == (g.KERNEL_RESIDENT, 16, threads)
